@@ -144,9 +144,9 @@ size_t bitsmoe_workspace_bytes(const bitsmoe_layer* layer, int T, int top_k);
  * CUDA graph or count launches).  A single token runs as one fused persistent
  * kernel (1) when the layer's per-block shares of the bases and factors fit
  * in shared memory, and up to 4 tokens as one such kernel per token (T);
- * otherwise the forward is a chain of 5 kernels, 8 with the tensor-core expert
- * factors (z gather, gate/up and down on tensor cores beside the dp2a kernels;
- * see bitsmoe_forward_plan).
+ * otherwise the forward is a chain of 5 kernels (routing, projection, gate/up,
+ * down, output basis), 6 with the tensor-core expert factors past 8 tokens
+ * (the gather of their gate/up operand; see bitsmoe_forward_plan).
  * Returns a negative error code for invalid arguments. */
 int bitsmoe_forward_launches(const bitsmoe_layer* layer, int T, int top_k);
 
@@ -156,12 +156,11 @@ int bitsmoe_forward_launches(const bitsmoe_layer* layer, int T, int top_k);
  *      fused kernel, else 5 <= T <= 8)
  *   4  tensor-core (tcgen05) shared-basis projections (every T > 8; the decode
  *      chain from 4 tokens)
- *   8  tensor-core gate/up factors with SiLU(gate) * up fused (T > 8 on layers
- *      without 16-bit units whose group is a multiple of 128 rows; otherwise
- *      the dp2a kernel) for the experts with at least 8 tokens (4 when a
- *      factor matrix holds at least 8 M codes), the dp2a kernel for the
- *      others: the codes enter the MMA as fp16 bit patterns
- *  16  tensor-core down factor (the same condition; always set with 8)
+ *   8  past 8 tokens: tensor-core gate/up factors (mma.sync over tiles of 8 or
+ *      16 tokens, the codes entering the products as fp16 bit patterns), for
+ *      every layer without 16-bit units; the others use the dp2a kernels.  The
+ *      decode chain takes the same kernels from 4 tokens on.
+ *  16  tensor-core down factor (always set with 8)
  *  32  with 1: the fused kernel is the clustered one, in which a thread-block
  *      cluster owns one (routing slot, 128-row block) pair of the token and
  *      its blocks exchange partial gate/up rows through distributed shared

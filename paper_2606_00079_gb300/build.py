@@ -3,8 +3,8 @@
 Ten translation units, compiled in parallel: the host packer (pack.cpp,
 plain C++), the CUDA kernel chain + C ABI (forward.cu), the two fused
 single-token decode kernels (fused.cu, and the clustered one in fused2.cu),
-the tensor-core projections (gemm.cu), the tensor-core expert factors
-(expert_tc.cu), the per-unit quantiser from float spectral vectors
+the tensor-core projections (gemm.cu), the tensor-core expert factors of
+calls with several tokens (expert_mma.cu), the per-unit quantiser from float spectral vectors
 (quantize.cu), the per-projection bit allocation (allocate.cu) and the
 importance beta from calibration tokens that the allocation weighs its losses
 by (importance.cu), and the shared-basis decomposition with the calibration
@@ -43,7 +43,7 @@ def _run(cmd):
 
 
 def sources():
-    return [os.path.join(CSRC, f) for f in ("pack.cpp", "forward.cu", "fused.cu", "fused2.cu", "gemm.cu", "expert_tc.cu",
+    return [os.path.join(CSRC, f) for f in ("pack.cpp", "forward.cu", "fused.cu", "fused2.cu", "gemm.cu", "expert_mma.cu",
                                               "quantize.cu", "allocate.cu", "importance.cu", "decompose.cu")]
 
 

@@ -43,26 +43,27 @@ struct Fwd {
   float* z;         // [2][T][n_pad]
   float* gu;        // [P][2][I_pad]
   float* s;         // [T][n_pad]
-  float* zT;        // [2][n_pad][T]: z again, token fastest (written for the tensor-core gate/up kernel)
-  int tc_min;       // > 0: experts with at least this many tokens take the tensor-core factor kernels,
-                    //      the dp2a kernels skip them (and the tensor-core kernels the others)
+  uint32_t* zmax;   // null, or [2][T]: cleared by the router, then max |z_h[t][j]| (fp32 bits) by the projection
 };
 
-// Buffers and sizes of the multi-token tensor-core expert kernels (expert_tc.cu).
-struct XArgs {
-  int NT;                 // rows of a token tile (16, 32 or 64): an expert's tokens in tiles of NT
-  int max_tiles;          // bound on the call's token tiles
+struct CStage;
+struct DStage;
+
+// Sizes and tables of the multi-token expert kernels on mma.sync (expert_mma.cu).
+struct MArgs {
+  int ntm;                // groups of 8 tokens a warp's pass takes at most (1 or 2)
+  int use_az;             // the gate/up operand is gathered by a kernel of its own (past the decode batch)
+  float* az;              // [2][rt][nsp]: alpha z 2^S of every routed token in unit-slot order
+  int rt, nsp;            // its rows (routed tokens, experts padded to 8) and slots a row
   int A_max;              // bound on the call's routed experts
-  int Rtot;               // rows of the h buffers (multiple of 16)
-  uint32_t ring;          // bytes of a CTA's copy ring (set at launch)
+  uint32_t gu_stage;      // bytes of a staged gate/up segment
+  int gu_r;               // row blocks a gate/up block works on at once
+  int dn_rc;              // row blocks of a down run
+  uint32_t dn_meta;       // bytes of a down tile's staged unit indices, alphas and scale/zero rows
+  const CStage* cst;      // [2][E][nseg]
+  const DStage* dst;      // [E][ul_max_tiles]
+  const uint8_t* meta;    // the records' slot metadata (mirror of the image's)
   const float* msa;       // [2][E] max over groups and slots of |scale * alpha| of gate/up (h, e)
-  const uint32_t* zmax;   // [2][T] max over j of |z_h[t][j]| (fp32 bits)
-  uint8_t* hb;            // [NRB][Rtot rows x 512 B]: h as an fp16 pair, a token tile of N rows at its first
-                          //   row R0 as the down kernel's B tile [half 2][piece 2][N rows][128 B] (swizzled)
-  float2* hs;             // [NRB][Rtot]: (sum of h over the row block's rows, 2^(24 - S) of its scaling)
-  int tc_min;             // experts with fewer tokens are left to the dp2a kernels
-  float* zv;              // z gathered per (projection, token tile) in unit-slot order: [K-block][128 slots][N]
-  uint64_t zv_floats;     // its length
 };
 
 // Staging records of the fused single-token kernel, derived from the image
@@ -81,7 +82,7 @@ struct CStage {            // one per gate/up item (h < 2, e, segment)
   uint8_t bits[kNumBk];    // their bit-widths
   uint16_t ntl[kNumBk];    // tiles per touched bucket
   uint32_t meta0;          // offset in the metadata mirror of row block 0's [unit | alpha | scale/zero G rows]
-  uint8_t pad_[4];
+  uint32_t slot0;          // first slot in the projection's slot arrays
 };
 static_assert(sizeof(CStage) == 80, "CStage layout");
 
@@ -215,16 +216,14 @@ cudaError_t launch_fused(const Fwd& p, const FusedArgs& f, int sms, cudaStream_t
 // unless y carries a residual).
 bool make_basis_map(void* map_out, const void* base, int rows, int cols_pad);
 cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cudaStream_t st, bool pdl,
-                           float* zT = nullptr, void* zero = nullptr, size_t zero_bytes = 0,
-                           uint32_t* zmax = nullptr);
-// Multi-token expert factors on tensor cores (expert_tc.cu): buffer sizes for T tokens,
-// z gathered per token tile in unit-slot order (reads zT), gate/up with h = SiLU(gate) up
-// into x.hb / x.hs (reads zmax), then the down factor of every routed expert into s
-// (zeroed before).  Persistent: `sms` CTAs.
-XArgs x_args(const ImageHeader& hd, int T, int k);
-cudaError_t launch_zgather(const Fwd& p, const XArgs& x, int sms, cudaStream_t st, bool pdl);
-cudaError_t launch_gu16(const Fwd& p, const XArgs& x, int sms, cudaStream_t st, bool pdl);
-cudaError_t launch_dn16(const Fwd& p, const XArgs& x, int sms, cudaStream_t st, bool pdl);
+                           void* zero = nullptr, size_t zero_bytes = 0, uint32_t* zmax = nullptr, bool zt = false);
+// Multi-token expert factors on mma.sync (expert_mma.cu): sizes for T tokens (false when the layer
+// does not fit; gu_stage from mma_gu_stage), then gate/up into p.gu and down into p.s (both zeroed
+// before).  Persistent: `sms` blocks.
+uint32_t mma_gu_stage(const std::vector<CStage>& cst, int G, bool az);
+uint64_t mma_az_floats(const ImageHeader& hd, int T, int k, int* rt, int* nsp);
+bool mma_args(const ImageHeader& hd, int T, int k, bool az, uint32_t gu_stage, MArgs* x);
+cudaError_t launch_expert_mma(bool down, const Fwd& p, const MArgs& x, int sms, cudaStream_t st, bool pdl);
 // Staging records of a packed image (host side, at upload).
 bool build_stage_tables(const uint8_t* img, std::vector<CStage>& cst, std::vector<DStage>& dst,
                         std::vector<uint8_t>& meta);

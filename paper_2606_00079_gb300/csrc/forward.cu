@@ -57,7 +57,8 @@ struct bitsmoe_layer {
   alignas(64) uint8_t map_in[128];    // TMA maps of the two input bases and of the output basis
   alignas(64) uint8_t map_out[128];
   bool maps = false;
-  bool tcx = false;            // expert factors on tensor cores: no 16-bit units, groups of whole row blocks
+  bool mma = false;            // multi-token expert factors on tensor cores: no 16-bit units, metadata mirror built
+  uint32_t gu_stage[2] = {0, 0};   // largest staged gate/up segment of those kernels (z gathered in the kernel, az)
   const float* d_msa = nullptr;   // [2][E] max |scale * alpha| of each gate/up (h, e) (inside d_stage's allocation)
   std::vector<uint8_t> meta;   // host copy of header + descriptors + segment table
   int seg_bytes = 0;           // largest gate/up item: code bytes inside one row block
@@ -241,6 +242,8 @@ __global__ void __launch_bounds__(kThreads) k_norm_router(NormArgs a) {
 // routing with a release flag that the gate/up and down kernels wait on.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads) k_route_publish(Fwd p) {
+  if (p.zmax)   // the projection takes the maxima, after this kernel
+    for (int i = threadIdx.x; i < 2 * p.T; i += blockDim.x) p.zmax[i] = 0u;
   if (threadIdx.x == 0) {   // before the trigger: no later kernel may see the previous call's flag
     p.status[0] = 0;
     p.route_flag[0] = 0;
@@ -275,6 +278,8 @@ __global__ void __launch_bounds__(kThreads) k_route_publish(Fwd p) {
 // resets) groups all pairs and publishes the routing with a release flag.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) k_router(Fwd p) {
+  if (p.zmax && blockIdx.x == 0)   // the projection takes the maxima, after this kernel
+    for (int i = threadIdx.x; i < 2 * p.T; i += blockDim.x) p.zmax[i] = 0u;
   if (blockIdx.x == 0 && threadIdx.x == 0) {   // before the trigger: no later kernel may see the previous flag
     p.status[0] = 0;
     p.route_flag[0] = 0;
@@ -331,19 +336,34 @@ __global__ void __launch_bounds__(1024) k_router(Fwd p) {
   __syncthreads();
   if (!last) return;
   __threadfence();
-  int* s_pe = reinterpret_cast<int*>(keys);   // reuse: all pairs' experts
-  int* s_cnt = s_pe + P;
-  int* s_start = s_cnt + E;
-  for (int q = tid; q < P; q += blockDim.x) s_pe[q] = __ldcg(p.pair_expert + q);
-  __syncthreads();
+  // Grouping by counting: warp w takes the w-th contiguous part of the pairs, counts its pairs per
+  // expert, and after a prefix over the warps places them in order (the rank inside a group of 32 by
+  // match.any).  1024 tokens, top-8: 122 us with one pass over all pairs per expert, see the bench table.
   const int warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-  for (int e = warp; e < E; e += nw) {
-    int c = 0;
-    for (int q0 = 0; q0 < P; q0 += 32) {
-      const int q = q0 + lane;
-      c += __popc(__ballot_sync(0xFFFFFFFFu, q < P && s_pe[q] == e));
+  uint16_t* s_pe = reinterpret_cast<uint16_t*>(keys);     // [P] reuse: all pairs' experts
+  uint16_t* s_h = s_pe + ((P + 1) & ~1);                  // [nw][E] pairs of each warp and expert, then their offset
+  int* s_cnt = reinterpret_cast<int*>(s_h + nw * ((E + 1) & ~1));
+  int* s_start = s_cnt + E;
+  const int hs = (E + 1) & ~1;
+  for (int q = tid; q < P; q += blockDim.x) s_pe[q] = (uint16_t)__ldcg(p.pair_expert + q);
+  for (int i = tid; i < nw * hs; i += blockDim.x) s_h[i] = 0;
+  __syncthreads();
+  const int part = (P + nw * 32 - 1) / (nw * 32) * 32, qb = warp * part, qe = min(P, qb + part);
+  for (int q0 = qb; q0 < qe; q0 += 32) {
+    const int q = q0 + lane, e = q < qe ? s_pe[q] : E + lane;   // lanes past the end match no other
+    const unsigned m = __match_any_sync(0xFFFFFFFFu, e);
+    if (q < qe && (m & ((1u << lane) - 1u)) == 0) s_h[warp * hs + e] += (uint16_t)__popc(m);
+    __syncwarp();
+  }
+  __syncthreads();
+  for (int e = tid; e < E; e += blockDim.x) {
+    int run = 0;
+    for (int w = 0; w < nw; ++w) {
+      const int c = s_h[w * hs + e];
+      s_h[w * hs + e] = (uint16_t)run;
+      run += c;
     }
-    if (lane == 0) s_cnt[e] = c;
+    s_cnt[e] = run;
   }
   __syncthreads();
   if (warp == 0) {
@@ -373,15 +393,18 @@ __global__ void __launch_bounds__(1024) k_router(Fwd p) {
     }
   }
   __syncthreads();
-  for (int e = warp; e < E; e += nw) {
-    int base = s_start[e];
-    for (int q0 = 0; q0 < P; q0 += 32) {
-      const int q = q0 + lane;
-      const bool m = q < P && s_pe[q] == e;
-      const unsigned b = __ballot_sync(0xFFFFFFFFu, m);
-      if (m) p.pair_list[base + __popc(b & ((1u << lane) - 1u))] = q;
-      base += __popc(b);
+  for (int q0 = qb; q0 < qe; q0 += 32) {
+    const int q = q0 + lane, e = q < qe ? s_pe[q] : E + lane;
+    const unsigned m = __match_any_sync(0xFFFFFFFFu, e);
+    const int r = __popc(m & ((1u << lane) - 1u));
+    int base = 0;
+    if (q < qe) base = s_h[warp * hs + e];
+    __syncwarp();
+    if (q < qe) {
+      p.pair_list[s_start[e] + base + r] = q;
+      if (r == 0) s_h[warp * hs + e] = (uint16_t)(base + __popc(m));
     }
+    __syncwarp();
   }
   __syncthreads();
   if (tid == 0) {   // the routing is published: kernels that stage by it may go on
@@ -811,7 +834,7 @@ __global__ void __launch_bounds__(kK2DecWarps * 32) k_gateup_dec(Fwd p) {
   const ExpertDesc& xd = p.desc[h * p.E + e];
   const ItemRec it = p.items[((size_t)h * p.E + e) * p.nseg + sg];
   const int ntok = p.expert_count[e], pst = p.expert_start[e];
-  if (it.nr == 0 || (p.tc_min > 0 && ntok >= p.tc_min)) {   // empty, or the tensor-core kernels' expert
+  if (it.nr == 0) {   // empty
     pdl_wait();
     return;
   }
@@ -1039,7 +1062,7 @@ __global__ void __launch_bounds__(kK3DecWarps * 32) k_down_dec(Fwd p) {
   const int r = item - a * ntg * nrc;
   const int tg = r / nrc, rc = r - tg * nrc;
   const ExpertDesc& xd = p.desc[2 * p.E + e];
-  if (tg * kK3DecWarps >= xd.ntiles || (p.tc_min > 0 && p.expert_count[e] >= p.tc_min)) {
+  if (tg * kK3DecWarps >= xd.ntiles) {
     pdl_wait();
     return;
   }
@@ -1203,18 +1226,6 @@ __global__ void __launch_bounds__(kK3DecWarps * 32) k_down_dec(Fwd p) {
 #ifndef BITSMOE_DECODE_MAX_TOKENS
 #define BITSMOE_DECODE_MAX_TOKENS 8
 #endif
-// Tokens from which an expert's factors use the tensor-core kernels (their cost follows the
-// codes, the dp2a kernels' the tokens): measured crossovers on GB300 are about 8 tokens for
-// Qwen3-sized experts (768 x 2048 codes a matrix) and at most 4 for Mixtral-sized ones
-// (14336 x 4096), whose per-item costs amortise over far more codes.
-#ifndef BITSMOE_TC_MIN_TOKENS
-inline int tc_min_tokens(const ImageHeader& hd) {
-  return (uint64_t)hd.I_pad * (uint64_t)hd.n_pad >= (8ull << 20) ? 4 : 8;
-}
-#else
-inline int tc_min_tokens(const ImageHeader&) { return BITSMOE_TC_MIN_TOKENS; }
-#endif
-
 // Small batches run the decode chain (every kernel routes all tokens itself; the
 // single token also the fused kernel), larger ones the tensor-core chain.
 inline bool decode_mode(const ImageHeader& hd, int T) {
@@ -1222,7 +1233,7 @@ inline bool decode_mode(const ImageHeader& hd, int T) {
 }
 
 struct WsLayout {
-  size_t status, pair_expert, pair_weight, expert_count, expert_start, pair_list, active, z, gu, s, zmax, zt, hb, hs, zv;
+  size_t status, pair_expert, pair_weight, expert_count, expert_start, pair_list, active, z, gu, s, zmax, az;
   size_t x_stage, logits_stage, y_stage;
   size_t sync;   // fused single-token kernel: grid-barrier counters
   size_t total;
@@ -1247,15 +1258,12 @@ WsLayout ws_layout(const ImageHeader& hd, int T, int k) {
   w.z = take(2 * (size_t)T * hd.n_pad * 4);
   w.gu = take(P * 2 * hd.I_pad * 4);
   w.s = take((size_t)T * hd.n_pad * 4);
-  // tensor-core expert factors (calls past the decode chain): max |z| per token (directly after
-  // s: one clear for both), z token fastest, h tiles and their row-block sums and scales
-  const bool tcx = !decode_mode(hd, T);
-  const XArgs xa = tcx ? x_args(hd, T, k) : XArgs{};
-  w.zmax = take(tcx ? 2 * (size_t)T * 4 : 0);
-  w.zt = take(tcx ? 2 * (size_t)T * hd.n_pad * 4 : 0);
-  w.hb = take(tcx ? (size_t)hd.NRB * xa.Rtot * 512 : 0);
-  w.hs = take(tcx ? (size_t)hd.NRB * xa.Rtot * 8 : 0);
-  w.zv = take(tcx ? (size_t)xa.zv_floats * 4 : 0);
+  // multi-token expert factors: max |z| per token (small batches: in the slack behind the status words)
+  // and, past the decode batch, their operand in unit-slot order
+  const bool batch = !decode_mode(hd, T);
+  int rt, nsp;
+  w.zmax = batch ? take(2 * (size_t)T * 4) : w.status + 64;
+  w.az = take(batch ? (size_t)mma_az_floats(hd, T, k, &rt, &nsp) * 4 : 0);
   w.x_stage = take((size_t)T * hd.D * 2);
   w.logits_stage = take((size_t)T * hd.E * 4);
   w.y_stage = take((size_t)T * hd.D * 4);
@@ -1498,6 +1506,13 @@ int f2_choose(const bitsmoe_layer* L, int top_k, F2Args* fa) {
   return ci;
 }
 
+// Whether the expert factors of a T-token call run on mma.sync (calls whose projection runs on the
+// tensor cores, which also takes max |z| per token).
+bool mma_fits(const bitsmoe_layer* L, int T, int top_k, MArgs* ma) {
+  const bool az = !decode_mode(L->hd(), T);
+  return L->mma && T >= 4 && mma_args(L->hd(), T, top_k, az, L->gu_stage[az], ma);
+}
+
 int forward_impl(const void* x, const float* logits, int T, int top_k, const bitsmoe_layer* L, float* y,
                  void* ws, size_t ws_bytes, cudaStream_t st, cudaEvent_t* ev = nullptr, bool accum = false,
                  const NormArgs* norm = nullptr, bool host_io = false) {
@@ -1564,7 +1579,6 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
   p.z = reinterpret_cast<float*>(wb + w.z);
   p.gu = reinterpret_cast<float*>(wb + w.gu);
   p.s = reinterpret_cast<float*>(wb + w.s);
-  p.zT = reinterpret_cast<float*>(wb + w.zt);
   const int sms = L->num_sms;
   int rc;
   auto mark = [&](int i) -> int {
@@ -1572,6 +1586,17 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
     return BITSMOE_OK;
   };
   const int G = std::max(1, kRows / hd.group);
+  // several tokens: the expert factors on mma.sync (they scale their operands by max |z| per token)
+  MArgs ma;
+  const bool mma = mma_fits(L, T, top_k, &ma);
+  if (mma) {
+    ma.cst = L->d_cst;
+    ma.dst = L->d_dst;
+    ma.meta = L->d_meta;
+    ma.msa = L->d_msa;
+    p.zmax = reinterpret_cast<uint32_t*>(wb + w.zmax);
+    ma.az = reinterpret_cast<float*>(wb + w.az);
+  }
   if (T == 1 && !norm) {   // one token: the clustered kernel when the layer fits it
     F2Args f2;
     const int ci = f2_choose(L, top_k, &f2);
@@ -1626,13 +1651,17 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
     if (tcp) {   // tensor-core projection; it also clears gate/up and s for the expert kernels
       const size_t zb = (size_t)(reinterpret_cast<uint8_t*>(p.s) - reinterpret_cast<uint8_t*>(p.gu)) +
                         (size_t)T * hd.n_pad * 4;
-      BM_CK(launch_gemm_tc(0, L->map_in, p, sms, st, pdl, nullptr, p.gu, zb));
+      BM_CK(launch_gemm_tc(0, L->map_in, p, sms, st, pdl, p.gu, zb, p.zmax, mma));
     } else if ((rc = launch_gemv_bulk(true, p, sms, st, pdl))) {
       return rc;
     }
     if ((rc = mark(2))) return rc;
     std::function<int()> between = ev ? std::function<int()>([&]() { return mark(3); }) : std::function<int()>();
-    if (T == 1) {
+    if (mma) {
+      BM_CK(launch_expert_mma(false, p, ma, sms, st, pdl));
+      if ((rc = mark(3))) return rc;
+      BM_CK(launch_expert_mma(true, p, ma, sms, st, pdl));
+    } else if (T == 1) {
       if (G == 1) rc = launch_k2k3_dec<1, 1>(p, A_max, sms, st, pdl, between);
       else if (G == 2) rc = launch_k2k3_dec<2, 1>(p, A_max, sms, st, pdl, between);
       else rc = launch_k2k3_dec<4, 1>(p, A_max, sms, st, pdl, between);
@@ -1649,44 +1678,24 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
   }
   const int tpb = std::max(1, 1024 / hd.E);
   const size_t router_smem =
-      std::max((size_t)tpb * (hd.E + top_k), (size_t)p.P + 2 * (size_t)hd.E + 1) * 4;   // selection | grouping
+      std::max((size_t)tpb * (hd.E + top_k) * 4,   // selection | grouping (pairs and 32 warps' counts in 16 bits)
+               2 * ((size_t)p.P + 1 + 32 * ((size_t)hd.E + 1)) + 4 * (2 * (size_t)hd.E + 1) + 8);
   if (router_smem > 200 * 1024) return BITSMOE_ERR_SHAPE;
   if ((rc = mark(0))) return rc;
   if ((rc = set_smem(k_router, router_smem))) return rc;
   if ((rc = launch(k_router, dim3((T + tpb - 1) / tpb), dim3(1024), router_smem, st, false, p))) return rc;
   if ((rc = mark(1))) return rc;
   const bool tc = L->maps;          // tensor-core projections for multi-token calls
-  const bool tcx = tc && L->tcx;    // and the expert factors on tensor cores
   const int A_max = std::min(hd.E, p.P);
-  if (tcx) {
-    // Experts with at least tc_min_tokens tokens take the tensor-core factor kernels (their codes
-    // are decoded once for all their tokens), the others the dp2a kernels (whose cost follows
-    // the tokens); each kind skips the other's experts, both add into s.  Cleared here: gu
-    // (dp2a gate/up adds into it), s, and the max |z| per token that the projection takes;
-    // z lies before them, zmax right after s.  The projection also stores z token-fastest.
-    p.tc_min = tc_min_tokens(hd);
-    XArgs xa = x_args(hd, T, top_k);
-    xa.tc_min = p.tc_min;
-    xa.msa = L->d_msa;
-    xa.zmax = reinterpret_cast<const uint32_t*>(wb + w.zmax);
-    xa.hb = wb + w.hb;
-    xa.hs = reinterpret_cast<float2*>(wb + w.hs);
-    xa.zv = reinterpret_cast<float*>(wb + w.zv);
-    BM_CK(cudaMemsetAsync(p.z, 0, w.zmax + 2 * (size_t)T * 4 - w.z, st));
-    BM_CK(launch_gemm_tc(0, L->map_in, p, sms, st, false, p.zT, nullptr, 0, reinterpret_cast<uint32_t*>(wb + w.zmax)));
+  if (mma) {
+    // z and max |z| per token, then gate/up and down over token tiles; the projection clears gu and s
+    const size_t zb = (size_t)(reinterpret_cast<uint8_t*>(p.s) - reinterpret_cast<uint8_t*>(p.gu)) +
+                      (size_t)T * hd.n_pad * 4;
+    BM_CK(launch_gemm_tc(0, L->map_in, p, sms, st, pdl, p.gu, zb, p.zmax));
     if ((rc = mark(2))) return rc;
-    BM_CK(launch_zgather(p, xa, sms, st, pdl));
-    BM_CK(launch_gu16(p, xa, sms, st, pdl));
-    if (G == 1) rc = launch_k2k3_dec<1, 4>(p, A_max, sms, st, pdl, std::function<int()>(), 1);
-    else if (G == 2) rc = launch_k2k3_dec<2, 4>(p, A_max, sms, st, pdl, std::function<int()>(), 1);
-    else rc = launch_k2k3_dec<4, 4>(p, A_max, sms, st, pdl, std::function<int()>(), 1);
-    if (rc) return rc;
+    BM_CK(launch_expert_mma(false, p, ma, sms, st, pdl));
     if ((rc = mark(3))) return rc;
-    BM_CK(launch_dn16(p, xa, sms, st, pdl));
-    if (G == 1) rc = launch_k2k3_dec<1, 4>(p, A_max, sms, st, pdl, std::function<int()>(), 2);
-    else if (G == 2) rc = launch_k2k3_dec<2, 4>(p, A_max, sms, st, pdl, std::function<int()>(), 2);
-    else rc = launch_k2k3_dec<4, 4>(p, A_max, sms, st, pdl, std::function<int()>(), 2);
-    if (rc) return rc;
+    BM_CK(launch_expert_mma(true, p, ma, sms, st, pdl));
   } else {
     if (tc) {
       // the dp2a gate/up and down kernels add into gu and s (cleared here with z, which lies
@@ -1822,16 +1831,12 @@ int upload(std::vector<uint8_t>&& img, int device, bitsmoe_layer** out) {
     const ImageHeader* h = header_of(img.data());
     L->maps = make_basis_map(L->map_in, d + h->off_basis_in, 2 * h->n, h->D_pad) &&
               make_basis_map(L->map_out, d + h->off_basis_out, h->D, h->n_pad);
-    bool ok16 = h->group % kRows == 0;
     const ExpertDesc* xd = desc_of(img.data());
-    for (int i = 0; i < 2 * h->E; ++i) {
-      for (int k = 0; k < xd[i].nbk; ++k)
-        if (xd[i].bk[k].bits >= 16) ok16 = false;
-    }
-    for (int i = 2 * h->E; i < 3 * h->E; ++i)
-      for (int k = 0; k < xd[i].nbk; ++k)
-        if (xd[i].bk[k].bits >= 16) ok16 = false;
-    L->tcx = ok16;
+    bool no16 = true;
+    for (int i = 0; i < 3 * h->E; ++i)
+      for (int k = 0; k < xd[i].nbk; ++k) no16 &= xd[i].bk[k].bits < 16;
+    for (int az = 0; az < 2; ++az) L->gu_stage[az] = mma_gu_stage(cst, std::max(1, kRows / h->group), az != 0);
+    L->mma = no16 && L->maps && L->meta_ok;
   }
   const ImageHeader* hd = header_of(img.data());
   const size_t meta_end = hd->off_basis_in;   // header + descriptors + segments
@@ -2000,8 +2005,9 @@ int forward_launches(const bitsmoe_layer* L, int T, int top_k, bool allow_f2) {
   const int s16 = (int)align_up(std::max(hd.seg_max_slots, 8), 64) + 8;
   if (decode && L->meta_ok && fused_plan(hd, T, top_k, L->seg_bytes, L->ul_max_chunks, s16, L->num_sms, &fa)) return 1;
   if (T <= kFusedMaxTokens && fused_fits(L, top_k)) return T;   // one fused forward per token
-  if (decode || !L->maps) return 5;
-  return L->tcx ? 8 : 5;   // router, projection, [z gather, gate/up tc,] gate/up, [down tc,] down, output basis
+  MArgs ma;
+  if (decode || !mma_fits(L, T, top_k, &ma)) return 5;   // router, projection, gate/up, down, output basis
+  return 6;                                              // and the gate/up operand's gather
 }
 }  // namespace
 
@@ -2017,7 +2023,8 @@ int bitsmoe_forward_plan(const bitsmoe_layer* L, int T, int top_k) {
   if (T <= kFusedMaxTokens && fused_fits(L, top_k)) return 1;
   const ImageHeader& hd = L->hd();
   if (decode_mode(hd, T)) return 2 | (L->maps && T >= 4 ? 4 : 0);
-  return L->maps ? 4 | (L->tcx ? 8 | 16 : 0) : 0;
+  MArgs ma;
+  return L->maps ? 4 | (mma_fits(L, T, top_k, &ma) ? 8 | 16 : 0) : 0;
 }
 
 int bitsmoe_block_forward_launches(const bitsmoe_layer* L, int T, int top_k) {

@@ -40,7 +40,7 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
 }
 
 struct GemmArgs {
-  int mode;          // 0: projection (B = x, writes z and optionally zT); 1: output basis (B = s hi/lo, y)
+  int mode;          // 0: projection (B = x, writes z); 1: output basis (B = s hi/lo, y)
   int M;             // rows of A (2n or D)
   int K;             // reduction length (D or n); A rows hold K_pad >= K elements
   int T;             // tokens of the call
@@ -57,8 +57,8 @@ struct GemmArgs {
   int accum;         // mode 1: y += (y holds the residual) instead of y =
   const uint16_t* x; // mode 0: [T][D] bf16 bits
   const float* s;    // mode 1: [T][n_pad]
-  float* z;          // mode 0: [2][T][n_pad]
-  float* zT;         // mode 0: null, or [2][n_pad][T] (token fastest): also written
+  float* z;          // mode 0: [2][T][n_pad], or with zt [2][n_pad][T] (token fastest)
+  int zt;
   uint32_t* zmax;    // mode 0: null, or [2][T] max_j |z_h[t][j]| as fp32 bits (zeroed before)
   float* y;          // mode 1: [T][D]
   float4* zero;      // null, or a buffer of later kernels to clear (after the PDL wait)
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
     // B stagers: rows = tokens, 64 K elements a stage in 8 chunks of 16 bytes, 128-byte swizzle.
     // A thread's chunks go four at a time; the next four are requested before the current ones
     // are converted and stored (and before the wait for a ring slot).
-    pdl_wait();   // activations come from earlier kernels
+    if (g.mode == 1) pdl_wait();   // s comes from the kernel before; x from kernels before the router
     const int bt = tid - 64;   // 0 .. kStagers - 1
     if (g.zero) {   // a buffer that the following kernels accumulate into
       const size_t nthr = (size_t)gridDim.x * gridDim.y * kStagers;
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-  if (wid < 2) pdl_wait();   // the stores below target buffers of earlier kernels (y may hold the residual)
+  pdl_wait();   // y may hold the residual; the router clears zmax
   {
     // this CTA's share of the rows: the sum over the cluster's partials, stored
     const int rs = 128 / g.splits, rbeg = (int)rank * rs;
@@ -286,8 +286,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
         if (in) {
           if (g.mode == 0) {
             const int h = m >= g.n, j = m - h * g.n;
-            g.z[((size_t)h * g.T + t) * g.n_pad + j] = sum;
-            if (g.zT) g.zT[((size_t)h * g.n_pad + j) * g.T + t] = sum;
+            g.z[g.zt ? ((size_t)h * g.n_pad + j) * g.T + t : ((size_t)h * g.T + t) * g.n_pad + j] = sum;
           } else {
             float* yp = g.y + (size_t)t * g.D + m;
             *yp = g.accum ? *yp + sum : sum;
@@ -354,10 +353,13 @@ bool make_basis_map(void* map_out, const void* base, int rows, int cols_pad) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// mode 0: z = Phi_{g,u}^T x (and zT, when given) for all T tokens; mode 1:
+// mode 0: z = Phi_{g,u}^T x for all T tokens (zt: stored token-fastest).  The kernel before it on the stream is
+// the router, which starts after all earlier work (it is launched without programmatic overlap), so the
+// projection reads x and clears `zero` while the router still runs and waits for it only before it
+// stores (qw3_skew, 8 tokens: the router's 8 us off the chain).  mode 1:
 // y = Phi_dn s, or y += Phi_dn s when p.accum.  Plain stores: nothing to clear.
-cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cudaStream_t st, bool pdl, float* zT,
-                           void* zero, size_t zero_bytes, uint32_t* zmax) {
+cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cudaStream_t st, bool pdl, void* zero,
+                           size_t zero_bytes, uint32_t* zmax, bool zt) {
   static_assert(sizeof(CUtensorMap) == 128, "tensor map size");
   GemmArgs g;
   std::memset(&g, 0, sizeof(g));
@@ -374,7 +376,7 @@ cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cud
   g.x = p.x;
   g.s = p.s;
   g.z = p.z;
-  g.zT = zT;
+  g.zt = zt;
   g.zmax = zmax;
   g.zero = static_cast<float4*>(zero);
   g.zero_n = zero_bytes / 16;
@@ -392,6 +394,7 @@ cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cud
   for (int t0 = 0; t0 < p.T; t0 += 256) {
     const int nt = std::min(256, p.T - t0);
     g.t0 = t0;
+    if (t0 > 0) g.zero = nullptr;   // cleared by the first launch
     g.N = (nt + 15) / 16 * 16;
     g.stage = kATile + (uint32_t)g.N * 128 * (mode == 1 ? 2 : 1);
     // K splits (a cluster per 128-row tile): at most one CTA per SM, at most 4 (larger clusters

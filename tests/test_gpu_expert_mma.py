@@ -1,0 +1,76 @@
+"""GPU parity of the multi-token expert factors (mma.sync tiles of 8 and 16 tokens) at the sizes where
+their tiling can go wrong: expert loads around a token group (1, 7, 8, 9, 15 .. 17, 33), one and several
+row blocks and runs of row blocks, several segments, K-step remainders of every bit-width, odd expert
+counts, all scale groups, and both sides of the decode batch (operand gathered in the kernel or by its
+own launch).
+
+Tolerance: the operands are fp16 pairs (at least 21 bits) and the codes exact, so what remains is fp32
+summation over at most n + I terms and the output basis' bf16 pair (2^-17 of each term of s): below
+2^-17 sqrt(n) max|Phi s| / max|y| <= 1e-4 at these sizes.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-4
+BITS = {0: 0.1, 1: 0.15, 2: 0.2, 3: 0.15, 4: 0.15, 6: 0.15, 8: 0.1}
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2606_00079_gb300 as bm
+    torch.cuda.set_device(0)
+    return torch, bm
+
+
+@pytest.mark.parametrize("T,E,k,D,n,I,group,bits", [
+    (5, 33, 3, 96, 75, 128, 128, BITS),         # decode batch, one row block, odd expert count
+    (8, 4, 2, 128, 200, 1152, 128, BITS),       # nine row blocks: a full and a partial run of the down kernel
+    (8, 5, 1, 72, 61, 64, 32, BITS),            # rows past the units' length, four groups a row block
+    (9, 33, 1, 64, 75, 384, 128, BITS),         # first size past the decode batch
+    (17, 33, 2, 100, 90, 256, 64, BITS),        # odd expert count, tiles of 16, two groups a row block
+    (33, 3, 1, 64, 130, 512, 256, BITS),        # groups of two row blocks
+    (34, 2, 2, 256, 1100, 256, 128, {1: 1.0}),  # several segments of one bit-width
+    (34, 2, 2, 64, 1030, 128, 128, {3: .5, 4: .5}),
+    (40, 2, 1, 64, 515, 256, 32, {6: .5, 8: .5}),
+])
+def test_expert_tiles(env, T, E, k, D, n, I, group, bits):
+    torch, bm = env
+    spec = synth.scaled_spec(synth.WORKLOADS["tiny"], D=D, E=E, I=I, n=n, group=group, top_k=k)
+    layer = (synth.make_layer(spec, seed=T + n, bits_dist=bits, alpha_scale=4.0) if n <= D
+             else wide_layer(spec, T + n, bits))
+    L = bm.bitsmoe_pack(layer, device=0)
+    plan = bm.bitsmoe_forward_plan(L, T, k)
+    assert plan == (bm.PLAN_DECODE_CHAIN | bm.PLAN_TC_PROJECTIONS if T <= 8 else
+                    bm.PLAN_TC_PROJECTIONS | bm.PLAN_TC_GATE_UP | bm.PLAN_TC_DOWN)
+    x, logits = synth.make_inputs(spec, T, seed=T)
+    # uneven loads: the first experts hold 1, 7, 8, 9, .. of the first choices
+    e, t = 0, 0
+    for load in (1, 7, 8, 9, 15, 17, 33):
+        logits[t:t + load, e % E] += 10.0
+        e, t = e + 1, t + load
+    ws = bm.Workspace(L, T, k)
+    for _ in range(2):   # the second call on a used workspace
+        y = bm.moe_forward(L, torch.from_numpy(x.view(np.int16)).cuda(), torch.from_numpy(logits).cuda(), k, ws=ws)
+    torch.cuda.synchronize()
+    assert bm.bitsmoe_last_device_status(ws.ptr) == 0
+    ref = oracle.moe_forward_factored(layer, x, logits, k)
+    assert np.max(np.abs(y.cpu().numpy() - ref)) <= TOL * np.max(np.abs(ref))
+
+
+def wide_layer(spec, seed, bits):
+    """A layer with more units than features (n > D): random bases of norm-1 columns."""
+    layer = synth.make_layer(synth.scaled_spec(spec, D=spec.n), seed=seed, bits_dist=bits, alpha_scale=4.0,
+                             basis_method="householder")
+    rng = np.random.default_rng(seed)
+    b = rng.standard_normal((3, spec.D, spec.n)) / np.sqrt(spec.D)
+    layer.update(D=spec.D, basis=synth.f32_to_bf16_bits(b.astype(np.float32)))
+    return layer
