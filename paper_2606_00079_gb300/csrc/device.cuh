@@ -52,12 +52,9 @@ struct DStage;
 // Sizes and tables of the multi-token expert kernels on mma.sync (expert_mma.cu).
 struct MArgs {
   int ntm;                // groups of 8 tokens a warp's pass takes at most (1 or 2)
-  int use_az;             // the gate/up operand is gathered by a kernel of its own (past the decode batch)
-  float* az;              // [2][rt][nsp]: alpha z 2^S of every routed token in unit-slot order
-  int rt, nsp;            // its rows (routed tokens, experts padded to 8) and slots a row
   int A_max;              // bound on the call's routed experts
-  uint32_t gu_stage;      // bytes of a staged gate/up segment
-  int gu_r;               // row blocks a gate/up block works on at once
+  uint32_t gu_stage;      // bytes of a group's staged gate/up segment
+  int gu_r, gu_kh;        // row blocks of a group of gate/up warps, groups of a block
   int dn_rc;              // row blocks of a down run
   uint32_t dn_meta;       // bytes of a down tile's staged unit indices, alphas and scale/zero rows
   const CStage* cst;      // [2][E][nseg]
@@ -82,7 +79,7 @@ struct CStage {            // one per gate/up item (h < 2, e, segment)
   uint8_t bits[kNumBk];    // their bit-widths
   uint16_t ntl[kNumBk];    // tiles per touched bucket
   uint32_t meta0;          // offset in the metadata mirror of row block 0's [unit | alpha | scale/zero G rows]
-  uint32_t slot0;          // first slot in the projection's slot arrays
+  uint8_t pad_[4];
 };
 static_assert(sizeof(CStage) == 80, "CStage layout");
 
@@ -216,13 +213,13 @@ cudaError_t launch_fused(const Fwd& p, const FusedArgs& f, int sms, cudaStream_t
 // unless y carries a residual).
 bool make_basis_map(void* map_out, const void* base, int rows, int cols_pad);
 cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cudaStream_t st, bool pdl,
-                           void* zero = nullptr, size_t zero_bytes = 0, uint32_t* zmax = nullptr, bool zt = false);
+                           void* zero = nullptr, size_t zero_bytes = 0, uint32_t* zmax = nullptr);
 // Multi-token expert factors on mma.sync (expert_mma.cu): sizes for T tokens (false when the layer
-// does not fit; gu_stage from mma_gu_stage), then gate/up into p.gu and down into p.s (both zeroed
+// does not fit; stages[ntm - 1][R] from mma_gu_stage), then gate/up into p.gu and down into p.s (both zeroed
 // before).  Persistent: `sms` blocks.
-uint32_t mma_gu_stage(const std::vector<CStage>& cst, int G, bool az);
-uint64_t mma_az_floats(const ImageHeader& hd, int T, int k, int* rt, int* nsp);
-bool mma_args(const ImageHeader& hd, int T, int k, bool az, uint32_t gu_stage, MArgs* x);
+constexpr int kMmaWarps = 12;
+uint32_t mma_gu_stage(const std::vector<CStage>& cst, int G, int ntm, int R);
+bool mma_args(const ImageHeader& hd, int T, int k, const uint32_t (&stages)[2][kMmaWarps + 1], MArgs* x);
 cudaError_t launch_expert_mma(bool down, const Fwd& p, const MArgs& x, int sms, cudaStream_t st, bool pdl);
 // Staging records of a packed image (host side, at upload).
 bool build_stage_tables(const uint8_t* img, std::vector<CStage>& cst, std::vector<DStage>& dst,

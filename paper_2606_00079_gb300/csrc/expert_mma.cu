@@ -32,9 +32,11 @@
 #include <mutex>
 
 #include "device.cuh"
+#include "tc.cuh"
 
 namespace {
 
+constexpr int kCW = kMmaWarps;      // consumer warps of the gate/up kernel
 constexpr int kStagePiece = 4096;   // bytes of down codes a warp stages at a time
 
 // Token tiles of the call, and their share of a kernel's work: active expert a has cnt[a] tokens from
@@ -47,10 +49,9 @@ struct MTiles {
   int* pst;
   int* ub;    // [na + 1]
   int* wb;    // [na + 1]
-  int* row;   // first row of the expert's tokens, experts padded to 8 rows
   int na;
 };
-__host__ __device__ inline uint32_t mtiles_bytes(int A_max) { return ((6u * (uint32_t)A_max + 2u) * 4u + 15u) & ~15u; }
+__host__ __device__ inline uint32_t mtiles_bytes(int A_max) { return ((5u * (uint32_t)A_max + 2u) * 4u + 15u) & ~15u; }
 
 __device__ MTiles mtiles_at(uint8_t* sm, int A_max) {
   MTiles t;
@@ -59,7 +60,6 @@ __device__ MTiles mtiles_at(uint8_t* sm, int A_max) {
   t.pst = t.cnt + A_max;
   t.ub = t.pst + A_max;
   t.wb = t.ub + A_max + 1;
-  t.row = t.wb + A_max + 1;
   t.na = 0;
   return t;
 }
@@ -83,30 +83,25 @@ __device__ void mtiles_build(const Fwd& p, int A_max, int NT, MTiles& t, F per_t
   }
   __syncthreads();
   if (tid < 32) {   // exclusive prefixes
-    int ru = 0, rw = 0, rr = 0;
+    int ru = 0, rw = 0;
     for (int a0 = 0; a0 < t.na; a0 += 32) {
       const int a = a0 + lane;
       const int u = a < t.na ? t.ub[a] : 0, w = a < t.na ? t.wb[a] : 0;
-      const int r8 = a < t.na ? (t.cnt[a] + 7) & ~7 : 0;
-      int ui = u, wi = w, ri = r8;
+      int ui = u, wi = w;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int v1 = __shfl_up_sync(0xFFFFFFFFu, ui, o), v2 = __shfl_up_sync(0xFFFFFFFFu, wi, o);
-        const int v3 = __shfl_up_sync(0xFFFFFFFFu, ri, o);
         if (lane >= o) {
           ui += v1;
           wi += v2;
-          ri += v3;
         }
       }
       if (a < t.na) {
         t.ub[a] = ru + ui - u;
         t.wb[a] = rw + wi - w;
-        t.row[a] = rr + ri - r8;
       }
       ru += __shfl_sync(0xFFFFFFFFu, ui, 31);
       rw += __shfl_sync(0xFFFFFFFFu, wi, 31);
-      rr += __shfl_sync(0xFFFFFFFFu, ri, 31);
     }
     if (lane == 0) {
       t.ub[t.na] = ru;
@@ -191,75 +186,37 @@ __device__ __forceinline__ void a_regs2(uint32_t w, int sh, uint32_t mul, uint32
 }
 
 // ---------------------------------------------------------------------------
-// Gate/up operand of calls past the decode batch
-// ---------------------------------------------------------------------------
-// az[h][row][slot]: alpha z 2^S of every (projection, routed token), in the order in which a warp of the
-// gate/up kernel reads it: a token tile of `rows` rows (a multiple of 8) holds [slot / 4][row][4], so that a
-// K-step of 8 tokens is one 16-byte load a lane (four full lines a warp).  Gathered in the kernel itself, z
-// costs four 4-byte loads from as many sectors for each of a tile's row blocks (1024 tokens of the
-// Qwen3-shaped layer: gate/up 988 us).
-constexpr int kZgThreads = 256;
-constexpr int kZgQuads = 128;   // slot quads of a work item (8 tokens each)
-
-__global__ void __launch_bounds__(kZgThreads) k_zgather(Fwd p, MArgs x) {
-  extern __shared__ __align__(128) uint8_t msm[];
-  __shared__ int s_ok;
-  const int tid = threadIdx.x, kNT = 8 * x.ntm;
-  MTiles tb = mtiles_at(msm, x.A_max);
-  pdl_trigger();
-  if (tid == 0) s_ok = wait_flag(p.route_flag);
-  __syncthreads();
-  if (!s_ok) {
-    if (tid == 0) atomicCAS(p.status, 0, BITSMOE_ERR_TIMEOUT);
-    pdl_wait();
-    return;
-  }
-  mtiles_build(p, x.A_max, 8, tb, [](int) { return 1; });
-  const int ng = tb.ub[tb.na], nch = (x.nsp / 4 + kZgQuads - 1) / kZgQuads;
-  pdl_wait();   // z and max |z| come from the projection
-  const int tk = tid & 7, q0 = tid >> 3;
-  for (int w = blockIdx.x; w < ng * 2 * nch; w += gridDim.x) {
-    const int gi = w % ng, hc = w / ng, h = hc & 1, ch = hc >> 1;
-    const int a = find_le(tb.ub, tb.na, gi), e = tb.e[a], n8 = gi - tb.ub[a];
-    const ExpertDesc& xd = p.desc[h * p.E + e];
-    const int nq = __ldg(&xd.nslots) >> 2;
-    const int* un = reinterpret_cast<const int*>(p.img + __ldg(&xd.unit_off));
-    const float* al = reinterpret_cast<const float*>(p.img + __ldg(&xd.alpha_off));
-    const int tt = n8 / x.ntm, rows = min(kNT, ((tb.cnt[a] - tt * kNT) + 7) & ~7);
-    const bool live = 8 * n8 + tk < tb.cnt[a];
-    const int tok = live ? p.pair_list[tb.pst[a] + 8 * n8 + tk] / p.k : 0;
-    const float bs = live ? scale_pow2(__ldg(x.msa + h * p.E + e) * __uint_as_float(__ldcg(p.zmax + h * p.T + tok))) : 0.f;
-    const float* z = p.z + ((size_t)h * p.T + tok) * p.n_pad;
-    float* dst = x.az + ((size_t)h * x.rt + tb.row[a] + tt * kNT) * x.nsp + (size_t)((n8 - tt * x.ntm) * 8 + tk) * 4;
-#pragma unroll
-    for (int i = 0; i < kZgQuads / (kZgThreads / 8); ++i) {
-      const int q = ch * kZgQuads + q0 + i * (kZgThreads / 8);
-      if (q < nq) {
-        const int4 u = __ldg(reinterpret_cast<const int4*>(un) + q);
-        const float4 av = __ldg(reinterpret_cast<const float4*>(al) + q);
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (live) v = make_float4(av.x * z[u.x] * bs, av.y * z[u.y] * bs, av.z * z[u.z] * bs, av.w * z[u.w] * bs);
-        *reinterpret_cast<float4*>(dst + (size_t)q * rows * 4) = v;
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
 // Gate/up
 // ---------------------------------------------------------------------------
 // Units in (token tile, projection, group of R row blocks, segment) order.  A block takes a contiguous run
-// of units; inside it, warp w has row block w % R of the group and part w / R of each run of segments, so
-// that the warps of a block read the same operand (L1).  A warp streams its segments' codes and slot
-// metadata through its own two-stage ring (two bulk copies a segment) and adds its partial rows into
-// gate/up.  The operand is az (AZ), or for the decode batch (at most 8 tokens, no extra launch) gathered
-// from z stored token-fastest, where a unit's 8 tokens are one sector.
+// of units.  Its 12 consumer warps form KH groups of R: the warps of a group work on the same segment, one
+// row block each, and the groups take parts of each run of segments.  4 / KH helper warps a group fill its
+// two-stage ring: bulk copies of the R row blocks' codes and scale/zero rows, and the operand alpha z 2^S of
+// the segment's slots, gathered from z once for the group (the consumers, at three warps a scheduler, cannot
+// hide a global load: gathering in them, or reading a gathered copy from memory, left long-scoreboard stalls
+// of 3 issue slots an instruction).  The consumers decode, multiply and add their partial rows into gate/up.
+constexpr int kHW = 4;                       // helper warps
+constexpr int kGuThreads = (kCW + kHW) * 32;
+constexpr int kMaxKH = 4;
+
 struct GCur {
   int pos;               // unit at which the current (tile, projection, row group) run starts (>= hi: the end)
   int end;               // its end (inside the block's units)
-  int a, tt, h, rb;      // expert index and token tile, projection, row block
-  int sg, sg1;           // segment, end of the warp's part
+  int a, tt, h, rg;      // expert index and token tile, projection, group of row blocks
+  int sg, sg1;           // segment, end of the group's part
   int first;
+};
+
+// A stage's description for the consumers.
+struct GInfo {
+  CStage rec;
+  int flags;             // 1 first of the run, 2 last, 4 end of the block's work
+  int h, rg, ntk, run;   // projection, group of row blocks, tokens of the tile, parity of the run
+  int pad_[3];
+};
+struct GRun {            // rows of a run's token tile
+  int pair[16];
+  float inv[16];         // 2^-S
 };
 
 // 32 rows (from byte row16 of a chunk) of K-step ks of a bucket: A registers of rows 4 g .. 4 g + 3.
@@ -276,7 +233,7 @@ __device__ __forceinline__ void rl_a(const uint8_t* code, int ks, int ntl, int r
     a_regs2<2, 1>(w.z, sh, mul, h.z, hs, lo[2], hi[2]);
     a_regs2<2, 1>(w.w, sh, mul, h.w, hs, lo[3], hi[3]);
   } else if (B == 6) {
-    const uint8_t* c = code + min(ks, ntl - 1) * (3 * kChunkBytes) + row16;
+    const uint8_t* c = code + ks * (3 * kChunkBytes) + row16;
     const uint4 w = ld4s(c + (t >> 1) * kChunkBytes), h = ld4s(c + 2 * kChunkBytes);
     const int sh = 4 * (t & 1), hs = 2 * t;
     const uint32_t mul = 1u << (code_pos<6>() - sh);
@@ -285,7 +242,7 @@ __device__ __forceinline__ void rl_a(const uint8_t* code, int ks, int ntl, int r
     a_regs2<4, 2>(w.z, sh, mul, h.z, hs, lo[2], hi[2]);
     a_regs2<4, 2>(w.w, sh, mul, h.w, hs, lo[3], hi[3]);
   } else {
-    const int tile = B == 1 ? ks >> 1 : min(B == 2 ? ks : B == 4 ? 2 * ks + (t >> 1) : 4 * ks + t, ntl - 1);
+    const int tile = B == 1 ? ks >> 1 : B == 2 ? ks : min(B == 4 ? 2 * ks + (t >> 1) : 4 * ks + t, ntl - 1);
     const int sh = B == 1 ? t + 4 * (ks & 1) : B == 2 ? 2 * t : B == 4 ? 4 * (t & 1) : 0;
     const uint32_t mul = 1u << (code_pos<B>() - sh);
     const uint4 w = ld4s(code + tile * kChunkBytes + row16);
@@ -296,45 +253,18 @@ __device__ __forceinline__ void rl_a(const uint8_t* code, int ks, int ntl, int r
   }
 }
 
-// What a lane reads its operand from (run of one token tile and projection).
+// Operand rows in shared memory: [slot quad][8 NTM rows][4 slots] fp32, the quads kQS bytes apart (32 bytes
+// of padding: the four K lanes of a warp then read different banks).
 template <int NTM>
-struct GOp {
-  const float* az;          // AZ: the tile's az, at this lane's token row
-  int rows4;                //     floats between slot quads
-  const float* zt[NTM];     // else: z column of this lane's token (unit-major)
-  int zstride;              //     floats between units
-  float bs[NTM];            //     2^S of this lane's token
-};
+__host__ __device__ constexpr int az_quad() { return 128 * NTM + 32; }
 
-// A warp's K-steps: KP an iteration; NT groups of 8 tokens; the next iteration's operand is loaded while
-// this one is computed, across the buckets of a segment (AZ: across the run's segments too).
-template <int NT, int KP, int NTM, bool AZ>
-__device__ __forceinline__ void gu_load(const GOp<NTM>& o, const int* su, int slot, int limit, float4 (&zn)[KP][NT]) {
-#pragma unroll
-  for (int k = 0; k < KP; ++k) {
-    const int s = min(slot + 16 * k, limit);
-    if (AZ) {
-      const float* q = o.az + (s >> 2) * o.rows4;
-#pragma unroll
-      for (int n = 0; n < NT; ++n) zn[k][n] = *reinterpret_cast<const float4*>(q + 32 * n);
-    } else {
-      const int4 u = *reinterpret_cast<const int4*>(su + s);
-#pragma unroll
-      for (int n = 0; n < NT; ++n)
-        zn[k][n] = make_float4(__ldcg(o.zt[n] + u.x * o.zstride), __ldcg(o.zt[n] + u.y * o.zstride),
-                               __ldcg(o.zt[n] + u.z * o.zstride), __ldcg(o.zt[n] + u.w * o.zstride));
-    }
-  }
-}
-
-// A bucket's run of tiles; s0: its first slot (in the segment, AZ: in the projection), limit: the last slot
-// quad that may be loaded ahead, sa / ssz at its first slot (ssz rows `zs` words apart), G scale groups
-// inside the 128 rows.
-template <int B, int NT, int KP, int NTM, int G, bool AZ>
-__device__ __forceinline__ void gu_bucket(const uint8_t* code, int ntl, const GOp<NTM>& o, const int* su, int s0, int limit,
-                                          const float* sa, const uint32_t* ssz, int zs, int lane, float4 (&zn)[KP][NT],
-                                          float (&acc)[8][NTM][4], float (&cs)[G][NTM]) {
+// A bucket's run of tiles: NT groups of 8 tokens, G scale groups inside the 128 rows; az: the operand of the
+// bucket's first slot at this lane's row, ssz: its scale/zero word (rows `zs` words apart).
+template <int B, int NT, int NTM, int G>
+__device__ __forceinline__ void gu_bucket(const uint8_t* code, int ntl, const uint8_t* az, const uint32_t* ssz, int zs,
+                                          int lane, float (&acc)[8][NTM][4], float (&cs)[G][NTM]) {
   constexpr float fB = 1.f / (float)(1 << (code_pos<B>() - 3));   // the code's position, taken back in B
+  constexpr int kQS = az_quad<NTM>(), JP = G <= 2 ? 2 : 1;
   const int g = lane >> 2, t = lane & 3;
   const int nsl = ntl * rl_units(B), nks = (nsl + 15) >> 4;
   float ce[G][NT];   // zero-point corrections
@@ -343,63 +273,45 @@ __device__ __forceinline__ void gu_bucket(const uint8_t* code, int ntl, const GO
 #pragma unroll
     for (int n = 0; n < NT; ++n) ce[gl][n] = 0.f;
 #pragma unroll 1
-  for (int ks = 0; ks < nks; ks += KP) {
-    float4 zc[KP][NT];
+  for (int ks = 0; ks < nks; ++ks) {
+    const int sl = 16 * ks + 4 * t, slc = min(sl, nsl - 4);
+    const float f = sl < nsl ? fB : 0.f;   // past the bucket: the codes read are another slot's
+    float4 zc[NT];
 #pragma unroll
-    for (int k = 0; k < KP; ++k)
-#pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        zc[k][n] = zn[k][n];
-        if (!AZ) {
-          zc[k][n].x *= o.bs[n];
-          zc[k][n].y *= o.bs[n];
-          zc[k][n].z *= o.bs[n];
-          zc[k][n].w *= o.bs[n];
-        }
-      }
-    gu_load<NT, KP, NTM, AZ>(o, su, s0 + (ks + KP < nks ? 16 * (ks + KP) : nsl) + 4 * t, limit, zn);
+    for (int n = 0; n < NT; ++n) zc[n] = *reinterpret_cast<const float4*>(az + (slc >> 2) * kQS + 128 * n);
 #pragma unroll
     for (int gl = 0; gl < G; ++gl) {
-      uint32_t bh[KP][NT][2], bl[KP][NT][2];
+      uint32_t bh[NT][2], bl[NT][2];
+      const uint4 sz = *reinterpret_cast<const uint4*>(ssz + gl * zs + slc);
+      const float w0 = f16lo(sz.x) * f, w1 = f16lo(sz.y) * f, w2 = f16lo(sz.z) * f, w3 = f16lo(sz.w) * f;
 #pragma unroll
-      for (int k = 0; k < KP; ++k) {
-        const int sl = 16 * (ks + k) + 4 * t, slc = min(sl, nsl - 4);
-        uint4 sz = *reinterpret_cast<const uint4*>(ssz + gl * zs + slc);
-        const float f = sl < nsl ? fB : 0.f;   // past the bucket: the codes read are another slot's
-        float w0 = f16lo(sz.x) * f, w1 = f16lo(sz.y) * f, w2 = f16lo(sz.z) * f, w3 = f16lo(sz.w) * f;
-        if (!AZ) {
-          const float4 al = *reinterpret_cast<const float4*>(sa + slc);
-          w0 *= al.x;
-          w1 *= al.y;
-          w2 *= al.z;
-          w3 *= al.w;
-        }
-#pragma unroll
-        for (int n = 0; n < NT; ++n) {
-          const float v0 = w0 * zc[k][n].x, v1 = w1 * zc[k][n].y, v2 = w2 * zc[k][n].z, v3 = w3 * zc[k][n].w;
-          ce[gl][n] = fmaf(f16hi(sz.x), v0, fmaf(f16hi(sz.y), v1, fmaf(f16hi(sz.z), v2, fmaf(f16hi(sz.w), v3, ce[gl][n]))));
-          split_pair(v0, v2, bh[k][n][0], bl[k][n][0]);
-          split_pair(v1, v3, bh[k][n][1], bl[k][n][1]);
-        }
+      for (int n = 0; n < NT; ++n) {
+        const float v0 = w0 * zc[n].x, v1 = w1 * zc[n].y, v2 = w2 * zc[n].z, v3 = w3 * zc[n].w;
+        ce[gl][n] = fmaf(f16hi(sz.x), v0, fmaf(f16hi(sz.y), v1, fmaf(f16hi(sz.z), v2, fmaf(f16hi(sz.w), v3, ce[gl][n]))));
+        split_pair(v0, v2, bh[n][0], bl[n][0]);
+        split_pair(v1, v3, bh[n][1], bl[n][1]);
       }
 #pragma unroll
-      for (int jj = 0; jj < 4 / G; ++jj) {
-        const int j = gl * (4 / G) + jj;
+      for (int jj = 0; jj < 4 / G; jj += JP) {
+        uint32_t lo[JP][4], hi[JP][4];
 #pragma unroll
-        for (int k = 0; k < KP; ++k) {
-          uint32_t lo[4], hi[4];
-          rl_a<B>(code, ks + k, ntl, 16 * (8 * j + g), t, lo, hi);
+        for (int q = 0; q < JP; ++q) rl_a<B>(code, ks, ntl, 16 * (8 * (gl * (4 / G) + jj + q) + g), t, lo[q], hi[q]);
 #pragma unroll
-          for (int n = 0; n < NT; ++n) {
-            mma_16816(acc[2 * j][n], lo[0], lo[1], hi[0], hi[1], bl[k][n][0], bl[k][n][1]);
-            mma_16816(acc[2 * j + 1][n], lo[2], lo[3], hi[2], hi[3], bl[k][n][0], bl[k][n][1]);
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+          for (int q = 0; q < JP; ++q) {
+            const int j = gl * (4 / G) + jj + q;
+            mma_16816(acc[2 * j][n], lo[q][0], lo[q][1], hi[q][0], hi[q][1], bl[n][0], bl[n][1]);
+            mma_16816(acc[2 * j + 1][n], lo[q][2], lo[q][3], hi[q][2], hi[q][3], bl[n][0], bl[n][1]);
           }
 #pragma unroll
-          for (int n = 0; n < NT; ++n) {
-            mma_16816(acc[2 * j][n], lo[0], lo[1], hi[0], hi[1], bh[k][n][0], bh[k][n][1]);
-            mma_16816(acc[2 * j + 1][n], lo[2], lo[3], hi[2], hi[3], bh[k][n][0], bh[k][n][1]);
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+          for (int q = 0; q < JP; ++q) {
+            const int j = gl * (4 / G) + jj + q;
+            mma_16816(acc[2 * j][n], lo[q][0], lo[q][1], hi[q][0], hi[q][1], bh[n][0], bh[n][1]);
+            mma_16816(acc[2 * j + 1][n], lo[q][2], lo[q][3], hi[q][2], hi[q][3], bh[n][0], bh[n][1]);
           }
-        }
       }
     }
   }
@@ -409,222 +321,293 @@ __device__ __forceinline__ void gu_bucket(const uint8_t* code, int ntl, const GO
     for (int n = 0; n < NT; ++n) cs[gl][n] = fmaf(ce[gl][n], 1.f / fB, cs[gl][n]);
 }
 
-template <int NT, int KP, int NTM, int G, bool AZ>
-__device__ __forceinline__ void gu_segment(const CStage& r, const uint8_t* st, const GOp<NTM>& o, int limit, int lane,
-                                           bool first, float4 (&zn)[KP][NTM], float (&acc)[8][NTM][4], float (&cs)[G][NTM]) {
-  const int zs = (int)(r.mb >> 2);
-  const int* su = reinterpret_cast<const int*>(st + r.bytes);                       // !AZ only
-  const float* sa = reinterpret_cast<const float*>(su + zs);                        // !AZ only
-  const uint32_t* sz = reinterpret_cast<const uint32_t*>(st + r.bytes + (AZ ? 0u : 2u * r.mb));
-  int s0 = AZ ? (int)r.slot0 : 0;
-  const int lim = AZ ? limit : zs - 4;
-  float4 z[KP][NT];
-#pragma unroll
-  for (int k = 0; k < KP; ++k)
-#pragma unroll
-    for (int n = 0; n < NT; ++n) z[k][n] = zn[k][n];
-  if (!AZ || first) gu_load<NT, KP, NTM, AZ>(o, su, s0 + 4 * (lane & 3), lim, z);
-  for (int q = 0; q < r.nr; ++q) {
+// A staged segment: st = the warp's codes, sz its scale/zero rows, az the group's operand at this lane's row.
+template <int NT, int NTM, int G>
+__device__ __forceinline__ void gu_segment(const CStage& r, const uint8_t* st, const uint32_t* sz, const uint8_t* az,
+                                           int lane, float (&acc)[8][NTM][4], float (&cs)[G][NTM]) {
+  const int zs = (int)(r.mb >> 2), nr = r.nr;
+  for (int q = 0; q < nr; ++q) {
     const int b = r.bits[q], ntl = r.ntl[q];
     switch (b) {
-      case 1: gu_bucket<1, NT, KP, NTM, G, AZ>(st, ntl, o, su, s0, lim, sa, sz, zs, lane, z, acc, cs); break;
-      case 2: gu_bucket<2, NT, KP, NTM, G, AZ>(st, ntl, o, su, s0, lim, sa, sz, zs, lane, z, acc, cs); break;
-      case 3: gu_bucket<3, NT, KP, NTM, G, AZ>(st, ntl, o, su, s0, lim, sa, sz, zs, lane, z, acc, cs); break;
-      case 4: gu_bucket<4, NT, KP, NTM, G, AZ>(st, ntl, o, su, s0, lim, sa, sz, zs, lane, z, acc, cs); break;
-      case 6: gu_bucket<6, NT, KP, NTM, G, AZ>(st, ntl, o, su, s0, lim, sa, sz, zs, lane, z, acc, cs); break;
-      default: gu_bucket<8, NT, KP, NTM, G, AZ>(st, ntl, o, su, s0, lim, sa, sz, zs, lane, z, acc, cs); break;
+      case 1: gu_bucket<1, NT, NTM, G>(st, ntl, az, sz, zs, lane, acc, cs); break;
+      case 2: gu_bucket<2, NT, NTM, G>(st, ntl, az, sz, zs, lane, acc, cs); break;
+      case 3: gu_bucket<3, NT, NTM, G>(st, ntl, az, sz, zs, lane, acc, cs); break;
+      case 4: gu_bucket<4, NT, NTM, G>(st, ntl, az, sz, zs, lane, acc, cs); break;
+      case 6: gu_bucket<6, NT, NTM, G>(st, ntl, az, sz, zs, lane, acc, cs); break;
+      default: gu_bucket<8, NT, NTM, G>(st, ntl, az, sz, zs, lane, acc, cs); break;
     }
     st += (uint32_t)ntl * rl_chunks(b) * kChunkBytes;
     const int ns = ntl * rl_units(b);
-    s0 += ns;
-    sa += ns;
+    az += (ns >> 2) * az_quad<NTM>();
     sz += ns;
   }
-#pragma unroll
-  for (int k = 0; k < KP; ++k)
-#pragma unroll
-    for (int n = 0; n < NT; ++n) zn[k][n] = z[k][n];
 }
 
-constexpr int kMW = 12;   // warps of a block
+// Registers of the consumer and helper warps: 3 x 128 x 144 + 128 x 80 = 65536, what the block is launched
+// with (512 x 128).
+__device__ __forceinline__ void regs_consumer() { asm volatile("setmaxnreg.inc.sync.aligned.u32 144;"); }
+__device__ __forceinline__ void regs_helper() { asm volatile("setmaxnreg.dec.sync.aligned.u32 80;"); }
 
-template <int NTM, int G, bool AZ>
-__global__ void __launch_bounds__(kMW * 32, 1) k_gu_mma(Fwd p, MArgs x) {
-  constexpr int kNT = 8 * NTM, KP = NTM == 1 ? 2 : 1;
-  const int kW = (int)blockDim.x >> 5;   // as many warps as their rings fit in shared memory
+template <int NTM, int G>
+__global__ void __launch_bounds__(kGuThreads, 1) k_gu_mma(Fwd p, MArgs x) {
+  constexpr int kNT = 8 * NTM, kQS = az_quad<NTM>();
   extern __shared__ __align__(128) uint8_t msm[];
-  __shared__ uint64_t bars[kMW][2];
-  __shared__ CStage recs[kMW][2];
+  __shared__ uint64_t full[kMaxKH][2], empty[kMaxKH][2];
+  __shared__ __align__(16) GInfo infos[kMaxKH][2];
+  __shared__ GRun runs[kMaxKH][2];
   __shared__ int s_ok;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3;
-  uint8_t* ring = msm + (size_t)wid * 2 * x.gu_stage;
-  MTiles tb = mtiles_at(msm + (size_t)kW * 2 * x.gu_stage, x.A_max);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int R = x.gu_r, KH = x.gu_kh, HG = kHW / KH;
+  MTiles tb = mtiles_at(msm + (size_t)KH * 2 * x.gu_stage, x.A_max);
 
   pdl_trigger();
-  if (lane == 0) {
-    mbar_init(&bars[wid][0]);
-    mbar_init(&bars[wid][1]);
+  if (tid == 0) {
+    for (int q = 0; q < KH; ++q)
+      for (int s = 0; s < 2; ++s) {
+        mbar_init_n(&full[q][s], 1 + HG);   // the copies' expectation, and each helper's part of the operand
+        mbar_init_n(&empty[q][s], R);
+      }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_ok = wait_flag(p.route_flag);
   }
-  if (tid == 0) s_ok = wait_flag(p.route_flag);
   __syncthreads();
   if (!s_ok) {
     if (tid == 0) atomicCAS(p.status, 0, BITSMOE_ERR_TIMEOUT);
     pdl_wait();
     return;
   }
-  const int R = x.gu_r, KH = kW / R, nrg = (p.NRB + R - 1) / R, M = 2 * nrg * p.nseg;
+  const int nrg = (p.NRB + R - 1) / R, M = 2 * nrg * p.nseg;
   mtiles_build(p, x.A_max, kNT, tb, [&](int) { return M; });
-  const int lo = cut_unit(tb, kNT, (int)blockIdx.x, (int)gridDim.x);
-  const int hi = cut_unit(tb, kNT, (int)blockIdx.x + 1, (int)gridDim.x);
-  const int wr = wid % R, wk = wid / R;   // row block of the group, part of the run (wk == KH: no work)
+  bool ok = true;
 
-  // the warp's part of the run that starts at c.pos, skipping runs that have none for it
-  auto first_of = [&](GCur& c) {
-    for (; c.pos < hi; c.pos = c.end) {
-      const int tau = c.pos / M;
-      int i = c.pos - tau * M;
-      c.h = i >= nrg * p.nseg;
-      i -= c.h * nrg * p.nseg;
-      const int rg = i / p.nseg, s0 = i - rg * p.nseg;
-      c.end = min(hi, c.pos + p.nseg - s0);
-      c.rb = rg * R + wr;
-      if (wk >= KH || c.rb >= p.NRB) continue;
-      const int len = c.end - c.pos;
-      c.sg = s0 + len * wk / KH;
-      c.sg1 = s0 + len * (wk + 1) / KH;
-      if (c.sg == c.sg1) continue;
-      c.a = find_le(tb.ub, tb.na, c.pos);
-      c.tt = (c.pos - tb.ub[c.a]) / M;
-      c.first = 1;
+  if (wid >= kCW) {
+    // ---- helpers
+    regs_helper();
+    const int hw = wid - kCW, gr = hw / HG, sub = hw - gr * HG;
+    if (gr >= KH) {
+      pdl_wait();
       return;
     }
-  };
-  auto advance = [&](GCur& c) {
-    c.first = 0;
-    if (++c.sg < c.sg1) return;
-    c.pos = c.end;
+    const int lo = cut_unit(tb, kNT, (int)blockIdx.x, (int)gridDim.x);
+    const int hi = cut_unit(tb, kNT, (int)blockIdx.x + 1, (int)gridDim.x);
+    uint8_t* ring = msm + (size_t)gr * 2 * x.gu_stage;
+    // the group's part of the run that starts at c.pos, skipping runs that have none for it
+    auto first_of = [&](GCur& c) {
+      for (; c.pos < hi; c.pos = c.end) {
+        const int tau = c.pos / M;
+        int i = c.pos - tau * M;
+        c.h = i >= nrg * p.nseg;
+        i -= c.h * nrg * p.nseg;
+        c.rg = i / p.nseg;
+        const int s0 = i - c.rg * p.nseg;
+        c.end = min(hi, c.pos + p.nseg - s0);
+        const int len = c.end - c.pos;
+        c.sg = s0 + len * gr / KH;
+        c.sg1 = s0 + len * (gr + 1) / KH;
+        if (c.sg == c.sg1) continue;
+        c.a = find_le(tb.ub, tb.na, c.pos);
+        c.tt = (c.pos - tb.ub[c.a]) / M;
+        c.first = 1;
+        return;
+      }
+    };
+    auto advance = [&](GCur& c) {
+      c.first = 0;
+      if (++c.sg < c.sg1) return;
+      c.pos = c.end;
+      first_of(c);
+    };
+    // word `lane` of the cursor's staging record
+    auto record = [&](const GCur& c) -> uint32_t {
+      if (c.pos >= hi || lane >= (int)(sizeof(CStage) / 4)) return 0u;
+      return __ldg(reinterpret_cast<const uint32_t*>(x.cst + ((size_t)c.h * p.E + tb.e[c.a]) * p.nseg + c.sg) + lane);
+    };
+    auto pair_of = [&](const GCur& c) {   // lane < 16: the pair of the tile's row `lane`
+      const int ntk = min(kNT, tb.cnt[c.a] - c.tt * kNT);
+      return p.pair_list[tb.pst[c.a] + c.tt * kNT + min(lane & 15, ntk - 1)];
+    };
+    GCur c;
+    c.pos = lo;
     first_of(c);
-  };
-  // word `lane` of the cursor's staging record
-  auto record = [&](const GCur& c) -> uint32_t {
-    if (c.pos >= hi || lane >= (int)(sizeof(CStage) / 4)) return 0u;
-    return __ldg(reinterpret_cast<const uint32_t*>(x.cst + ((size_t)c.h * p.E + tb.e[c.a]) * p.nseg + c.sg) + lane);
-  };
-  auto issue = [&](int s, const GCur& c, uint32_t rw) {
-    if (lane < (int)(sizeof(CStage) / 4)) reinterpret_cast<uint32_t*>(&recs[wid][s])[lane] = rw;
-    const uint64_t code0 = (uint64_t)__shfl_sync(0xFFFFFFFFu, rw, 0) | ((uint64_t)__shfl_sync(0xFFFFFFFFu, rw, 1) << 32);
-    const uint32_t rbs = __shfl_sync(0xFFFFFFFFu, rw, 8), bytes = __shfl_sync(0xFFFFFFFFu, rw, 10);
-    const uint32_t mb = __shfl_sync(0xFFFFFFFFu, rw, 11), meta0 = __shfl_sync(0xFFFFFFFFu, rw, 18);
-    if (lane == 0) {
-      uint64_t* bar = &bars[wid][s];
-      uint8_t* dst = ring + (size_t)s * x.gu_stage;
-      // the record's metadata of a row block: unit indices, alphas (not needed beside az), scale/zero rows
-      const uint32_t skip = AZ ? 2u * mb : 0u, mt = bytes ? (2u + G) * mb - skip : 0u;
-      fence_proxy_async();   // the stage was last read by the generic proxy
-      mbar_expect_tx(bar, bytes + mt);
-      if (bytes) {
-        bulk_g2s(dst, p.img + code0 + (uint64_t)c.rb * rbs, bytes, bar);
-        bulk_g2s(dst + bytes, x.meta + meta0 + (size_t)c.rb * (2u + G) * mb + skip, mt, bar);
-      }
-    }
-  };
-
-  GCur c;
-  c.pos = lo;
-  first_of(c);
-  uint32_t rn = 0;
-  GCur n = c;
-  if (c.pos < hi) {
-    issue(0, c, record(c));
-    advance(n);
-    rn = record(n);
-  }
-  pdl_wait();   // z and max |z| come from the projection
-  bool ok = true;
-  float acc[8][NTM][4];
-  float cs[G][NTM];
-  GOp<NTM> o;
-  float4 zn[KP][NTM];
-  float inv[NTM];   // 2^-S of this lane's token
-  int ntk = 0, limit = 0;
-  bool need = false;   // the run's first operand is still to be loaded
-  for (int i = 0; c.pos < hi; ++i) {
-    __syncwarp();   // the other stage has been read by every lane
-    if (n.pos < hi) issue((i + 1) & 1, n, rn);
-    GCur n2 = n;
-    if (n.pos < hi) advance(n2);
-    rn = record(n2);
-    if (c.first) {   // the run's tokens, their operand and its powers of two
-      const int e = tb.e[c.a];
-      ntk = min(kNT, tb.cnt[c.a] - c.tt * kNT);
-      const float ms = __ldg(x.msa + c.h * p.E + e);
-      if (AZ) {
-        o.rows4 = 4 * min(kNT, (ntk + 7) & ~7);
-        o.az = x.az + ((size_t)c.h * x.rt + tb.row[c.a] + c.tt * kNT) * x.nsp + 4 * g;
-        limit = max(0, __ldg(&p.desc[c.h * p.E + e].nslots) - 4);
-      }
-      o.zstride = p.T;
-      need = true;
-#pragma unroll
-      for (int q = 0; q < NTM; ++q) {
-        const int tok = p.pair_list[tb.pst[c.a] + c.tt * kNT + min(8 * q + g, ntk - 1)] / p.k;
-        o.zt[q] = p.z + (size_t)c.h * p.n_pad * p.T + tok;
-        o.bs[q] = scale_pow2(ms * __uint_as_float(__ldcg(p.zmax + c.h * p.T + tok)));
-        inv[q] = 1.f / o.bs[q];
-#pragma unroll
-        for (int m = 0; m < 8; ++m)
-#pragma unroll
-          for (int w = 0; w < 4; ++w) acc[m][q][w] = 0.f;
-#pragma unroll
-        for (int gl = 0; gl < G; ++gl) cs[gl][q] = 0.f;
-      }
-    }
-    ok &= mbar_wait(&bars[wid][i & 1], (uint32_t)(i >> 1) & 1u);
-    __syncwarp();
-    const CStage& r = recs[wid][i & 1];
-    const uint8_t* st = ring + (size_t)(i & 1) * x.gu_stage;
-    if (r.nr > 0) {
-      if (NTM == 1 || ntk <= 8) gu_segment<1, KP, NTM, G, AZ>(r, st, o, limit, lane, need, zn, acc, cs);
-      else gu_segment<NTM, KP, NTM, G, AZ>(r, st, o, limit, lane, need, zn, acc, cs);
-      need = false;
-    }
-    if (c.sg + 1 == c.sg1) {   // the part's end: its partial rows into gate/up
-#pragma unroll
-      for (int q = 0; q < NTM; ++q) {
-        if (8 * q >= ntk) break;
-        float co[G];
-#pragma unroll
-        for (int gl = 0; gl < G; ++gl) {   // the token's correction, summed over the K lanes
-          float v = cs[gl][q];
-          v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
-          v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
-          co[gl] = v;
+    uint32_t rw = record(c);
+    int pr = c.pos < hi ? pair_of(c) : 0;
+    int tok = 0, run = 0;
+    float bs = 1.f;
+    for (int i = 0;; ++i) {
+      const int s = i & 1;
+      if (i >= 2) ok &= mbar_wait(&empty[gr][s], (uint32_t)((i >> 1) - 1) & 1u);
+      __syncwarp();
+      GInfo& f = infos[gr][s];
+      if (c.pos >= hi) {
+        if (lane == 0) {
+          if (sub == 0) {
+            f.flags = 4;
+            mbar_arrive(&full[gr][s]);
+          }
+          mbar_arrive(&full[gr][s]);
         }
+        if (i == 0) pdl_wait();
+        break;
+      }
+      GCur n = c;
+      advance(n);
+      const int ntk = min(kNT, tb.cnt[c.a] - c.tt * kNT);
+      const uint32_t bytes = __shfl_sync(0xFFFFFFFFu, rw, 10), mb = __shfl_sync(0xFFFFFFFFu, rw, 11);
+      const uint32_t meta0 = __shfl_sync(0xFFFFFFFFu, rw, 18), zb = G * mb;
+      uint8_t* st = ring + (size_t)s * x.gu_stage;
+      if (sub == 0) {   // the description, and the copies: lane r < R codes, lane 16 + r scale/zero rows of row block r
+        const uint64_t code0 =
+            (uint64_t)__shfl_sync(0xFFFFFFFFu, rw, 0) | ((uint64_t)__shfl_sync(0xFFFFFFFFu, rw, 1) << 32);
+        const uint32_t rbs = __shfl_sync(0xFFFFFFFFu, rw, 8);
+        if (lane < (int)(sizeof(CStage) / 4)) reinterpret_cast<uint32_t*>(&f.rec)[lane] = rw;
+        const int nrb = min(R, p.NRB - c.rg * R);
+        if (lane == 0) {
+          f.flags = (c.first ? 1 : 0) | (c.sg + 1 == c.sg1 ? 2 : 0);
+          f.h = c.h;
+          f.rg = c.rg;
+          f.ntk = ntk;
+          f.run = run & 1;
+          mbar_expect_tx(&full[gr][s], (uint32_t)nrb * (bytes + zb));
+        }
+        __syncwarp();
+        const int r = lane & 15, rb = c.rg * R + r;
+        if (r < nrb && bytes) {
+          fence_proxy_async();   // the stage was last read by the generic proxy
+          if (lane < 16) bulk_g2s(st + (size_t)r * bytes, p.img + code0 + (uint64_t)rb * rbs, bytes, &full[gr][s]);
+          else bulk_g2s(st + (size_t)R * bytes + (size_t)r * zb, x.meta + meta0 + (size_t)rb * (2u + G) * mb + 2u * mb, zb,
+                        &full[gr][s]);
+        }
+      }
+      // units and alphas of the segment's slots (the record's metadata), then the operand
+      const int nq = (int)(mb >> 4);
+      const int4* un = reinterpret_cast<const int4*>(x.meta + meta0);
+      const float4* al = reinterpret_cast<const float4*>(x.meta + meta0 + mb);
+      int4 u0 = make_int4(0, 0, 0, 0);
+      float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (lane < nq) {
+        u0 = __ldg(un + lane);
+        a0 = __ldg(al + lane);
+      }
+      if (i == 0) pdl_wait();   // z and max |z| come from the projection
+      if (c.first) {
+        tok = pr / p.k;
+        bs = scale_pow2(__ldg(x.msa + c.h * p.E + tb.e[c.a]) * __uint_as_float(__ldcg(p.zmax + c.h * p.T + tok)));
+        if (sub == 0 && lane < 16) {
+          runs[gr][run & 1].pair[lane] = pr;
+          runs[gr][run & 1].inv[lane] = 1.f / bs;
+        }
+      }
+      const uint32_t rwn = record(n);
+      const int prn = n.pos < hi && n.first ? pair_of(n) : pr;
+      uint8_t* az = st + (size_t)R * (bytes + zb);
+      const int r0 = ntk * sub / HG, r1 = ntk * (sub + 1) / HG;
+      const float* zh = p.z + (size_t)c.h * p.T * p.n_pad;
+      for (int q = lane; q - lane < nq; q += 32) {
+        if (q != lane && q < nq) {
+          u0 = __ldg(un + q);
+          a0 = __ldg(al + q);
+        }
+        for (int r = r0; r < r1; r += 4) {
+          float4 v[4];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int col = 2 * t + u;
-          const float iv = __shfl_sync(0xFFFFFFFFu, inv[q], 4 * col), f24 = 2097152.f * iv;   // 2^(24 - 3 - S)
-          float cc[G];
+          for (int w = 0; w < 4; ++w) {
+            const float* z = zh + (size_t)__shfl_sync(0xFFFFFFFFu, tok, min(r + w, r1 - 1)) * p.n_pad;
+            if (q < nq) v[w] = make_float4(z[u0.x], z[u0.y], z[u0.z], z[u0.w]);
+          }
 #pragma unroll
-          for (int gl = 0; gl < G; ++gl) cc[gl] = __shfl_sync(0xFFFFFFFFu, co[gl], 4 * col) * iv;
-          if (8 * q + col < ntk) {
-            const int pr = p.pair_list[tb.pst[c.a] + c.tt * kNT + 8 * q + col];
-            float* gp = p.gu + ((size_t)pr * 2 + c.h) * p.I_pad + c.rb * kRows + 4 * g;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float k0 = cc[j * G / 4];
-              red_add_v4(gp + 32 * j, fmaf(acc[2 * j][q][u], f24, -k0), fmaf(acc[2 * j][q][u + 2], f24, -k0),
-                         fmaf(acc[2 * j + 1][q][u], f24, -k0), fmaf(acc[2 * j + 1][q][u + 2], f24, -k0));
-            }
+          for (int w = 0; w < 4; ++w) {
+            const float b = __shfl_sync(0xFFFFFFFFu, bs, min(r + w, r1 - 1));
+            if (q < nq && r + w < r1)
+              *reinterpret_cast<float4*>(az + (size_t)q * kQS + (r + w) * 16) =
+                  make_float4(a0.x * v[w].x * b, a0.y * v[w].y * b, a0.z * v[w].z * b, a0.w * v[w].w * b);
           }
         }
       }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full[gr][s]);
+      run += c.sg + 1 == c.sg1;
+      c = n;
+      rw = rwn;
+      pr = prn;
     }
-    c = n;
-    n = n2;
+  } else {
+    // ---- consumers
+    regs_consumer();
+    pdl_wait();   // gate/up are cleared by the projection
+    const int gr = wid / R, wr = wid - gr * R, g = lane >> 2, t = lane & 3;
+    if (gr < KH) {
+      const uint8_t* ring = msm + (size_t)gr * 2 * x.gu_stage;
+      float acc[8][NTM][4];
+      float cs[G][NTM];
+      for (int i = 0;; ++i) {
+        const int s = i & 1;
+        ok &= mbar_wait(&full[gr][s], (uint32_t)(i >> 1) & 1u);
+        __syncwarp();
+        const GInfo& f = infos[gr][s];
+        const int flags = f.flags;
+        if (flags & 4) break;
+        if (flags & 1) {
+#pragma unroll
+          for (int q = 0; q < NTM; ++q) {
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+#pragma unroll
+              for (int w = 0; w < 4; ++w) acc[m][q][w] = 0.f;
+#pragma unroll
+            for (int gl = 0; gl < G; ++gl) cs[gl][q] = 0.f;
+          }
+        }
+        const int rb = f.rg * R + wr, ntk = f.ntk;
+        if (rb < p.NRB) {
+          const uint32_t bytes = f.rec.bytes, zb = G * f.rec.mb;
+          const uint8_t* st = ring + (size_t)s * x.gu_stage;
+          const uint32_t* sz = reinterpret_cast<const uint32_t*>(st + (size_t)R * bytes + (size_t)wr * zb);
+          const uint8_t* az = st + (size_t)R * (bytes + zb) + g * 16;
+          if (NTM == 1 || ntk <= 8) gu_segment<1, NTM, G>(f.rec, st + (size_t)wr * bytes, sz, az, lane, acc, cs);
+          else gu_segment<NTM, NTM, G>(f.rec, st + (size_t)wr * bytes, sz, az, lane, acc, cs);
+          if (flags & 2) {   // the part's end: its partial rows into gate/up
+            const GRun& rr = runs[gr][f.run];
+#pragma unroll
+            for (int q = 0; q < NTM; ++q) {
+              if (8 * q >= ntk) break;
+              float co[G];
+#pragma unroll
+              for (int gl = 0; gl < G; ++gl) {   // the token's correction, summed over the K lanes
+                float v = cs[gl][q];
+                v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+                v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
+                co[gl] = v;
+              }
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const int col = 2 * t + u;
+                const float iv = rr.inv[8 * q + col], f24 = 2097152.f * iv;   // 2^(24 - 3 - S)
+                float cc[G];
+#pragma unroll
+                for (int gl = 0; gl < G; ++gl) cc[gl] = __shfl_sync(0xFFFFFFFFu, co[gl], 4 * col) * iv;
+                if (8 * q + col < ntk) {
+                  float* gp = p.gu + ((size_t)rr.pair[8 * q + col] * 2 + f.h) * p.I_pad + rb * kRows + 4 * g;
+#pragma unroll
+                  for (int j = 0; j < 4; ++j) {
+                    const float k0 = cc[j * G / 4];
+                    red_add_v4(gp + 32 * j, fmaf(acc[2 * j][q][u], f24, -k0), fmaf(acc[2 * j][q][u + 2], f24, -k0),
+                               fmaf(acc[2 * j + 1][q][u], f24, -k0), fmaf(acc[2 * j + 1][q][u + 2], f24, -k0));
+                  }
+                }
+              }
+            }
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[gr][s]);
+      }
+    }
   }
   if (!ok && lane == 0) atomicCAS(p.status, 0, BITSMOE_ERR_TIMEOUT);
 }
+
+// Warps of a down block (512 threads of 128 registers, 384 of 168).
+__host__ __device__ constexpr int dn_warps(int ntm) { return ntm == 1 ? 16 : 12; }
 
 // ---------------------------------------------------------------------------
 // Down
@@ -641,70 +624,112 @@ struct DCur {
   int seq;               // unit tiles the warp has started (parity of the metadata slot)
 };
 
-// K-step ks (16 rows) of a row block: A registers of unit `u16 / 16` of the tile
+// The packed words of four K-steps (64 rows, half hf of a row block) of one unit (its 16-byte chunks at
+// `ln`, 512 bytes apart) that this lane needs, and from them the A registers of K-step 4 hf + k.
 template <int B>
-__device__ __forceinline__ void ul_a(const uint8_t* code, int ks, int u16, int t, uint32_t& lo, uint32_t& hi) {
-  auto word = [&](int chunk, int w) {
-    return *reinterpret_cast<const uint32_t*>(code + chunk * kChunkBytes + u16 + 4 * w);
-  };
-  const int sh = B == 1 ? t + 4 * (ks & 1) : B == 2 || B == 3 ? 2 * t : B == 8 ? 0 : 4 * (t & 1);
+struct UlWords {
+  uint32_t w[4];   // word of K-step k
+  uint32_t h[4];   // 3 and 6 bits: its high-plane word
+};
+template <int B>
+__device__ __forceinline__ void ul_load(const uint8_t* ln, int hf, int t, UlWords<B>& u) {
+  auto word = [&](int chunk, int w) { return *reinterpret_cast<const uint32_t*>(ln + chunk * kChunkBytes + 4 * w); };
+  if (B == 1) {          // a word = 32 rows: two K-steps
+    const uint2 v = *reinterpret_cast<const uint2*>(ln + 8 * hf);
+    u.w[0] = u.w[1] = v.x;
+    u.w[2] = u.w[3] = v.y;
+  } else if (B == 2 || B == 3) {   // a word = a K-step
+    const uint4 v = *reinterpret_cast<const uint4*>(ln + hf * kChunkBytes);
+    u.w[0] = v.x;
+    u.w[1] = v.y;
+    u.w[2] = v.z;
+    u.w[3] = v.w;
+    if (B == 3) {
+      const uint2 x = *reinterpret_cast<const uint2*>(ln + 2 * kChunkBytes + 8 * hf);
+      u.h[0] = u.h[1] = x.x;
+      u.h[2] = u.h[3] = x.y;
+    }
+  } else if (B == 4 || B == 6) {   // a word = 8 rows: lanes t < 2 the first of a K-step's two words
+#pragma unroll
+    for (int k = 0; k < 4; ++k) u.w[k] = word(2 * hf + (k >> 1), 2 * (k & 1) + (t >> 1));
+    if (B == 6) {
+      const uint4 x = *reinterpret_cast<const uint4*>(ln + (4 + hf) * kChunkBytes);
+      u.h[0] = x.x;
+      u.h[1] = x.y;
+      u.h[2] = x.z;
+      u.h[3] = x.w;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) u.w[k] = word(4 * hf + k, t);
+  }
+}
+template <int B>
+__device__ __forceinline__ void ul_a(const UlWords<B>& u, int k, int t, uint32_t& lo, uint32_t& hi) {
+  const int sh = B == 1 ? t + 4 * (k & 1) : B == 2 || B == 3 ? 2 * t : B == 8 ? 0 : 4 * (t & 1);
   const uint32_t mul = 1u << (code_pos<B>() - sh);
-  if (B == 1) a_regs<1>(word(0, ks >> 1), sh, mul, lo, hi);
-  else if (B == 2) a_regs<2>(word(ks >> 2, ks & 3), sh, mul, lo, hi);
-  else if (B == 4) a_regs<4>(word(ks >> 1, 2 * (ks & 1) + (t >> 1)), sh, mul, lo, hi);
-  else if (B == 8) a_regs<8>(word(ks, t), sh, mul, lo, hi);
-  else if (B == 3) a_regs2<2, 1>(word(ks >> 2, ks & 3), sh, mul, word(2, ks >> 1), t + 4 * (ks & 1), lo, hi);
-  else a_regs2<4, 2>(word(ks >> 1, 2 * (ks & 1) + (t >> 1)), sh, mul, word(4 + (ks >> 2), ks & 3), 2 * t, lo, hi);
+  if (B == 3) a_regs2<2, 1>(u.w[k], sh, mul, u.h[k], t + 4 * (k & 1), lo, hi);
+  else if (B == 6) a_regs2<4, 2>(u.w[k], sh, mul, u.h[k], 2 * t, lo, hi);
+  else a_regs<B>(u.w[k], sh, mul, lo, hi);
 }
 
-// One row block of a tile: out += scale (P 2^(24 - S) - zero sum(h)) per group
+// One row block of a tile: out += scale (P 2^(24 - S) - zero sum(h)) per group.  The hi and lo products of a
+// token group keep accumulators of their own, so that consecutive products do not wait for one another.
 template <int B, int NT, int NTM, int G>
 __device__ __forceinline__ void dn_rb(const uint8_t* code, const uint4* hf, int hstride, const float4* hz, int zstride,
                                       const uint32_t* sz, int lane, float (&out)[2][NTM][4]) {
   constexpr float fP = 1.f / (float)(1 << code_pos<B>());   // the codes' position
+  constexpr int KS = 8 / G;                                  // K-steps of a group
   const int g = lane >> 2, t = lane & 3;
+  float P[2][NT][4], Q[2][NT][4];
 #pragma unroll
-  for (int gl = 0; gl < G; ++gl) {
-    float P[2][NT][4];
+  for (int half = 0; half < 2; ++half) {
+    UlWords<B> w[4];
 #pragma unroll
-    for (int m = 0; m < 2; ++m)
+    for (int u = 0; u < 4; ++u) ul_load<B>(code + 16 * (g + 8 * u), half, t, w[u]);
 #pragma unroll
-      for (int n = 0; n < NT; ++n)
+    for (int k = 0; k < 4; ++k) {
+      const int ks = 4 * half + k, gl = ks / KS;
+      if (ks % KS == 0) {
 #pragma unroll
-        for (int w = 0; w < 4; ++w) P[m][n][w] = 0.f;
+        for (int m = 0; m < 2; ++m)
 #pragma unroll
-    for (int k = 0; k < 8 / G; ++k) {
-      const int ks = gl * (8 / G) + k;
+          for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) P[m][n][q] = Q[m][n][q] = 0.f;
+      }
       uint32_t lo[4], hi[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) ul_a<B>(code, ks, 16 * (g + 8 * u), t, lo[u], hi[u]);
+      for (int u = 0; u < 4; ++u) ul_a<B>(w[u], k, t, lo[u], hi[u]);
 #pragma unroll
       for (int n = 0; n < NT; ++n) {
         const uint4 b = hf[n * hstride + ks * 32 + lane];
         mma_16816(P[0][n], lo[0], lo[1], hi[0], hi[1], b.x, b.y);
         mma_16816(P[1][n], lo[2], lo[3], hi[2], hi[3], b.x, b.y);
-        mma_16816(P[0][n], lo[0], lo[1], hi[0], hi[1], b.z, b.w);
-        mma_16816(P[1][n], lo[2], lo[3], hi[2], hi[3], b.z, b.w);
+        mma_16816(Q[0][n], lo[0], lo[1], hi[0], hi[1], b.z, b.w);
+        mma_16816(Q[1][n], lo[2], lo[3], hi[2], hi[3], b.z, b.w);
       }
-    }
-    float sc[4], zp[4];
+      if (ks % KS == KS - 1) {
+        float sc[4], zp[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint32_t w = sz[gl * 32 + g + 8 * u];
-      sc[u] = f16lo(w);
-      zp[u] = f16hi(w);
-    }
+        for (int u = 0; u < 4; ++u) {
+          const uint32_t v = sz[gl * 32 + g + 8 * u];
+          sc[u] = f16lo(v);
+          zp[u] = f16hi(v);
+        }
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      float4 z = hz[gl * zstride + n * 4 + t];   // tokens 2 t and 2 t + 1: (sum, 2^(24 - S)) each
-      z.y *= fP;
-      z.w *= fP;
+        for (int n = 0; n < NT; ++n) {
+          float4 z = hz[gl * zstride + n * 4 + t];   // tokens 2 t and 2 t + 1: (sum, 2^(24 - S)) each
+          z.y *= fP;
+          z.w *= fP;
 #pragma unroll
-      for (int m = 0; m < 2; ++m) {
-        out[m][n][0] = fmaf(sc[2 * m], fmaf(P[m][n][0], z.y, -zp[2 * m] * z.x), out[m][n][0]);
-        out[m][n][1] = fmaf(sc[2 * m], fmaf(P[m][n][1], z.w, -zp[2 * m] * z.z), out[m][n][1]);
-        out[m][n][2] = fmaf(sc[2 * m + 1], fmaf(P[m][n][2], z.y, -zp[2 * m + 1] * z.x), out[m][n][2]);
-        out[m][n][3] = fmaf(sc[2 * m + 1], fmaf(P[m][n][3], z.w, -zp[2 * m + 1] * z.z), out[m][n][3]);
+          for (int m = 0; m < 2; ++m) {
+            out[m][n][0] = fmaf(sc[2 * m], fmaf(P[m][n][0] + Q[m][n][0], z.y, -zp[2 * m] * z.x), out[m][n][0]);
+            out[m][n][1] = fmaf(sc[2 * m], fmaf(P[m][n][1] + Q[m][n][1], z.w, -zp[2 * m] * z.z), out[m][n][1]);
+            out[m][n][2] = fmaf(sc[2 * m + 1], fmaf(P[m][n][2] + Q[m][n][2], z.y, -zp[2 * m + 1] * z.x), out[m][n][2]);
+            out[m][n][3] = fmaf(sc[2 * m + 1], fmaf(P[m][n][3] + Q[m][n][3], z.w, -zp[2 * m + 1] * z.z), out[m][n][3]);
+          }
+        }
       }
     }
   }
@@ -754,8 +779,8 @@ __host__ __device__ inline DPlan d_plan(int ntm, int G, int warps, const MArgs& 
 }
 
 template <int NTM, int G>
-__global__ void __launch_bounds__(kMW * 32, 1) k_dn_mma(Fwd p, MArgs x) {
-  constexpr int kW = kMW, kNT = 8 * NTM;
+__global__ void __launch_bounds__(dn_warps(NTM) * 32, 1) k_dn_mma(Fwd p, MArgs x) {
+  constexpr int kW = dn_warps(NTM), kNT = 8 * NTM;
   extern __shared__ __align__(128) uint8_t msm[];
   __shared__ uint64_t bars[kW][2];
   __shared__ int s_ok;
@@ -962,61 +987,51 @@ __global__ void __launch_bounds__(kMW * 32, 1) k_dn_mma(Fwd p, MArgs x) {
 
 namespace bmoe {
 
-// Largest staged gate/up segment of a layer: codes, unit indices, alphas and G scale/zero rows.
-uint32_t mma_gu_stage(const std::vector<CStage>& cst, int G, bool az) {
+// Largest staged segment of a gate/up group of R row blocks: codes and G scale/zero rows of each, and the
+// operand of ntm groups of 8 tokens.
+uint32_t mma_gu_stage(const std::vector<CStage>& cst, int G, int ntm, int R) {
   uint32_t m = 0;
   for (const CStage& r : cst)
-    if (r.bytes) m = std::max(m, r.bytes + ((az ? 0u : 2u) + (uint32_t)G) * r.mb);
+    if (r.bytes)
+      m = std::max(m, (uint32_t)R * (r.bytes + (uint32_t)G * r.mb) +
+                          (r.mb / 16u) * (uint32_t)(ntm == 1 ? az_quad<1>() : az_quad<2>()));
   return (m + 127u) & ~127u;
 }
 
 constexpr uint32_t kMaxSmem = 222u * 1024u;   // dynamic shared memory of a block (static parts beside it)
 
-static uint32_t gu_smem(const MArgs& x, int warps) { return (uint32_t)warps * 2u * x.gu_stage + mtiles_bytes(x.A_max); }
-// Warps of a gate/up block: as many as kMW whose rings fit, 0 when not even four do.
-static int gu_warps(const MArgs& x) {
-  int w = kMW;
-  while (w >= 4 && gu_smem(x, w) > kMaxSmem) --w;
-  return w >= 4 ? w : 0;
-}
+static uint32_t gu_smem(const MArgs& x) { return (uint32_t)x.gu_kh * 2u * x.gu_stage + mtiles_bytes(x.A_max); }
 
-// Row blocks a gate/up block works on at once: the split warps = R x parts with the fewest idle warps
-// (the larger R where equal: its warps share the operand's reads).
-static int gu_rows(int NRB, int warps) {
-  int best = 1;
+// The split of the consumer warps into KH groups of R row blocks: the fewest idle warps among the splits
+// whose rings fit (the larger R where equal: its warps share the gathered operand).
+static bool gu_split(int NRB, const uint32_t* stages, MArgs* x) {
   double bu = 0;
-  for (int R = std::min(NRB, warps); R >= 1; --R) {
-    const double u = (double)NRB / ((NRB + R - 1) / R * R) * (R * (warps / R)) / warps;
+  for (int R = std::min(NRB, kCW); R >= 1; --R) {
+    MArgs c = *x;
+    c.gu_r = R;
+    c.gu_kh = std::min(kMaxKH, kCW / R);
+    c.gu_stage = stages[R];
+    while (c.gu_kh > 1 && gu_smem(c) > kMaxSmem) --c.gu_kh;
+    if (!c.gu_stage || gu_smem(c) > kMaxSmem) continue;
+    const double u = (double)NRB / ((NRB + R - 1) / R * R) * (R * c.gu_kh) / kCW;
     if (u > bu + 1e-9) {
       bu = u;
-      best = R;
+      *x = c;
     }
   }
-  return best;
+  return bu > 0;
 }
 
-uint64_t mma_az_floats(const ImageHeader& hd, int T, int k, int* rt, int* nsp) {
-  const int P = T * k, A = std::min(hd.E, P);
-  *rt = (int)align_up((uint64_t)P + 7 * (uint64_t)A, 8);
-  *nsp = (int)align_up((uint64_t)hd.n + 7 * 32, 4);   // units and the padding of seven buckets (< 32 slots each)
-  return 2ull * (uint64_t)*rt * (uint64_t)*nsp;
-}
-
-bool mma_args(const ImageHeader& hd, int T, int k, bool az, uint32_t gu_stage, MArgs* x) {
+bool mma_args(const ImageHeader& hd, int T, int k, const uint32_t (&stages)[2][kCW + 1], MArgs* x) {
   std::memset(x, 0, sizeof(*x));
   const int G = std::max(1, kRows / hd.group);
   x->ntm = T <= 16 ? 1 : 2;
   x->A_max = std::min(hd.E, T * k);
-  x->use_az = az;
-  mma_az_floats(hd, T, k, &x->rt, &x->nsp);
-  x->gu_stage = gu_stage;
-  const int gw = gu_stage > 0 ? gu_warps(*x) : 0;
-  if (gw <= 0) return false;
-  x->gu_r = gu_rows(hd.NRB, gw);
+  if (!gu_split(hd.NRB, stages[x->ntm - 1], x)) return false;
   const int need = std::max(1, hd.group / kRows);   // whole groups a run of row blocks
   x->dn_rc = std::max(need, std::min(hd.NRB, 8) / need * need);
   x->dn_meta = 256u + 128u * (uint32_t)(x->dn_rc * kRows / hd.group);
-  return d_plan(x->ntm, G, kMW, *x).total <= kMaxSmem;
+  return d_plan(x->ntm, G, dn_warps(x->ntm), *x).total <= kMaxSmem;
 }
 
 template <class K>
@@ -1046,22 +1061,13 @@ static cudaError_t mm_launch(K kernel, int grid, int threads, uint32_t smem, con
 
 template <int NTM, int G>
 static cudaError_t mm_pair(bool down, const Fwd& p, const MArgs& x, int sms, cudaStream_t st, bool pdl) {
-  static uint32_t done[3] = {0, 0, 0};
-  if (down) return mm_launch(k_dn_mma<NTM, G>, sms, kMW * 32, d_plan(NTM, G, kMW, x).total, p, x, st, pdl, &done[0]);
-  const int w = gu_warps(x);
-  if constexpr (NTM == 1) {
-    if (!x.use_az) return mm_launch(k_gu_mma<1, G, false>, sms, w * 32, gu_smem(x, w), p, x, st, pdl, &done[1]);
-  }
-  return mm_launch(k_gu_mma<NTM, G, true>, sms, w * 32, gu_smem(x, w), p, x, st, pdl, &done[2]);
+  static uint32_t done[2] = {0, 0};
+  if (down) return mm_launch(k_dn_mma<NTM, G>, sms, dn_warps(NTM) * 32, d_plan(NTM, G, dn_warps(NTM), x).total, p, x, st, pdl, &done[0]);
+  return mm_launch(k_gu_mma<NTM, G>, sms, kGuThreads, gu_smem(x), p, x, st, pdl, &done[1]);
 }
 
 cudaError_t launch_expert_mma(bool down, const Fwd& p, const MArgs& x, int sms, cudaStream_t st, bool pdl) {
   const int G = std::max(1, kRows / p.group);
-  if (!down && x.use_az) {
-    static uint32_t done = 0;
-    const cudaError_t e = mm_launch(k_zgather, 4 * sms, kZgThreads, mtiles_bytes(x.A_max), p, x, st, pdl, &done);
-    if (e != cudaSuccess) return e;
-  }
   if (x.ntm == 2)
     return G == 1 ? mm_pair<2, 1>(down, p, x, sms, st, pdl)
                   : G == 2 ? mm_pair<2, 2>(down, p, x, sms, st, pdl) : mm_pair<2, 4>(down, p, x, sms, st, pdl);

@@ -58,7 +58,7 @@ struct bitsmoe_layer {
   alignas(64) uint8_t map_out[128];
   bool maps = false;
   bool mma = false;            // multi-token expert factors on tensor cores: no 16-bit units, metadata mirror built
-  uint32_t gu_stage[2] = {0, 0};   // largest staged gate/up segment of those kernels (z gathered in the kernel, az)
+  uint32_t gu_stage[2][kMmaWarps + 1] = {};   // largest staged gate/up segment of those kernels, per [token groups - 1][R]
   const float* d_msa = nullptr;   // [2][E] max |scale * alpha| of each gate/up (h, e) (inside d_stage's allocation)
   std::vector<uint8_t> meta;   // host copy of header + descriptors + segment table
   int seg_bytes = 0;           // largest gate/up item: code bytes inside one row block
@@ -1233,7 +1233,7 @@ inline bool decode_mode(const ImageHeader& hd, int T) {
 }
 
 struct WsLayout {
-  size_t status, pair_expert, pair_weight, expert_count, expert_start, pair_list, active, z, gu, s, zmax, az;
+  size_t status, pair_expert, pair_weight, expert_count, expert_start, pair_list, active, z, gu, s, zmax;
   size_t x_stage, logits_stage, y_stage;
   size_t sync;   // fused single-token kernel: grid-barrier counters
   size_t total;
@@ -1259,11 +1259,7 @@ WsLayout ws_layout(const ImageHeader& hd, int T, int k) {
   w.gu = take(P * 2 * hd.I_pad * 4);
   w.s = take((size_t)T * hd.n_pad * 4);
   // multi-token expert factors: max |z| per token (small batches: in the slack behind the status words)
-  // and, past the decode batch, their operand in unit-slot order
-  const bool batch = !decode_mode(hd, T);
-  int rt, nsp;
-  w.zmax = batch ? take(2 * (size_t)T * 4) : w.status + 64;
-  w.az = take(batch ? (size_t)mma_az_floats(hd, T, k, &rt, &nsp) * 4 : 0);
+  w.zmax = decode_mode(hd, T) ? w.status + 64 : take(2 * (size_t)T * 4);
   w.x_stage = take((size_t)T * hd.D * 2);
   w.logits_stage = take((size_t)T * hd.E * 4);
   w.y_stage = take((size_t)T * hd.D * 4);
@@ -1509,8 +1505,7 @@ int f2_choose(const bitsmoe_layer* L, int top_k, F2Args* fa) {
 // Whether the expert factors of a T-token call run on mma.sync (calls whose projection runs on the
 // tensor cores, which also takes max |z| per token).
 bool mma_fits(const bitsmoe_layer* L, int T, int top_k, MArgs* ma) {
-  const bool az = !decode_mode(L->hd(), T);
-  return L->mma && T >= 4 && mma_args(L->hd(), T, top_k, az, L->gu_stage[az], ma);
+  return L->mma && T >= 4 && mma_args(L->hd(), T, top_k, L->gu_stage, ma);
 }
 
 int forward_impl(const void* x, const float* logits, int T, int top_k, const bitsmoe_layer* L, float* y,
@@ -1595,7 +1590,6 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
     ma.meta = L->d_meta;
     ma.msa = L->d_msa;
     p.zmax = reinterpret_cast<uint32_t*>(wb + w.zmax);
-    ma.az = reinterpret_cast<float*>(wb + w.az);
   }
   if (T == 1 && !norm) {   // one token: the clustered kernel when the layer fits it
     F2Args f2;
@@ -1651,7 +1645,7 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
     if (tcp) {   // tensor-core projection; it also clears gate/up and s for the expert kernels
       const size_t zb = (size_t)(reinterpret_cast<uint8_t*>(p.s) - reinterpret_cast<uint8_t*>(p.gu)) +
                         (size_t)T * hd.n_pad * 4;
-      BM_CK(launch_gemm_tc(0, L->map_in, p, sms, st, pdl, p.gu, zb, p.zmax, mma));
+      BM_CK(launch_gemm_tc(0, L->map_in, p, sms, st, pdl, p.gu, zb, p.zmax));
     } else if ((rc = launch_gemv_bulk(true, p, sms, st, pdl))) {
       return rc;
     }
@@ -1835,7 +1829,8 @@ int upload(std::vector<uint8_t>&& img, int device, bitsmoe_layer** out) {
     bool no16 = true;
     for (int i = 0; i < 3 * h->E; ++i)
       for (int k = 0; k < xd[i].nbk; ++k) no16 &= xd[i].bk[k].bits < 16;
-    for (int az = 0; az < 2; ++az) L->gu_stage[az] = mma_gu_stage(cst, std::max(1, kRows / h->group), az != 0);
+    for (int ntm = 1; ntm <= 2; ++ntm)
+      for (int R = 1; R <= kMmaWarps; ++R) L->gu_stage[ntm - 1][R] = mma_gu_stage(cst, std::max(1, kRows / h->group), ntm, R);
     L->mma = no16 && L->maps && L->meta_ok;
   }
   const ImageHeader* hd = header_of(img.data());
@@ -2000,14 +1995,11 @@ int forward_launches(const bitsmoe_layer* L, int T, int top_k, bool allow_f2) {
   if (T == 0) return 0;
   F2Args f2;
   if (allow_f2 && T == 1 && f2_choose(L, top_k, &f2) >= 0) return 1;
-  const bool decode = decode_mode(hd, T);
   FusedArgs fa;
   const int s16 = (int)align_up(std::max(hd.seg_max_slots, 8), 64) + 8;
-  if (decode && L->meta_ok && fused_plan(hd, T, top_k, L->seg_bytes, L->ul_max_chunks, s16, L->num_sms, &fa)) return 1;
+  if (decode_mode(hd, T) && L->meta_ok && fused_plan(hd, T, top_k, L->seg_bytes, L->ul_max_chunks, s16, L->num_sms, &fa)) return 1;
   if (T <= kFusedMaxTokens && fused_fits(L, top_k)) return T;   // one fused forward per token
-  MArgs ma;
-  if (decode || !mma_fits(L, T, top_k, &ma)) return 5;   // router, projection, gate/up, down, output basis
-  return 6;                                              // and the gate/up operand's gather
+  return 5;   // router, projection, gate/up, down, output basis
 }
 }  // namespace
 

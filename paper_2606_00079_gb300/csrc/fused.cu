@@ -783,7 +783,6 @@ bool build_stage_tables(const uint8_t* img, std::vector<CStage>& cst, std::vecto
       if (it.nr == 0) continue;
       r.code0 = x.code_base + it.byte0;
       r.unit0 = x.unit_off + (uint64_t)it.slot0 * 4;
-      r.slot0 = it.slot0;
       r.alpha0 = x.alpha_off + (uint64_t)it.slot0 * 4;
       r.sz0 = x.sz_off + (uint64_t)it.slot0 * 4;
       r.rb_stride = (uint32_t)x.rb_stride;

@@ -57,8 +57,7 @@ struct GemmArgs {
   int accum;         // mode 1: y += (y holds the residual) instead of y =
   const uint16_t* x; // mode 0: [T][D] bf16 bits
   const float* s;    // mode 1: [T][n_pad]
-  float* z;          // mode 0: [2][T][n_pad], or with zt [2][n_pad][T] (token fastest)
-  int zt;
+  float* z;          // mode 0: [2][T][n_pad]
   uint32_t* zmax;    // mode 0: null, or [2][T] max_j |z_h[t][j]| as fp32 bits (zeroed before)
   float* y;          // mode 1: [T][D]
   float4* zero;      // null, or a buffer of later kernels to clear (after the PDL wait)
@@ -286,7 +285,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
         if (in) {
           if (g.mode == 0) {
             const int h = m >= g.n, j = m - h * g.n;
-            g.z[g.zt ? ((size_t)h * g.n_pad + j) * g.T + t : ((size_t)h * g.T + t) * g.n_pad + j] = sum;
+            g.z[((size_t)h * g.T + t) * g.n_pad + j] = sum;
           } else {
             float* yp = g.y + (size_t)t * g.D + m;
             *yp = g.accum ? *yp + sum : sum;
@@ -353,13 +352,13 @@ bool make_basis_map(void* map_out, const void* base, int rows, int cols_pad) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// mode 0: z = Phi_{g,u}^T x for all T tokens (zt: stored token-fastest).  The kernel before it on the stream is
+// mode 0: z = Phi_{g,u}^T x for all T tokens.  The kernel before it on the stream is
 // the router, which starts after all earlier work (it is launched without programmatic overlap), so the
 // projection reads x and clears `zero` while the router still runs and waits for it only before it
 // stores (qw3_skew, 8 tokens: the router's 8 us off the chain).  mode 1:
 // y = Phi_dn s, or y += Phi_dn s when p.accum.  Plain stores: nothing to clear.
 cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cudaStream_t st, bool pdl, void* zero,
-                           size_t zero_bytes, uint32_t* zmax, bool zt) {
+                           size_t zero_bytes, uint32_t* zmax) {
   static_assert(sizeof(CUtensorMap) == 128, "tensor map size");
   GemmArgs g;
   std::memset(&g, 0, sizeof(g));
@@ -376,7 +375,6 @@ cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cud
   g.x = p.x;
   g.s = p.s;
   g.z = p.z;
-  g.zt = zt;
   g.zmax = zmax;
   g.zero = static_cast<float4*>(zero);
   g.zero_n = zero_bytes / 16;
