@@ -54,8 +54,9 @@ struct MArgs {
   int ntm;                // groups of 8 tokens a warp's pass takes at most (1 or 2)
   int A_max;              // bound on the call's routed experts
   uint32_t gu_stage;      // bytes of a group's staged gate/up segment
+  int seg_stride;         // step through a run's segments (coprime to nseg)
   int gu_r, gu_kh;        // row blocks of a group of gate/up warps, groups of a block
-  int dn_rc;              // row blocks of a down run
+  int dn_rc, dn_st;       // row blocks of a down run, stages of a consumer's ring
   uint32_t dn_meta;       // bytes of a down tile's staged unit indices, alphas and scale/zero rows
   const CStage* cst;      // [2][E][nseg]
   const DStage* dst;      // [E][ul_max_tiles]

@@ -30,13 +30,14 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <numeric>
 
 #include "device.cuh"
 #include "tc.cuh"
 
 namespace {
 
-constexpr int kCW = kMmaWarps;      // consumer warps of the gate/up kernel
+constexpr int kCW = kMmaWarps;      // consumer warps of both kernels
 constexpr int kStagePiece = 4096;   // bytes of down codes a warp stages at a time
 
 // Token tiles of the call, and their share of a kernel's work: active expert a has cnt[a] tokens from
@@ -65,7 +66,7 @@ __device__ MTiles mtiles_at(uint8_t* sm, int A_max) {
 }
 // Relative time of a tile of nt tokens (measured: the decode of the codes is shared by a tile's groups of
 // 8 tokens, the operand and the products are not).
-__device__ __forceinline__ int tile_weight(int nt) { return 1 + 3 * ((nt + 7) >> 3); }
+__device__ __forceinline__ int tile_weight(int nt) { return 1 + ((nt + 7) >> 3); }
 
 // Whole block; the routing is published.  per_tile(e): units of a token tile of expert e.
 template <class F>
@@ -123,7 +124,8 @@ __device__ __forceinline__ int find_le(const int* base, int n, int v) {
 }
 // First unit of block b of nb.
 __device__ int cut_unit(const MTiles& t, int NT, int b, int nb) {
-  const int W = t.wb[t.na], x = (int)((long long)W * b / nb);
+  const int W = t.wb[t.na], wq = W / nb;
+  const int x = wq * b + (W - wq * nb) * b / nb;   // W b / nb in 32 bits
   if (b >= nb || x >= W) return t.ub[t.na];
   const int a = find_le(t.wb, t.na, x);   // the last expert that starts at or before: one with units
   const int c = t.cnt[a], f = c / NT, tiles = f + (c > f * NT), m = (t.ub[a + 1] - t.ub[a]) / tiles;
@@ -188,22 +190,24 @@ __device__ __forceinline__ void a_regs2(uint32_t w, int sh, uint32_t mul, uint32
 // ---------------------------------------------------------------------------
 // Gate/up
 // ---------------------------------------------------------------------------
-// Units in (token tile, projection, group of R row blocks, segment) order.  A block takes a contiguous run
-// of units.  Its 12 consumer warps form KH groups of R: the warps of a group work on the same segment, one
+// Units in (token tile, projection, group of R row blocks, segment) order, the segments of a run taken with a
+// stride: they hold equal bytes, so a segment of 1-bit units has four times the slots (and work) of one of
+// 4-bit units, and a stride spreads them over the blocks and groups (in order, the blocks of the 8-token call
+// ended between 21 and 33 us).  A block takes a contiguous run of units.  Its 12 consumer warps form KH groups of R: the warps of a group work on the same segment, one
 // row block each, and the groups take parts of each run of segments.  4 / KH helper warps a group fill its
 // two-stage ring: bulk copies of the R row blocks' codes and scale/zero rows, and the operand alpha z 2^S of
 // the segment's slots, gathered from z once for the group (the consumers, at three warps a scheduler, cannot
 // hide a global load: gathering in them, or reading a gathered copy from memory, left long-scoreboard stalls
 // of 3 issue slots an instruction).  The consumers decode, multiply and add their partial rows into gate/up.
-constexpr int kHW = 4;                       // helper warps
-constexpr int kGuThreads = (kCW + kHW) * 32;
+constexpr int kHW = 4;                       // helper warps of both kernels
+constexpr int kMmThreads = (kCW + kHW) * 32;
 constexpr int kMaxKH = 4;
 
 struct GCur {
   int pos;               // unit at which the current (tile, projection, row group) run starts (>= hi: the end)
   int end;               // its end (inside the block's units)
   int a, tt, h, rg;      // expert index and token tile, projection, group of row blocks
-  int sg, sg1;           // segment, end of the group's part
+  int i, i1;             // index of the segment in the run's order, end of the block's part of the run
   int first;
 };
 
@@ -343,13 +347,8 @@ __device__ __forceinline__ void gu_segment(const CStage& r, const uint8_t* st, c
   }
 }
 
-// Registers of the consumer and helper warps: 3 x 128 x 144 + 128 x 80 = 65536, what the block is launched
-// with (512 x 128).
-__device__ __forceinline__ void regs_consumer() { asm volatile("setmaxnreg.inc.sync.aligned.u32 144;"); }
-__device__ __forceinline__ void regs_helper() { asm volatile("setmaxnreg.dec.sync.aligned.u32 80;"); }
-
 template <int NTM, int G>
-__global__ void __launch_bounds__(kGuThreads, 1) k_gu_mma(Fwd p, MArgs x) {
+__global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
   constexpr int kNT = 8 * NTM, kQS = az_quad<NTM>();
   extern __shared__ __align__(128) uint8_t msm[];
   __shared__ uint64_t full[kMaxKH][2], empty[kMaxKH][2];
@@ -382,7 +381,6 @@ __global__ void __launch_bounds__(kGuThreads, 1) k_gu_mma(Fwd p, MArgs x) {
 
   if (wid >= kCW) {
     // ---- helpers
-    regs_helper();
     const int hw = wid - kCW, gr = hw / HG, sub = hw - gr * HG;
     if (gr >= KH) {
       pdl_wait();
@@ -401,10 +399,9 @@ __global__ void __launch_bounds__(kGuThreads, 1) k_gu_mma(Fwd p, MArgs x) {
         c.rg = i / p.nseg;
         const int s0 = i - c.rg * p.nseg;
         c.end = min(hi, c.pos + p.nseg - s0);
-        const int len = c.end - c.pos;
-        c.sg = s0 + len * gr / KH;
-        c.sg1 = s0 + len * (gr + 1) / KH;
-        if (c.sg == c.sg1) continue;
+        c.i = s0 + (gr + tau + c.h) % KH;   // every KH-th segment; which group starts changes from run to run
+        c.i1 = s0 + c.end - c.pos;
+        if (c.i >= c.i1) continue;
         c.a = find_le(tb.ub, tb.na, c.pos);
         c.tt = (c.pos - tb.ub[c.a]) / M;
         c.first = 1;
@@ -413,32 +410,55 @@ __global__ void __launch_bounds__(kGuThreads, 1) k_gu_mma(Fwd p, MArgs x) {
     };
     auto advance = [&](GCur& c) {
       c.first = 0;
-      if (++c.sg < c.sg1) return;
+      if ((c.i += KH) < c.i1) return;
       c.pos = c.end;
       first_of(c);
     };
     // word `lane` of the cursor's staging record
     auto record = [&](const GCur& c) -> uint32_t {
       if (c.pos >= hi || lane >= (int)(sizeof(CStage) / 4)) return 0u;
-      return __ldg(reinterpret_cast<const uint32_t*>(x.cst + ((size_t)c.h * p.E + tb.e[c.a]) * p.nseg + c.sg) + lane);
+      return __ldg(reinterpret_cast<const uint32_t*>(x.cst + ((size_t)c.h * p.E + tb.e[c.a]) * p.nseg + c.i * x.seg_stride % p.nseg) + lane);
     };
     auto pair_of = [&](const GCur& c) {   // lane < 16: the pair of the tile's row `lane`
       const int ntk = min(kNT, tb.cnt[c.a] - c.tt * kNT);
       return p.pair_list[tb.pst[c.a] + c.tt * kNT + min(lane & 15, ntk - 1)];
     };
-    GCur c;
+    // Pipeline, so that no latency but the copies' own follows the release of a stage: the records are loaded
+    // two stages ahead, the units and alphas of a stage's first 128 slots one stage ahead, and their z (the
+    // first kRB rows) before the wait for the stage.
+    constexpr int kRB = 4 * NTM;
+    GCur c, n;
     c.pos = lo;
     first_of(c);
-    uint32_t rw = record(c);
-    int pr = c.pos < hi ? pair_of(c) : 0;
+    n = c;
+    uint32_t rw = record(c), rwn = 0;
+    int pr = 0, prn = 0;
+    if (c.pos < hi) {
+      pr = pair_of(c);
+      advance(n);
+      rwn = record(n);
+      prn = n.pos < hi && n.first ? pair_of(n) : pr;
+    }
+    auto units = [&](uint32_t r, int q, int4& u, float4& al) {   // slot quad q of the segment of record r
+      const uint32_t mb = __shfl_sync(0xFFFFFFFFu, r, 11), m0 = __shfl_sync(0xFFFFFFFFu, r, 18);
+      u = make_int4(0, 0, 0, 0);
+      al = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (q < (int)(mb >> 4)) {
+        u = __ldg(reinterpret_cast<const int4*>(x.meta + m0) + q);
+        al = __ldg(reinterpret_cast<const float4*>(x.meta + m0 + mb) + q);
+      }
+    };
+    int4 uc, un;
+    float4 ac, an;
+    units(rw, lane, uc, ac);
     int tok = 0, run = 0;
     float bs = 1.f;
     for (int i = 0;; ++i) {
       const int s = i & 1;
-      if (i >= 2) ok &= mbar_wait(&empty[gr][s], (uint32_t)((i >> 1) - 1) & 1u);
-      __syncwarp();
       GInfo& f = infos[gr][s];
       if (c.pos >= hi) {
+        if (i >= 2) ok &= mbar_wait(&empty[gr][s], (uint32_t)((i >> 1) - 1) & 1u);
+        __syncwarp();
         if (lane == 0) {
           if (sub == 0) {
             f.flags = 4;
@@ -449,20 +469,21 @@ __global__ void __launch_bounds__(kGuThreads, 1) k_gu_mma(Fwd p, MArgs x) {
         if (i == 0) pdl_wait();
         break;
       }
-      GCur n = c;
-      advance(n);
       const int ntk = min(kNT, tb.cnt[c.a] - c.tt * kNT);
-      const uint32_t bytes = __shfl_sync(0xFFFFFFFFu, rw, 10), mb = __shfl_sync(0xFFFFFFFFu, rw, 11);
-      const uint32_t meta0 = __shfl_sync(0xFFFFFFFFu, rw, 18), zb = G * mb;
+      const int r0 = ntk * sub / HG, r1 = ntk * (sub + 1) / HG;   // this helper's rows
+      const uint32_t bytes = __shfl_sync(0xFFFFFFFFu, rw, 10), mb = __shfl_sync(0xFFFFFFFFu, rw, 11), zb = G * mb;
+      const int nq = (int)(mb >> 4);
       uint8_t* st = ring + (size_t)s * x.gu_stage;
-      if (sub == 0) {   // the description, and the copies: lane r < R codes, lane 16 + r scale/zero rows of row block r
+      uint8_t* az = st + (size_t)R * (bytes + zb);
+      const float* zh = p.z + (size_t)c.h * p.T * p.n_pad;
+      auto copies = [&]() {   // the description, and lane r < R: codes, lane 16 + r: scale/zero rows of row block r
         const uint64_t code0 =
             (uint64_t)__shfl_sync(0xFFFFFFFFu, rw, 0) | ((uint64_t)__shfl_sync(0xFFFFFFFFu, rw, 1) << 32);
-        const uint32_t rbs = __shfl_sync(0xFFFFFFFFu, rw, 8);
+        const uint32_t rbs = __shfl_sync(0xFFFFFFFFu, rw, 8), meta0 = __shfl_sync(0xFFFFFFFFu, rw, 18);
         if (lane < (int)(sizeof(CStage) / 4)) reinterpret_cast<uint32_t*>(&f.rec)[lane] = rw;
         const int nrb = min(R, p.NRB - c.rg * R);
         if (lane == 0) {
-          f.flags = (c.first ? 1 : 0) | (c.sg + 1 == c.sg1 ? 2 : 0);
+          f.flags = (c.first ? 1 : 0) | (c.i + KH >= c.i1 ? 2 : 0);
           f.h = c.h;
           f.rg = c.rg;
           f.ntk = ntk;
@@ -477,62 +498,73 @@ __global__ void __launch_bounds__(kGuThreads, 1) k_gu_mma(Fwd p, MArgs x) {
           else bulk_g2s(st + (size_t)R * bytes + (size_t)r * zb, x.meta + meta0 + (size_t)rb * (2u + G) * mb + 2u * mb, zb,
                         &full[gr][s]);
         }
+      };
+      if (i == 0) {   // the first stage's copies before the wait for the projection
+        if (sub == 0) copies();
+        pdl_wait();   // z and max |z|
       }
-      // units and alphas of the segment's slots (the record's metadata), then the operand
-      const int nq = (int)(mb >> 4);
-      const int4* un = reinterpret_cast<const int4*>(x.meta + meta0);
-      const float4* al = reinterpret_cast<const float4*>(x.meta + meta0 + mb);
-      int4 u0 = make_int4(0, 0, 0, 0);
-      float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (lane < nq) {
-        u0 = __ldg(un + lane);
-        a0 = __ldg(al + lane);
-      }
-      if (i == 0) pdl_wait();   // z and max |z| come from the projection
       if (c.first) {
         tok = pr / p.k;
         bs = scale_pow2(__ldg(x.msa + c.h * p.E + tb.e[c.a]) * __uint_as_float(__ldcg(p.zmax + c.h * p.T + tok)));
-        if (sub == 0 && lane < 16) {
-          runs[gr][run & 1].pair[lane] = pr;
-          runs[gr][run & 1].inv[lane] = 1.f / bs;
-        }
       }
-      const uint32_t rwn = record(n);
-      const int prn = n.pos < hi && n.first ? pair_of(n) : pr;
-      uint8_t* az = st + (size_t)R * (bytes + zb);
-      const int r0 = ntk * sub / HG, r1 = ntk * (sub + 1) / HG;
-      const float* zh = p.z + (size_t)c.h * p.T * p.n_pad;
-      for (int q = lane; q - lane < nq; q += 32) {
-        if (q != lane && q < nq) {
-          u0 = __ldg(un + q);
-          a0 = __ldg(al + q);
+      float4 v[kRB];
+      auto gather = [&](int r, const int4& u, bool live) {   // rows r .. r + kRB - 1 of one slot quad
+#pragma unroll
+        for (int w = 0; w < kRB; ++w) {
+          const float* z = zh + (size_t)__shfl_sync(0xFFFFFFFFu, tok, max(0, min(r + w, r1 - 1))) * p.n_pad;
+          if (live && r + w < r1) v[w] = make_float4(z[u.x], z[u.y], z[u.z], z[u.w]);
         }
-        for (int r = r0; r < r1; r += 4) {
-          float4 v[4];
+      };
+      auto put = [&](int r, int q, const float4& al) {
 #pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            const float* z = zh + (size_t)__shfl_sync(0xFFFFFFFFu, tok, min(r + w, r1 - 1)) * p.n_pad;
-            if (q < nq) v[w] = make_float4(z[u0.x], z[u0.y], z[u0.z], z[u0.w]);
-          }
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            const float b = __shfl_sync(0xFFFFFFFFu, bs, min(r + w, r1 - 1));
-            if (q < nq && r + w < r1)
-              *reinterpret_cast<float4*>(az + (size_t)q * kQS + (r + w) * 16) =
-                  make_float4(a0.x * v[w].x * b, a0.y * v[w].y * b, a0.z * v[w].z * b, a0.w * v[w].w * b);
-          }
+        for (int w = 0; w < kRB; ++w) {
+          const float b = __shfl_sync(0xFFFFFFFFu, bs, max(0, min(r + w, r1 - 1)));
+          if (q < nq && r + w < r1)
+            *reinterpret_cast<float4*>(az + (size_t)q * kQS + (r + w) * 16) =
+                make_float4(al.x * v[w].x * b, al.y * v[w].y * b, al.z * v[w].z * b, al.w * v[w].w * b);
+        }
+      };
+      gather(r0, uc, lane < nq);
+      units(rwn, lane, un, an);   // of the next stage
+      GCur n2 = n;
+      if (n.pos < hi) advance(n2);
+      const uint32_t rwn2 = record(n2);
+      const int prn2 = n2.pos < hi && n2.first ? pair_of(n2) : prn;
+      if (i >= 2) ok &= mbar_wait(&empty[gr][s], (uint32_t)((i >> 1) - 1) & 1u);
+      __syncwarp();
+      if (i > 0 && sub == 0) copies();
+      if (c.first && sub == 0 && lane < 16) {
+        runs[gr][run & 1].pair[lane] = pr;
+        runs[gr][run & 1].inv[lane] = 1.f / bs;
+      }
+      put(r0, lane, ac);
+      for (int r = r0 + kRB; r < r1; r += kRB) {
+        gather(r, uc, lane < nq);
+        put(r, lane, ac);
+      }
+      for (int q = 32; q < nq; q += 32) {   // more than 128 slots
+        int4 u;
+        float4 al;
+        units(rw, q + lane, u, al);
+        for (int r = r0; r < r1; r += kRB) {
+          gather(r, u, q + lane < nq);
+          put(r, q + lane, al);
         }
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&full[gr][s]);
-      run += c.sg + 1 == c.sg1;
+      run += c.i + KH >= c.i1;
       c = n;
+      n = n2;
       rw = rwn;
+      rwn = rwn2;
       pr = prn;
+      prn = prn2;
+      uc = un;
+      ac = an;
     }
   } else {
     // ---- consumers
-    regs_consumer();
     pdl_wait();   // gate/up are cleared by the projection
     const int gr = wid / R, wr = wid - gr * R, g = lane >> 2, t = lane & 3;
     if (gr < KH) {
@@ -606,22 +638,25 @@ __global__ void __launch_bounds__(kGuThreads, 1) k_gu_mma(Fwd p, MArgs x) {
   if (!ok && lane == 0) atomicCAS(p.status, 0, BITSMOE_ERR_TIMEOUT);
 }
 
-// Warps of a down block (512 threads of 128 registers, 384 of 168).
-__host__ __device__ constexpr int dn_warps(int ntm) { return ntm == 1 ? 16 : 12; }
-
 // ---------------------------------------------------------------------------
 // Down
 // ---------------------------------------------------------------------------
-// Unit-lane tiles (32 units): a warp item = (token tile, run of row blocks, unit tile).  The items of a
-// block are consecutive; for each (token tile, run) among them the block forms h = SiLU(gate) up once, as
-// B fragments in shared memory, and its warps take the unit tiles, whose codes they stream in pieces of
-// at most kStagePiece bytes through their own two-stage ring.
+// Unit-lane tiles (32 units): an item = (token tile, run of row blocks, unit tile); a segment = the items of
+// one (token tile, run).  A block takes consecutive items and its consumer warps every kCW-th of them,
+// whatever their segment; they stream their tiles' codes in pieces of at most kStagePiece bytes through their
+// own rings of three stages (with two, a piece's copy took longer than the work on the other: 254 us at
+// 1024 tokens with the tensor pipe 34% busy).  Four helper warps form h = SiLU(gate) up of each segment, as B fragments in one of
+// two shared-memory slots, while the consumers work on the segment before (formed by all warps between two
+// block barriers, h took 3.6 us of latency a segment, and a block whose 12 items lay in two segments ran twice
+// as long: the 8-token call's blocks ended between 44 and 55 us).
 struct DCur {
-  int pos, end;          // segment of the block's range: [pos, end) of the flat items, one (tile, run)
-  int tau, a, tt, rc;    // its token tile (expert a's tile tt) and run of row blocks
+  int p;                 // flat item (>= hi: the end)
+  int pos, end;          // its segment: items [pos, end) of the block's range
+  int ord;               // the segment's number in the block
+  int a, tt, rc;         // expert index, token tile, run of row blocks
   int tile0;             // unit tile of item `pos`
-  int tile, rb, nrb;     // the warp's unit tile, row block and row blocks of the piece
-  int seq;               // unit tiles the warp has started (parity of the metadata slot)
+  int rb;                // row block of the run
+  int ms;                // the tile's metadata slot
 };
 
 // The packed words of four K-steps (64 rows, half hf of a row block) of one unit (its 16-byte chunks at
@@ -757,49 +792,69 @@ __device__ __forceinline__ void dn_piece(int b, int nrb, const uint8_t* code, co
   }
 }
 
+constexpr int kDnStages = 3;   // most stages of a consumer's ring
+
+// Rows of a segment's token tile.
+struct DRow {
+  int off;      // token * n_pad
+  float pw;     // gate weight
+};
+
 // Shared-memory plan of k_dn_mma.
 struct DPlan {
-  uint32_t ring, meta, hf, hz, tabs, total;
+  uint32_t ring, meta, hf, hz, rows, tabs, total;
+  uint32_t hfs, hzs;   // bytes of an h slot: fragments, sums
 };
-__host__ __device__ inline DPlan d_plan(int ntm, int G, int warps, const MArgs& x) {
+__host__ __device__ inline DPlan d_plan(int ntm, int G, const MArgs& x) {
   DPlan s;
   uint32_t o = 0;
   s.ring = o;
-  o += (uint32_t)warps * 2u * kStagePiece;
+  o += (uint32_t)(kCW * x.dn_st) * kStagePiece;
   s.meta = o;
-  o += (uint32_t)warps * 2u * x.dn_meta;
+  o += (uint32_t)(kCW * x.dn_st) * x.dn_meta;
+  s.hfs = (uint32_t)ntm * x.dn_rc * 8u * 32u * 16u;
   s.hf = o;
-  o += (uint32_t)ntm * x.dn_rc * 8u * 32u * 16u;
+  o += 2u * s.hfs;
+  s.hzs = (uint32_t)x.dn_rc * G * ntm * 8u * 8u;
   s.hz = o;
-  o += (uint32_t)x.dn_rc * G * ntm * 8u * 8u;
+  o += 2u * s.hzs;
+  s.rows = o;
+  o += 2u * 16u * (uint32_t)sizeof(DRow);
   s.tabs = o;
   o += mtiles_bytes(x.A_max);
   s.total = (o + 15u) & ~15u;
   return s;
 }
 
+// Registers of the down kernel's consumer and helper warps: 3 x 128 x 144 + 128 x 80 = 65536, what the block is launched
+// with (512 x 128).
+__device__ __forceinline__ void regs_consumer() { asm volatile("setmaxnreg.inc.sync.aligned.u32 144;"); }
+__device__ __forceinline__ void regs_helper() { asm volatile("setmaxnreg.dec.sync.aligned.u32 80;"); }
+
 template <int NTM, int G>
-__global__ void __launch_bounds__(dn_warps(NTM) * 32, 1) k_dn_mma(Fwd p, MArgs x) {
-  constexpr int kW = dn_warps(NTM), kNT = 8 * NTM;
+__global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
+  constexpr int kNT = 8 * NTM;
   extern __shared__ __align__(128) uint8_t msm[];
-  __shared__ uint64_t bars[kW][2];
+  __shared__ uint64_t bars[kCW][kDnStages], hfull[2], hempty[2];
+  __shared__ int tbits[kCW][kDnStages];
   __shared__ int s_ok;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3;
-  const DPlan L = d_plan(NTM, G, kW, x);
-  uint8_t* ring = msm + L.ring + (size_t)wid * 2 * kStagePiece;
-  uint8_t* meta = msm + L.meta + (size_t)wid * 2 * x.dn_meta;
-  uint4* hf = reinterpret_cast<uint4*>(msm + L.hf);       // [NTM][dn_rc][8 K-steps][32 lanes]
-  float2* hz = reinterpret_cast<float2*>(msm + L.hz);     // [dn_rc][G][kNT] (sum of h, 2^(24 - S))
+  const DPlan L = d_plan(NTM, G, x);
   MTiles tb = mtiles_at(msm + L.tabs, x.A_max);
   const int RC = x.dn_rc, nrc = (p.NRB + RC - 1) / RC;
   const ExpertDesc* dd = p.desc + 2 * p.E;
 
   pdl_trigger();
-  if (lane == 0) {
-    mbar_init(&bars[wid][0]);
-    mbar_init(&bars[wid][1]);
+  if (tid == 0) {
+    for (int w = 0; w < kCW; ++w)
+      for (int s = 0; s < kDnStages; ++s) mbar_init_n(&bars[w][s], 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init_n(&hfull[s], kHW);
+      mbar_init_n(&hempty[s], kCW);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_ok = wait_flag(p.route_flag);
   }
-  if (tid == 0) s_ok = wait_flag(p.route_flag);
   __syncthreads();
   if (!s_ok) {
     if (tid == 0) atomicCAS(p.status, 0, BITSMOE_ERR_TIMEOUT);
@@ -809,8 +864,9 @@ __global__ void __launch_bounds__(dn_warps(NTM) * 32, 1) k_dn_mma(Fwd p, MArgs x
   mtiles_build(p, x.A_max, kNT, tb, [&](int e) { return nrc * __ldg(&dd[e].ntiles); });
   const int lo = cut_unit(tb, kNT, (int)blockIdx.x, (int)gridDim.x);
   const int hi = cut_unit(tb, kNT, (int)blockIdx.x + 1, (int)gridDim.x);
+  bool ok = true;
 
-  // the segment that starts at flat item c.pos (< hi)
+  // the segment that starts at item c.pos (< hi)
   auto seg_at = [&](DCur& c) {
     c.a = find_le(tb.ub, tb.na, c.pos);   // the last expert that starts at or before: one with items
     const int nt = (tb.ub[c.a + 1] - tb.ub[c.a]) / (((tb.cnt[c.a] + kNT - 1) / kNT) * nrc);
@@ -820,110 +876,155 @@ __global__ void __launch_bounds__(dn_warps(NTM) * 32, 1) k_dn_mma(Fwd p, MArgs x
     c.rc = tr - c.tt * nrc;
     c.end = min(hi, c.pos + nt - c.tile0);
   };
-  auto piece_len = [&](int bits, int left) { return min(left, bits <= 1 ? 8 : bits <= 2 ? 4 : bits <= 4 ? 2 : 1); };
-  // the warp's first unit tile at or after the segment, skipping segments without one
-  auto first_tile = [&](DCur& c) {
-    for (;;) {
-      if (c.pos >= hi) return;
-      seg_at(c);
-      c.tile = c.tile0 + wid;
-      c.rb = 0;
-      if (c.tile < c.tile0 + (c.end - c.pos)) return;
-      c.pos = c.end;
-    }
-  };
-  // words of the unit tile's staging record (12 words: lane l holds word l)
-  auto record = [&](const DCur& c) -> uint32_t {
-    if (c.pos >= hi || lane >= (int)(sizeof(DStage) / 4)) return 0u;
-    return __ldg(reinterpret_cast<const uint32_t*>(x.dst + (size_t)tb.e[c.a] * p.ul_max_tiles + c.tile) + lane);
-  };
   auto run_nrb = [&](const DCur& c) { return min(RC, p.NRB - c.rc * RC); };
-  auto issue = [&](int s, DCur& c, uint32_t rw) {
-    const uint64_t code = (uint64_t)__shfl_sync(0xFFFFFFFFu, rw, 0) | ((uint64_t)__shfl_sync(0xFFFFFFFFu, rw, 1) << 32);
-    const uint32_t bits = __shfl_sync(0xFFFFFFFFu, rw, 9), mt = __shfl_sync(0xFFFFFFFFu, rw, 10);
-    c.nrb = piece_len((int)bits, run_nrb(c) - c.rb);
-    if (lane == 0) {
-      uint64_t* bar = &bars[wid][s];
-      const uint32_t bytes = (uint32_t)c.nrb * bits * kChunkBytes;
-      fence_proxy_async();   // the stage was last read by the generic proxy
-      uint32_t tx = bytes, szb = 0;
-      if (c.rb == 0) {   // the tile's units, alphas and its scale/zero rows of this run
-        const int g0 = c.rc * RC * kRows / p.group, g1 = min(p.NG, ((c.rc * RC + run_nrb(c)) * kRows + p.group - 1) / p.group);
-        szb = (uint32_t)(g1 - g0) * 128u;
-        tx += 256u + szb;
-        mbar_expect_tx(bar, tx);
-        uint8_t* md = meta + (size_t)(c.seq & 1) * x.dn_meta;
-        bulk_g2s(md, x.meta + mt, 256u, bar);
-        bulk_g2s(md + 256, x.meta + mt + 256u + (uint32_t)g0 * 128u, szb, bar);
-      } else {
-        mbar_expect_tx(bar, tx);
-      }
-      bulk_g2s(ring + (size_t)s * kStagePiece, p.img + code + (uint64_t)(c.rc * RC + c.rb) * bits * kChunkBytes, bytes, bar);
-    }
-  };
-  auto advance = [&](DCur& c) {   // the next piece
-    c.rb += c.nrb;
-    if (c.rb < run_nrb(c)) return;
-    c.rb = 0;
-    c.tile += kW;
-    ++c.seq;
-    if (c.tile < c.tile0 + (c.end - c.pos)) return;
-    c.pos = c.end;
-    first_tile(c);
-  };
 
-  DCur n;   // the piece being staged
-  n.pos = lo;
-  n.seq = 0;
-  n.nrb = 0;
-  first_tile(n);
-  uint32_t rn = record(n), rnn = 0;
-  int i = 0;        // pieces consumed
-  DCur c = n;       // the piece being consumed
-  uint32_t rcw = rn;
-  if (n.pos < hi) {
-    issue(0, n, rn);
-    c = n;
-    advance(n);
-    rn = record(n);
-  }
-  pdl_wait();   // gate/up come from the previous kernel
-  bool ok = true;
-  DCur sgm;
-  for (sgm.pos = lo; sgm.pos < hi; sgm.pos = sgm.end) {
-    seg_at(sgm);
-    __syncthreads();   // the previous segment's h has been read
-    const int nrb = run_nrb(sgm), ntk = min(kNT, tb.cnt[sgm.a] - sgm.tt * kNT);
-    const int pst = tb.pst[sgm.a] + sgm.tt * kNT;
-    const int ntc = (ntk + 7) & ~7;
-    for (int w = wid; w < ntc * nrb; w += kW) {   // a warp per (token, row block): 4 rows a lane
-      const int tk = w / nrb, rb = w - tk * nrb;
-      float4 h4 = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (tk < ntk) {
-        const int pr = p.pair_list[pst + tk];
-        const float* gp = p.gu + (size_t)pr * 2 * p.I_pad + (sgm.rc * RC + rb) * kRows + 4 * lane;
-        const float4 gv = __ldcg(reinterpret_cast<const float4*>(gp));
-        const float4 uv = __ldcg(reinterpret_cast<const float4*>(gp + p.I_pad));
-        h4.x = gv.x / (1.f + __expf(-gv.x)) * uv.x;
-        h4.y = gv.y / (1.f + __expf(-gv.y)) * uv.y;
-        h4.z = gv.z / (1.f + __expf(-gv.z)) * uv.z;
-        h4.w = gv.w / (1.f + __expf(-gv.w)) * uv.w;
+  if (wid >= kCW) {
+    // ---- helpers: h of one segment after the other
+    regs_helper();
+    pdl_wait();   // gate/up come from the previous kernel
+    const int hw = wid - kCW;
+    DCur c;
+    c.pos = lo;
+    for (int k = 0; c.pos < hi; ++k, c.pos = c.end) {
+      seg_at(c);
+      const int s = k & 1, nrb = run_nrb(c), ntk = min(kNT, tb.cnt[c.a] - c.tt * kNT), rb0 = c.rc * RC;
+      const int pr = p.pair_list[tb.pst[c.a] + c.tt * kNT + min(lane & 15, ntk - 1)];
+      const float pw = hw == 0 ? p.pair_weight[pr] : 0.f;
+      if (k >= 2) ok &= mbar_wait(&hempty[s], (uint32_t)((k >> 1) - 1) & 1u);
+      __syncwarp();
+      uint4* hf = reinterpret_cast<uint4*>(msm + L.hf + s * L.hfs);     // [NTM][RC][8 K-steps][32 lanes]
+      float2* hz = reinterpret_cast<float2*>(msm + L.hz + s * L.hzs);   // [RC][G][kNT] (sum of h, 2^(24 - S))
+      if (hw == 0 && lane < 16) {
+        DRow r;
+        r.off = pr / p.k * p.n_pad;
+        r.pw = pw;
+        reinterpret_cast<DRow*>(msm + L.rows)[s * 16 + lane] = r;
       }
-      const float am = warp_max(fmaxf(fmaxf(fabsf(h4.x), fabsf(h4.y)), fmaxf(fabsf(h4.z), fabsf(h4.w))));
-      float sum = (h4.x + h4.y) + (h4.z + h4.w);
+      // a warp per (token, row block), 4 rows a lane; four at a time (rows past the tile's tokens are left
+      // as they are: their columns of the products are not read)
+      constexpr int kB = 4;
+      for (int w0 = hw; w0 < ntk * nrb; w0 += kB * kHW) {
+        float4 gv[kB], uv[kB];
 #pragma unroll
-      for (int o = 16 / G; o; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-      const float sc = scale_pow2(am);
-      uint4 v;
-      split_pair(h4.x * sc, h4.z * sc, v.x, v.z);
-      split_pair(h4.y * sc, h4.w * sc, v.y, v.w);
-      hf[((size_t)(tk >> 3) * RC + rb) * 256 + (lane >> 2) * 32 + (tk & 7) * 4 + (lane & 3)] = v;
-      if ((lane & (32 / G - 1)) == 0) hz[((size_t)rb * G + lane / (32 / G)) * kNT + tk] = make_float2(sum, 16777216.f / sc);
+        for (int q = 0; q < kB; ++q) {
+          const int w = min(w0 + q * kHW, ntk * nrb - 1), tk = w / nrb, rb = w - tk * nrb;
+          const float* gp = p.gu + (size_t)__shfl_sync(0xFFFFFFFFu, pr, tk) * 2 * p.I_pad + (rb0 + rb) * kRows + 4 * lane;
+          gv[q] = __ldcg(reinterpret_cast<const float4*>(gp));
+          uv[q] = __ldcg(reinterpret_cast<const float4*>(gp + p.I_pad));
+        }
+#pragma unroll
+        for (int q = 0; q < kB; ++q) {
+          const int w = w0 + q * kHW;
+          if (w >= ntk * nrb) break;
+          const int tk = w / nrb, rb = w - tk * nrb;
+          float4 h4;
+          h4.x = gv[q].x / (1.f + __expf(-gv[q].x)) * uv[q].x;
+          h4.y = gv[q].y / (1.f + __expf(-gv[q].y)) * uv[q].y;
+          h4.z = gv[q].z / (1.f + __expf(-gv[q].z)) * uv[q].z;
+          h4.w = gv[q].w / (1.f + __expf(-gv[q].w)) * uv[q].w;
+          const float am = warp_max(fmaxf(fmaxf(fabsf(h4.x), fabsf(h4.y)), fmaxf(fabsf(h4.z), fabsf(h4.w))));
+          float sum = (h4.x + h4.y) + (h4.z + h4.w);
+#pragma unroll
+          for (int o = 16 / G; o; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+          const float sc = scale_pow2(am);
+          uint4 v;
+          split_pair(h4.x * sc, h4.z * sc, v.x, v.z);
+          split_pair(h4.y * sc, h4.w * sc, v.y, v.w);
+          hf[((size_t)(tk >> 3) * RC + rb) * 256 + (lane >> 2) * 32 + (tk & 7) * 4 + (lane & 3)] = v;
+          if ((lane & (32 / G - 1)) == 0)
+            hz[((size_t)rb * G + lane / (32 / G)) * kNT + tk] = make_float2(sum, 16777216.f / sc);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&hfull[s]);
     }
-    __syncthreads();
-    // this warp's unit tiles of the segment
-    const int tend = sgm.tile0 + (sgm.end - sgm.pos);
-    for (int tile = sgm.tile0 + wid; tile < tend; tile += kW) {
+  } else {
+    // ---- consumers
+    regs_consumer();
+    const int S = x.dn_st;
+    uint8_t* ring = msm + L.ring + (size_t)wid * S * kStagePiece;
+    uint8_t* meta = msm + L.meta + (size_t)wid * S * x.dn_meta;
+    auto piece_len = [&](int bits, int left) { return min(left, bits <= 1 ? 8 : bits <= 2 ? 4 : bits <= 4 ? 2 : 1); };
+    auto walk = [&](DCur& c) {   // to the segment of item c.p (the block's end: past its last segment)
+      while (c.pos < hi && c.p >= c.end) {
+        c.pos = c.end;
+        ++c.ord;
+        if (c.pos < hi) seg_at(c);
+      }
+    };
+    // word `lane` of the unit tile's staging record
+    auto record = [&](const DCur& c) -> uint32_t {
+      if (c.p >= hi || lane >= (int)(sizeof(DStage) / 4)) return 0u;
+      return __ldg(reinterpret_cast<const uint32_t*>(x.dst + (size_t)tb.e[c.a] * p.ul_max_tiles + c.tile0 + c.p - c.pos) +
+                   lane);
+    };
+    auto advance = [&](DCur& c, int nrb) {   // past a piece of nrb row blocks; true: to another tile
+      c.rb += nrb;
+      if (c.rb < run_nrb(c)) return false;
+      c.rb = 0;
+      c.p += kCW;
+      if (++c.ms == S) c.ms = 0;
+      walk(c);
+      return true;
+    };
+
+    DCur n;   // the piece to be staged next, S - 1 ahead of the one consumed
+    n.p = lo + wid;
+    n.pos = lo;
+    n.ord = n.ms = n.rb = 0;
+    if (lo < hi) seg_at(n);
+    walk(n);
+    DCur c = n;
+    uint32_t rn = record(n);
+    int ps = 0;   // its stage
+    auto issue = [&]() {
+      if (n.p >= hi) return;
+      const uint64_t code = (uint64_t)__shfl_sync(0xFFFFFFFFu, rn, 0) | ((uint64_t)__shfl_sync(0xFFFFFFFFu, rn, 1) << 32);
+      const uint32_t bits = __shfl_sync(0xFFFFFFFFu, rn, 9), mt = __shfl_sync(0xFFFFFFFFu, rn, 10);
+      const int nrb = piece_len((int)bits, run_nrb(n) - n.rb);
+      if (lane == 0) {
+        uint64_t* bar = &bars[wid][ps];
+        const uint32_t bytes = (uint32_t)nrb * bits * kChunkBytes;
+        fence_proxy_async();   // the stage was last read by the generic proxy
+        if (n.rb == 0) {   // the tile's units, alphas and its scale/zero rows of this run
+          const int g0 = n.rc * RC * kRows / p.group;
+          const int g1 = min(p.NG, ((n.rc * RC + run_nrb(n)) * kRows + p.group - 1) / p.group);
+          const uint32_t szb = (uint32_t)(g1 - g0) * 128u;
+          mbar_expect_tx(bar, bytes + 256u + szb);
+          uint8_t* md = meta + (size_t)n.ms * x.dn_meta;
+          tbits[wid][n.ms] = (int)bits;
+          bulk_g2s(md, x.meta + mt, 256u, bar);
+          bulk_g2s(md + 256, x.meta + mt + 256u + (uint32_t)g0 * 128u, szb, bar);
+        } else {
+          mbar_expect_tx(bar, bytes);
+        }
+        bulk_g2s(ring + (size_t)ps * kStagePiece, p.img + code + (uint64_t)(n.rc * RC + n.rb) * bits * kChunkBytes, bytes,
+                 bar);
+      }
+      if (++ps == S) ps = 0;
+      if (advance(n, nrb)) rn = record(n);
+    };
+    for (int k = 0; k < S - 1; ++k) issue();
+    pdl_wait();   // s is cleared, and h's inputs are written, by earlier kernels
+    int held = -1;   // the segment whose h the warp holds
+    auto hold = [&](int ord) {
+      while (held < ord) {
+        if (held >= 0) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&hempty[held & 1]);
+        }
+        ++held;
+        ok &= mbar_wait(&hfull[held & 1], (uint32_t)(held >> 1) & 1u);
+        __syncwarp();
+      }
+    };
+    int cs = 0;
+    uint32_t cph = 0;   // stage and phase of the piece being consumed
+    while (c.p < hi) {   // a unit tile
+      hold(c.ord);
+      const int hs = held & 1, nrb = run_nrb(c), ntk = min(kNT, tb.cnt[c.a] - c.tt * kNT);
+      const uint4* hf = reinterpret_cast<const uint4*>(msm + L.hf + hs * L.hfs);
+      const float4* hz4 = reinterpret_cast<const float4*>(msm + L.hz + hs * L.hzs);
       float out[2][NTM][4];
 #pragma unroll
       for (int m = 0; m < 2; ++m)
@@ -931,54 +1032,51 @@ __global__ void __launch_bounds__(dn_warps(NTM) * 32, 1) k_dn_mma(Fwd p, MArgs x
         for (int q = 0; q < NTM; ++q)
 #pragma unroll
           for (int w = 0; w < 4; ++w) out[m][q][w] = 0.f;
-      const int bits = (int)__shfl_sync(0xFFFFFFFFu, rcw, 9);
-      const uint8_t* md = meta + (size_t)(c.seq & 1) * x.dn_meta;
-      for (int rb = 0; rb < nrb; ++i) {
-        __syncwarp();   // the other stage has been read by every lane
-        const int np = c.nrb;
-        const DCur nc = n;
-        rnn = rn;
-        if (n.pos < hi) {
-          issue((i + 1) & 1, n, rn);
-          c = n;
-          advance(n);
-          rn = record(n);
-        } else {
-          c = nc;
-        }
-        ok &= mbar_wait(&bars[wid][i & 1], (uint32_t)(i >> 1) & 1u);
+      const uint8_t* md = meta + (size_t)c.ms * x.dn_meta;
+      int bits = 0;
+      for (int rb = 0; rb < nrb;) {
+        __syncwarp();   // the stage before has been read by every lane
+        issue();
+        ok &= mbar_wait(&bars[wid][cs], cph);
         __syncwarp();
-        const uint8_t* code = ring + (size_t)(i & 1) * kStagePiece;
+        if (rb == 0) bits = tbits[wid][c.ms];
+        const int np = piece_len(bits, nrb - rb);
+        const uint8_t* code = ring + (size_t)cs * kStagePiece;
         const uint32_t* szp = reinterpret_cast<const uint32_t*>(md + 256);
-        const float4* hz4 = reinterpret_cast<const float4*>(hz);
         if (NTM == 1 || ntk <= 8)
           dn_piece<1, NTM, G>(bits, np, code, hf, RC * 256, hz4, kNT / 2, szp, rb, p.group, lane, out);
         else
           dn_piece<NTM, NTM, G>(bits, np, code, hf, RC * 256, hz4, kNT / 2, szp, rb, p.group, lane, out);
         rb += np;
-        rcw = rnn;
+        if (++cs == S) {
+          cs = 0;
+          cph ^= 1u;
+        }
       }
       // s += g alpha out
       const int* un = reinterpret_cast<const int*>(md);
       const float* al = reinterpret_cast<const float*>(md + 128);
+      const DRow* rows = reinterpret_cast<const DRow*>(msm + L.rows) + hs * 16;
 #pragma unroll
       for (int q = 0; q < NTM; ++q) {
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           const int tk = 8 * q + 2 * t + u;
           if (tk >= ntk) continue;
-          const int pr = p.pair_list[pst + tk];
-          const float pw = p.pair_weight[pr];
-          float* sp = p.s + (size_t)(pr / p.k) * p.n_pad;
+          const DRow r = rows[tk];
+          float* sp = p.s + r.off;
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
             const float a = al[g + 8 * v];
-            if (a != 0.f) atomicAdd(sp + un[g + 8 * v], pw * a * out[v >> 1][q][u + 2 * (v & 1)]);
+            if (a != 0.f) atomicAdd(sp + un[g + 8 * v], r.pw * a * out[v >> 1][q][u + 2 * (v & 1)]);
           }
         }
       }
       __syncwarp();   // the tile's metadata slot may be refilled
+      advance(c, nrb);
     }
+    // the segments that are left (the cursor has walked to the block's end: ord = their number)
+    if (c.ord > 0) hold(c.ord - 1);
   }
   if (!ok && lane == 0) atomicCAS(p.status, 0, BITSMOE_ERR_TIMEOUT);
 }
@@ -998,7 +1096,7 @@ uint32_t mma_gu_stage(const std::vector<CStage>& cst, int G, int ntm, int R) {
   return (m + 127u) & ~127u;
 }
 
-constexpr uint32_t kMaxSmem = 222u * 1024u;   // dynamic shared memory of a block (static parts beside it)
+constexpr uint32_t kMaxSmem = 224u * 1024u;   // dynamic shared memory of a block (static parts beside it)
 
 static uint32_t gu_smem(const MArgs& x) { return (uint32_t)x.gu_kh * 2u * x.gu_stage + mtiles_bytes(x.A_max); }
 
@@ -1028,10 +1126,22 @@ bool mma_args(const ImageHeader& hd, int T, int k, const uint32_t (&stages)[2][k
   x->ntm = T <= 16 ? 1 : 2;
   x->A_max = std::min(hd.E, T * k);
   if (!gu_split(hd.NRB, stages[x->ntm - 1], x)) return false;
-  const int need = std::max(1, hd.group / kRows);   // whole groups a run of row blocks
-  x->dn_rc = std::max(need, std::min(hd.NRB, 8) / need * need);
-  x->dn_meta = 256u + 128u * (uint32_t)(x->dn_rc * kRows / hd.group);
-  return d_plan(x->ntm, G, dn_warps(x->ntm), *x).total <= kMaxSmem;
+  x->seg_stride = std::max(1, (int)(0.382 * hd.nseg + 0.5));
+  while (std::gcd(x->seg_stride, hd.nseg) != 1) ++x->seg_stride;
+  // A down run: whole groups; at most 4 row blocks, so that the two h slots leave room for three stages a
+  // consumer and that a block's 12 consumers have several items each (one of 13 items of a whole expert's rows,
+  // 8 us each, doubled the 8-token call's time); up to 8 past 256 tokens, where the additions into s, one
+  // sector each, weigh more (1024 tokens: 334 us with runs of 3, 262 us with 6).
+  const int need = std::max(1, hd.group / kRows), most = T > 256 ? 8 : 4;
+  const int runs = std::max((hd.NRB + most - 1) / most, T <= 16 ? 3 : T <= 256 ? 2 : 1), rows = (hd.NRB + runs - 1) / runs;
+  const int rc0 = std::max(need, (rows + need - 1) / need * need);
+  for (int pass = 0; pass < 2; ++pass)
+    for (x->dn_rc = rc0; x->dn_rc >= need; x->dn_rc -= need) {
+      x->dn_meta = 256u + 128u * (uint32_t)(x->dn_rc * kRows / hd.group);
+      for (x->dn_st = kDnStages; x->dn_st >= (pass || T > 256 ? 2 : 3); --x->dn_st)
+        if (d_plan(x->ntm, G, *x).total <= kMaxSmem) return true;
+    }
+  return false;
 }
 
 template <class K>
@@ -1062,8 +1172,8 @@ static cudaError_t mm_launch(K kernel, int grid, int threads, uint32_t smem, con
 template <int NTM, int G>
 static cudaError_t mm_pair(bool down, const Fwd& p, const MArgs& x, int sms, cudaStream_t st, bool pdl) {
   static uint32_t done[2] = {0, 0};
-  if (down) return mm_launch(k_dn_mma<NTM, G>, sms, dn_warps(NTM) * 32, d_plan(NTM, G, dn_warps(NTM), x).total, p, x, st, pdl, &done[0]);
-  return mm_launch(k_gu_mma<NTM, G>, sms, kGuThreads, gu_smem(x), p, x, st, pdl, &done[1]);
+  if (down) return mm_launch(k_dn_mma<NTM, G>, sms, kMmThreads, d_plan(NTM, G, x).total, p, x, st, pdl, &done[0]);
+  return mm_launch(k_gu_mma<NTM, G>, sms, kMmThreads, gu_smem(x), p, x, st, pdl, &done[1]);
 }
 
 cudaError_t launch_expert_mma(bool down, const Fwd& p, const MArgs& x, int sms, cudaStream_t st, bool pdl) {
