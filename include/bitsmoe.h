@@ -145,7 +145,8 @@ size_t bitsmoe_workspace_bytes(const bitsmoe_layer* layer, int T, int top_k);
  * kernel (1) when the layer's per-block shares of the bases and factors fit
  * in shared memory, and up to 4 tokens as one such kernel per token (T);
  * otherwise the forward is a chain of 5 kernels (routing, projection, gate/up,
- * down, output basis; see bitsmoe_forward_plan).
+ * down, output basis; see bitsmoe_forward_plan), 6 past 16 tokens on layers
+ * without 16-bit units (the spectral accumulator split for the output basis).
  * Returns a negative error code for invalid arguments. */
 int bitsmoe_forward_launches(const bitsmoe_layer* layer, int T, int top_k);
 

@@ -43,6 +43,7 @@ struct Fwd {
   float* z;         // [2][T][n_pad]
   float* gu;        // [P][2][I_pad]
   float* s;         // [T][n_pad]
+  uint16_t* sb;     // null, or [2][T][n_pad]: bf16 hi and lo of s for the output basis (past kSplitTokens tokens)
   uint32_t* zmax;   // null, or [2][T]: cleared by the router, then max |z_h[t][j]| (fp32 bits) by the projection
 };
 
@@ -208,6 +209,7 @@ bool fused_plan(const ImageHeader& hd, int T, int top_k, int seg_bytes, int ul_m
                 FusedArgs* f);
 // Prep kernel + fused kernel on `st` (grid = sms blocks).
 cudaError_t launch_fused(const Fwd& p, const FusedArgs& f, int sms, cudaStream_t st, bool pdl);
+constexpr int kSplitTokens = 64;
 // Tensor-core projections (gemm.cu): a TMA map of a bf16 basis [rows][cols_pad]
 // (128 bytes, written to map_out), and the launch of z += Phi^T x (mode 0) or
 // y += Phi_dn s (mode 1) for all T tokens of p (z, resp. y, zeroed before
@@ -374,113 +376,6 @@ __device__ __forceinline__ uint32_t order_key(float f) {
   if ((u & 0x7FFFFFFFu) > 0x7F800000u) return 0u;
   if (u == 0x80000000u) return 0x80000000u;   // -0 and +0 are equal logits: they tie
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-// ---------------------------------------------------------------------------
-// Routing of all T tokens by one block into shared memory (small batches):
-// keys[T*E] | pe[P] | pw[P] | cnt[E] | start[E+1] | act[E+1] | plist[P].
-// Same rule as k_router.  Contains __syncthreads (call from the whole block).
-// ---------------------------------------------------------------------------
-__host__ __device__ constexpr int route_words(int T, int E, int P) { return T * E + 3 * P + 3 * E + 3; }
-
-struct RouteView {
-  const int* pe;
-  const float* pw;
-  const int* cnt;
-  const int* start;
-  const int* act;
-  const int* plist;
-};
-
-__device__ RouteView route_block(const Fwd& p, uint32_t* sm) {
-  const int E = p.E, k = p.k, T = p.T, P = p.P, tid = threadIdx.x, nt = blockDim.x;
-  uint32_t* keys = sm;
-  int* pe = reinterpret_cast<int*>(keys + T * E);
-  float* pw = reinterpret_cast<float*>(pe + P);
-  int* cnt = reinterpret_cast<int*>(pw + P);
-  int* start = cnt + E;
-  int* act = start + E + 1;
-  int* plist = act + E + 1;
-  for (int i = tid; i < T * E; i += nt) keys[i] = order_key(p.logits[i]);
-  for (int i = tid; i < E; i += nt) cnt[i] = 0;
-  __syncthreads();
-  // rank of each logit in its token's row (ties to the lower index)
-  for (int i = tid; i < T * E; i += nt) {
-    const int t = i / E, e = i - t * E;
-    const uint32_t key = keys[i];
-    // the logit back from its key (the key map is a bijection on non-NaN floats)
-    const float logit = __uint_as_float((key & 0x80000000u) ? (key & 0x7FFFFFFFu) : ~key);
-    const uint32_t* row = keys + t * E;
-    int rank = 0;
-    if ((E & 3) == 0 && ((t * E) & 3) == 0) {
-      const uint4* r4 = reinterpret_cast<const uint4*>(row);
-#pragma unroll 4
-      for (int f4 = 0; f4 < (E >> 2); ++f4) {
-        const uint4 o = r4[f4];
-        const int f = f4 << 2;
-        rank += (o.x > key) | ((o.x == key) & (f < e));
-        rank += (o.y > key) | ((o.y == key) & (f + 1 < e));
-        rank += (o.z > key) | ((o.z == key) & (f + 2 < e));
-        rank += (o.w > key) | ((o.w == key) & (f + 3 < e));
-      }
-    } else {
-      for (int f = 0; f < E; ++f) {
-        const uint32_t o = row[f];
-        rank += (o > key) | ((o == key) & (f < e));
-      }
-    }
-    if (rank < k) {
-      pe[t * k + rank] = e;
-      pw[t * k + rank] = key ? logit : __int_as_float(0x7FC00000);   // key 0: NaN logit
-    }
-  }
-  __syncthreads();
-  for (int t = tid; t < T; t += nt) {
-    float* w = pw + t * k;
-    const float m = w[0];
-    float sum = 0.f;
-    for (int r = 0; r < k; ++r) sum += expf(w[r] - m);
-    const float inv = 1.f / sum;
-    for (int r = 0; r < k; ++r) w[r] = expf(w[r] - m) * inv;
-  }
-  for (int q = tid; q < P; q += nt) atomicAdd(&cnt[pe[q]], 1);
-  __syncthreads();
-  if (tid < 32) {   // exclusive scans of counts and of "routed" flags, one warp
-    const int lane = tid, per = (E + 31) >> 5, e0 = min(E, lane * per), e1 = min(E, e0 + per);
-    int c = 0, na = 0;
-    for (int e = e0; e < e1; ++e) {
-      c += cnt[e];
-      na += cnt[e] > 0;
-    }
-    int ci = c, ai = na;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int vc = __shfl_up_sync(0xFFFFFFFFu, ci, o), va = __shfl_up_sync(0xFFFFFFFFu, ai, o);
-      if (lane >= o) {
-        ci += vc;
-        ai += va;
-      }
-    }
-    int run = ci - c, ra = ai - na;
-    for (int e = e0; e < e1; ++e) {
-      start[e] = run;
-      run += cnt[e];
-      if (cnt[e] > 0) act[1 + ra++] = e;
-    }
-    if (lane == 31) {
-      start[E] = ci;
-      act[0] = ai;
-    }
-  }
-  __syncthreads();
-  for (int q = tid; q < P; q += nt) {   // stable order: pairs of one expert by increasing q
-    const int ex = pe[q];
-    int r = 0;
-    for (int q2 = 0; q2 < q; ++q2) r += pe[q2] == ex;
-    plist[start[ex] + r] = q;
-  }
-  __syncthreads();
-  return RouteView{pe, pw, cnt, start, act, plist};
 }
 
 template <int PB, int TB>

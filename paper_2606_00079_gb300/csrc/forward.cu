@@ -144,7 +144,8 @@ __global__ void __launch_bounds__(kThreads) k_norm_router(NormArgs a) {
     }
   }
   pdl_wait();
-  for (int t0 = 0; t0 < a.T; t0 += TB) {
+  const int tfirst = blockIdx.y * TB;
+  for (int t0 = tfirst; t0 < a.T; t0 += gridDim.y * TB) {
     const int tb = min(TB, a.T - t0);
     __syncthreads();
     float ss[TB];
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(kThreads) k_norm_router(NormArgs a) {
       for (int tt = 0; tt < TB; ++tt) acc[tt] = 0.f;
       for (int c0 = 0; c0 < nch; c0 += 256) {
         uint4 v[8];
-        if (row == row0 && c0 == 0 && t0 == 0) {
+        if (row == row0 && c0 == 0 && t0 == tfirst) {
 #pragma unroll
           for (int u = 0; u < 8; ++u) v[u] = pre[u];
         } else {
@@ -236,50 +237,18 @@ __global__ void __launch_bounds__(kThreads) k_norm_router(NormArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// Decode-mode router: first kernel of the chain.  It lets the projection
-// kernel launch at once, then routes while the memory system is still idle
-// (the logits load is not queued behind the basis streams) and publishes the
-// routing with a release flag that the gate/up and down kernels wait on.
+// K0: routing, the first kernel of the chain.  k largest logits per token (ties to the
+// lower expert index), gate weights = softmax over the selected k, then a stable
+// grouping of the (token, slot) pairs p = t * k + slot by expert.  It lets the
+// projection launch at once; a warp selects for a token (the k maxima one after
+// the other by redux, 0.2 us for top-8 of 128; ranking every logit against every
+// other took 2 us and, at 8 tokens, kept the projection waiting), a block for 32;
+// the last block to finish (a counter in the workspace, which it resets) groups all
+// pairs and publishes the routing with a release flag.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_route_publish(Fwd p) {
-  if (p.zmax)   // the projection takes the maxima, after this kernel
-    for (int i = threadIdx.x; i < 2 * p.T; i += blockDim.x) p.zmax[i] = 0u;
-  if (threadIdx.x == 0) {   // before the trigger: no later kernel may see the previous call's flag
-    p.status[0] = 0;
-    p.route_flag[0] = 0;
-    __threadfence();
-  }
-  __syncthreads();
-  pdl_trigger();
-  extern __shared__ uint32_t smem_rp[];
-  const RouteView rv = route_block(p, smem_rp);
-  for (int i = threadIdx.x; i < p.P; i += blockDim.x) {
-    p.pair_expert[i] = rv.pe[i];
-    p.pair_weight[i] = rv.pw[i];
-    p.pair_list[i] = rv.plist[i];
-  }
-  for (int i = threadIdx.x; i <= p.E; i += blockDim.x) {
-    if (i < p.E) p.expert_count[i] = rv.cnt[i];
-    p.expert_start[i] = rv.start[i];
-    p.active[i] = rv.act[i];
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    st_release(p.route_flag, 1);
-  }
-}
+constexpr int kRouteWarps = 32;
 
-// ---------------------------------------------------------------------------
-// K0: routing.  k largest logits per token (ties to the lower expert index),
-// gate weights = softmax over the selected k, then a stable grouping of the
-// (token, slot) pairs p = t * k + slot by expert.  Blocks select for tpb
-// tokens each; the last block to finish (a counter in the workspace, which it
-// resets) groups all pairs and publishes the routing with a release flag.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_router(Fwd p) {
-  if (p.zmax && blockIdx.x == 0)   // the projection takes the maxima, after this kernel
-    for (int i = threadIdx.x; i < 2 * p.T; i += blockDim.x) p.zmax[i] = 0u;
+__global__ void __launch_bounds__(kRouteWarps * 32) k_router(Fwd p) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {   // before the trigger: no later kernel may see the previous flag
     p.status[0] = 0;
     p.route_flag[0] = 0;
@@ -287,47 +256,63 @@ __global__ void __launch_bounds__(1024) k_router(Fwd p) {
   }
   __syncthreads();
   pdl_trigger();
-  // shared: keys [tpb][E] | pair expert [P] | count [E] | start [E+1]
+  if (p.zmax && blockIdx.x == 0)   // the projection takes the maxima, after this kernel
+    for (int i = threadIdx.x; i < 2 * p.T; i += blockDim.x) p.zmax[i] = 0u;
+  // shared: keys [32 warps][E], reused by the grouping
   extern __shared__ uint32_t keys[];
   __shared__ int last;
   const int E = p.E, k = p.k, T = p.T, P = p.P;
-  const int tid = threadIdx.x;
-  const int tpb = max(1, (int)blockDim.x / E);
-  {   // this block's tokens
-    const int tt = tid / E, e = tid - tt * E, t = blockIdx.x * tpb + tt;
-    const bool valid = tt < tpb && t < T;
-    float lg = 0.f;
-    if (valid) {
-      lg = p.logits[(size_t)t * E + e];
-      keys[tt * E + e] = order_key(lg);
-    }
-    __syncthreads();
-    if (valid) {
-      const uint32_t key = keys[tt * E + e];
-      const uint32_t* row = keys + tt * E;
-      int rank = 0;
-      for (int f = 0; f < E; ++f) {
-        const uint32_t o = row[f];
-        rank += (o > key) | ((o == key) & (f < e));
-      }
-      if (rank < k) {
-        p.pair_expert[t * k + rank] = e;
-        reinterpret_cast<float*>(keys)[tpb * E + tt * k + rank] = lg;   // logits of the selected, in rank order
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int t = blockIdx.x * kRouteWarps + warp;
+  if (t < T) {
+    uint32_t* row = keys + warp * E;   // order key + 1; 0 once selected
+    uint32_t b = 0;                    // this lane's largest (experts lane, lane + 32, ..) and its first expert
+    int be = 0;
+    for (int i = lane; i < E; i += 32) {
+      const uint32_t v = order_key(p.logits[(size_t)t * E + i]) + 1u;
+      row[i] = v;
+      if (v > b) {
+        b = v;
+        be = i;
       }
     }
-    __syncthreads();
-    for (int q = tid; q < tpb * k; q += blockDim.x) {   // softmax over the k selected of each token
-      const int t2 = blockIdx.x * tpb + q / k, r = q - (q / k) * k;
-      if (t2 >= T) continue;
-      const float* w = reinterpret_cast<const float*>(keys) + tpb * E + (q / k) * k;
-      const float m = w[0];
-      float sum = 0.f;
-      for (int r2 = 0; r2 < k; ++r2) sum += expf(w[r2] - m);
-      p.pair_weight[t2 * k + r] = expf(w[r] - m) * (1.f / sum);
+    float w = 0.f;   // lane r: the r-th selected logit
+    int e = 0;
+    for (int r = 0; r < k; ++r) {
+      const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, b);
+      const int sel = (int)__reduce_min_sync(0xFFFFFFFFu, b == m ? (uint32_t)be : 0xFFFFFFFFu);
+      if (lane == r) {
+        const uint32_t key = m - 1u;   // the logit back from its key (a bijection on non-NaN floats)
+        w = key ? __uint_as_float((key & 0x80000000u) ? (key & 0x7FFFFFFFu) : ~key) : __int_as_float(0x7FC00000);
+        e = sel;
+      }
+      if (lane == (sel & 31)) {   // its lane's next largest
+        row[sel] = 0;
+        b = 0;
+        for (int i = lane; i < E; i += 32) {
+          const uint32_t v = row[i];
+          if (v > b) {
+            b = v;
+            be = i;
+          }
+        }
+      }
+      __syncwarp();
+    }
+    const float m = __shfl_sync(0xFFFFFFFFu, w, 0), ev = expf(w - m);
+    float sum = 0.f;
+    for (int r = 0; r < k; ++r) sum += __shfl_sync(0xFFFFFFFFu, ev, r);
+    if (lane < k) {
+      p.pair_expert[t * k + lane] = e;
+      p.pair_weight[t * k + lane] = ev * (1.f / sum);
     }
   }
+  if (gridDim.x == 1) {
+    __threadfence_block();
+    last = 1;
+  }
   __syncthreads();
-  if (tid == 0) {
+  if (tid == 0 && gridDim.x > 1) {
     __threadfence();
     const int old = atomicAdd(p.status + 2, 1);
     last = old == (int)gridDim.x - 1;
@@ -339,7 +324,8 @@ __global__ void __launch_bounds__(1024) k_router(Fwd p) {
   // Grouping by counting: warp w takes the w-th contiguous part of the pairs, counts its pairs per
   // expert, and after a prefix over the warps places them in order (the rank inside a group of 32 by
   // match.any).  1024 tokens, top-8: 122 us with one pass over all pairs per expert, see the bench table.
-  const int warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+  const int part = (P + kRouteWarps * 32 - 1) / (kRouteWarps * 32) * 32;
+  const int nw = (P + part - 1) / part;                   // warps that have pairs
   uint16_t* s_pe = reinterpret_cast<uint16_t*>(keys);     // [P] reuse: all pairs' experts
   uint16_t* s_h = s_pe + ((P + 1) & ~1);                  // [nw][E] pairs of each warp and expert, then their offset
   int* s_cnt = reinterpret_cast<int*>(s_h + nw * ((E + 1) & ~1));
@@ -348,7 +334,7 @@ __global__ void __launch_bounds__(1024) k_router(Fwd p) {
   for (int q = tid; q < P; q += blockDim.x) s_pe[q] = (uint16_t)__ldcg(p.pair_expert + q);
   for (int i = tid; i < nw * hs; i += blockDim.x) s_h[i] = 0;
   __syncthreads();
-  const int part = (P + nw * 32 - 1) / (nw * 32) * 32, qb = warp * part, qe = min(P, qb + part);
+  const int qb = warp * part, qe = min(P, qb + part);
   for (int q0 = qb; q0 < qe; q0 += 32) {
     const int q = q0 + lane, e = q < qe ? s_pe[q] : E + lane;   // lanes past the end match no other
     const unsigned m = __match_any_sync(0xFFFFFFFFu, e);
@@ -1233,7 +1219,7 @@ inline bool decode_mode(const ImageHeader& hd, int T) {
 }
 
 struct WsLayout {
-  size_t status, pair_expert, pair_weight, expert_count, expert_start, pair_list, active, z, gu, s, zmax;
+  size_t status, pair_expert, pair_weight, expert_count, expert_start, pair_list, active, z, gu, s, zmax, sb;
   size_t x_stage, logits_stage, y_stage;
   size_t sync;   // fused single-token kernel: grid-barrier counters
   size_t total;
@@ -1260,6 +1246,7 @@ WsLayout ws_layout(const ImageHeader& hd, int T, int k) {
   w.s = take((size_t)T * hd.n_pad * 4);
   // multi-token expert factors: max |z| per token (small batches: in the slack behind the status words)
   w.zmax = decode_mode(hd, T) ? w.status + 64 : take(2 * (size_t)T * 4);
+  w.sb = take(!decode_mode(hd, T) && T > kSplitTokens ? 2 * (size_t)T * hd.n_pad * 2 : 0);
   w.x_stage = take((size_t)T * hd.D * 2);
   w.logits_stage = take((size_t)T * hd.E * 4);
   w.y_stage = take((size_t)T * hd.D * 4);
@@ -1380,6 +1367,16 @@ int launch_gemv_bulk(bool proj, const Fwd& p, int sms, cudaStream_t st, bool pdl
   return launch_gemv_bulk_tb<8>(proj, p, sms, st, pdl);
 }
 
+// Selection: 32 rows of keys; grouping: the pairs' experts and 32 warps' counts in 16 bits, counts and starts.
+int launch_router(const Fwd& p, cudaStream_t st) {
+  const size_t smem = std::max((size_t)kRouteWarps * p.E * 4, 2 * ((size_t)p.P + 2 + kRouteWarps * ((size_t)p.E + 1)) +
+                                                                  4 * (2 * (size_t)p.E + 2));
+  if (smem > 200 * 1024) return BITSMOE_ERR_SHAPE;
+  int rc;
+  if ((rc = set_smem(k_router, smem))) return rc;
+  return launch(k_router, dim3((p.T + kRouteWarps - 1) / kRouteWarps), dim3(kRouteWarps * 32), smem, st, false, p);
+}
+
 // parts: 1 the gate/up kernel, 2 the down kernel, 3 both
 template <int G, int TB>
 int launch_k2k3_dec(const Fwd& p, int A_max, int sms, cudaStream_t st, bool pdl,
@@ -1434,7 +1431,9 @@ int launch_norm_router_tb(const NormArgs& a, int sms, cudaStream_t st) {
   int rc;
   if ((rc = set_smem(k_norm_router<TB>, smem))) return rc;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(std::max(1, std::min((a.E + kWarps - 1) / kWarps, sms)));
+  // router rows x token tiles: the token tiles side by side (one after another in 16 blocks, 32 tokens of the
+  // Qwen3-shaped router took about 90 us)
+  cfg.gridDim = dim3(std::max(1, std::min((a.E + kWarps - 1) / kWarps, sms)), std::min((a.T + TB - 1) / TB, 4096));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -1449,9 +1448,8 @@ int launch_norm_router_tb(const NormArgs& a, int sms, cudaStream_t st) {
 
 int launch_norm_router(const NormArgs& a, int sms, cudaStream_t st) {
   if (a.T <= 1) return launch_norm_router_tb<1>(a, sms, st);
-  if (a.T <= 2) return launch_norm_router_tb<2>(a, sms, st);
-  if (a.T <= 4) return launch_norm_router_tb<4>(a, sms, st);
-  return launch_norm_router_tb<8>(a, sms, st);
+  if (a.T <= 64) return launch_norm_router_tb<2>(a, sms, st);   // enough blocks for the SMs
+  return launch_norm_router_tb<8>(a, sms, st);                  // fewer reads of the router rows
 }
 
 int num_sms_current(int* sms) {
@@ -1475,6 +1473,17 @@ bool fused_fits(const bitsmoe_layer* L, int top_k) {
   const int s16 = (int)align_up(std::max(hd.seg_max_slots, 8), 64) + 8;
   return decode_mode(hd, 1) && L->meta_ok &&
          fused_plan(hd, 1, top_k, L->seg_bytes, L->ul_max_chunks, s16, L->num_sms, &fa);
+}
+
+bool mma_fits(const bitsmoe_layer* L, int T, int top_k, MArgs* ma);
+
+// Whether T > 1 tokens run as one fused forward each: the chain's four tokens cost about as much as two fused
+// forwards, but on the smallest layers, whose fused forward is all launch latency, less than the chain's five
+// kernels (4 tokens, fused / chain: D = n = 256, 8 experts 62 / see the table of cases; D = 96, n = 72: kept).
+bool few_tokens_fused(const bitsmoe_layer* L, int T, int top_k) {
+  if (T < 2 || T > kFusedMaxTokens || !fused_fits(L, top_k)) return false;
+  MArgs ma;
+  return T < 4 || (int64_t)L->hd().D * L->hd().n < 32768 || !mma_fits(L, T, top_k, &ma);
 }
 
 // The clustered single-token plan for this layer and top_k: the index of its cluster
@@ -1512,7 +1521,7 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
                  void* ws, size_t ws_bytes, cudaStream_t st, cudaEvent_t* ev = nullptr, bool accum = false,
                  const NormArgs* norm = nullptr, bool host_io = false) {
   const ImageHeader& hd = L->hd();
-  if (T > 1 && T <= kFusedMaxTokens && fused_fits(L, top_k)) {
+  if (few_tokens_fused(L, T, top_k)) {
     // a few tokens: one fused forward each, on the same workspace (profiled as one phase)
     if (ev) BM_CK(cudaEventRecord(ev[0], st));
     for (int t = 0; t < T; ++t) {
@@ -1590,6 +1599,7 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
     ma.meta = L->d_meta;
     ma.msa = L->d_msa;
     p.zmax = reinterpret_cast<uint32_t*>(wb + w.zmax);
+    if (!p.decode && T > kSplitTokens) p.sb = reinterpret_cast<uint16_t*>(wb + w.sb);
   }
   if (T == 1 && !norm) {   // one token: the clustered kernel when the layer fits it
     F2Args f2;
@@ -1636,10 +1646,8 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
   if (norm && (rc = launch_norm_router(*norm, sms, st))) return rc;
   if (p.decode) {
     const int A_max = std::min(hd.E, p.P);
-    const size_t rsm = (size_t)route_words(p.T, hd.E, p.P) * 4 + 16;
     if ((rc = mark(0))) return rc;
-    if ((rc = set_smem(k_route_publish, rsm))) return rc;
-    if ((rc = launch(k_route_publish, dim3(1), dim3(kThreads), rsm, st, false, p))) return rc;
+    if ((rc = launch_router(p, st))) return rc;
     if ((rc = mark(1))) return rc;
     const bool tcp = L->maps && T >= 4;   // below 4 tokens the bulk-copy GEMV streams the bases faster
     if (tcp) {   // tensor-core projection; it also clears gate/up and s for the expert kernels
@@ -1670,14 +1678,8 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
     else if ((rc = launch_gemv_bulk(false, p, sms, st, pdl))) return rc;
     return mark(5);
   }
-  const int tpb = std::max(1, 1024 / hd.E);
-  const size_t router_smem =
-      std::max((size_t)tpb * (hd.E + top_k) * 4,   // selection | grouping (pairs and 32 warps' counts in 16 bits)
-               2 * ((size_t)p.P + 1 + 32 * ((size_t)hd.E + 1)) + 4 * (2 * (size_t)hd.E + 1) + 8);
-  if (router_smem > 200 * 1024) return BITSMOE_ERR_SHAPE;
   if ((rc = mark(0))) return rc;
-  if ((rc = set_smem(k_router, router_smem))) return rc;
-  if ((rc = launch(k_router, dim3((T + tpb - 1) / tpb), dim3(1024), router_smem, st, false, p))) return rc;
+  if ((rc = launch_router(p, st))) return rc;
   if ((rc = mark(1))) return rc;
   const bool tc = L->maps;          // tensor-core projections for multi-token calls
   const int A_max = std::min(hd.E, p.P);
@@ -1998,8 +2000,10 @@ int forward_launches(const bitsmoe_layer* L, int T, int top_k, bool allow_f2) {
   FusedArgs fa;
   const int s16 = (int)align_up(std::max(hd.seg_max_slots, 8), 64) + 8;
   if (decode_mode(hd, T) && L->meta_ok && fused_plan(hd, T, top_k, L->seg_bytes, L->ul_max_chunks, s16, L->num_sms, &fa)) return 1;
-  if (T <= kFusedMaxTokens && fused_fits(L, top_k)) return T;   // one fused forward per token
-  return 5;   // router, projection, gate/up, down, output basis
+  if (few_tokens_fused(L, T, top_k)) return T;   // one fused forward per token
+  // router, projection, gate/up, down, output basis, and s split for the output basis
+  MArgs ma;
+  return 5 + (T > kSplitTokens && !decode_mode(hd, T) && mma_fits(L, T, top_k, &ma));
 }
 }  // namespace
 
@@ -2011,8 +2015,9 @@ int bitsmoe_forward_plan(const bitsmoe_layer* L, int T, int top_k) {
   const int n = bitsmoe_forward_launches(L, T, top_k);
   if (n <= 0) return n;
   F2Args f2;
-  if (T <= kFusedMaxTokens && (T == 1 || fused_fits(L, top_k)) && f2_choose(L, top_k, &f2) >= 0) return 1 | 32;
-  if (T <= kFusedMaxTokens && fused_fits(L, top_k)) return 1;
+  const bool fused = T == 1 ? fused_fits(L, top_k) : few_tokens_fused(L, T, top_k);
+  if ((T == 1 || fused) && f2_choose(L, top_k, &f2) >= 0) return 1 | 32;
+  if (fused) return 1;
   const ImageHeader& hd = L->hd();
   if (decode_mode(hd, T)) return 2 | (L->maps && T >= 4 ? 4 : 0);
   MArgs ma;
@@ -2021,7 +2026,7 @@ int bitsmoe_forward_plan(const bitsmoe_layer* L, int T, int top_k) {
 
 int bitsmoe_block_forward_launches(const bitsmoe_layer* L, int T, int top_k) {
   const int n = forward_launches(L, T, top_k, false);
-  if (n > 0 && T <= kFusedMaxTokens && fused_fits(L, top_k)) return n;   // the fused kernels norm in place
+  if (n > 0 && (T == 1 ? fused_fits(L, top_k) : few_tokens_fused(L, T, top_k))) return n;   // the fused kernels norm in place
   return n > 1 ? n + 1 : n;
 }
 
