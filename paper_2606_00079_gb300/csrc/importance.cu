@@ -17,17 +17,19 @@
 // all on the float factors of the decomposition, before anything is quantised.  Steps:
 //
 //   k_imp_route    one block per token: the k largest logits (ties to the lower index),
-//                  softmax over them -> the dense affinity matrix G (T x E) and, per
-//                  expert, the list of its tokens with their gate weights
-//   k_gemm<Z>      Z_h = Phi_h^T X for h = gate, up            (n x T)
+//                  softmax over them -> the dense affinity matrix G (T x E) and the tokens
+//                  of each expert
+//   k_imp_lists    each expert's tokens in token order with their gate weights, one block
+//                  an expert
+//   k_gemm<Z>      Z_h = Phi_h^T X for h = gate, up            (stored T x n)
 //   k_gemm<BGU>    beta_h[e, k] = sum_t Z_h[k, t]^2 G[t, e]    (a contraction over tokens)
 //   k_gemm<AG>     a_g = P_g,e (alpha_g,e * Z_g[:, tokens of e])          per expert
 //   k_gemm<AUH>    h   = SiLU(a_g) * (P_u,e (alpha_u,e * Z_u[:, tokens]))  per expert
 //   k_gemm<DN>     beta_dn[e, k] = sum_j g_j (P_dn,e^T h)[k, j]^2          per expert
 //
-// Every contraction is fp32 on the CUDA cores (64 x 64 output tiles, four by four per
-// thread): the factors are fp32 and the result is compared with an fp64 oracle at a tight
-// tolerance, which bf16 tensor-core operands would not meet.
+// Every contraction is fp32 on the CUDA cores: the factors are fp32 and the result is
+// compared with an fp64 oracle at a tight tolerance, which bf16 tensor-core operands would
+// not meet.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -38,8 +40,8 @@
 
 namespace {
 
-constexpr int kTM = 64, kTN = 64, kTK = 16;   // output tile and K step
-constexpr int kGT = 256;                      // threads of a GEMM block (16 x 16, 4 x 4 each)
+constexpr int kTM = 128, kTN = 64, kTK = 16;  // output tile and K step
+constexpr int kGT = 256;                      // threads of a GEMM block (16 x 16, 8 x 4 outputs each)
 
 enum GemmKind { kZ = 0, kBGU = 1, kAG = 2, kAUH = 3, kDN = 4 };
 
@@ -53,9 +55,10 @@ struct ImpArgs {
   int T, D, E, I, n, k;
   // workspace
   float* G;                // [T][E] affinities
-  float* z;                // [2][n][T]
+  float* z;                // [2][T][n]
   int* cnt;                // [E] tokens per expert
   int* off;                // [E + 1] start of each expert's list (exclusive scan of cnt)
+  int* toff;               // [E + 1] its first column tile (exclusive scan of the lists' tiles of kTN)
   int* tok;                // [T * k] token of each (expert, slot), grouped by expert
   float* tw;               // [T * k] its gate weight
   float* ag;               // [I][T * k] a_g, then h, by the expert's columns
@@ -105,29 +108,61 @@ __global__ void k_imp_route(ImpArgs a) {
   }
 }
 
-// Token lists per expert: one block; the experts' starts by an exclusive scan, then each
-// token's (expert, weight) pairs in token order (one thread per expert keeps the order).
-__global__ void k_imp_lists(ImpArgs a) {
-  __shared__ int base[1025];
-  if (threadIdx.x == 0) {
-    int run = 0;
-    for (int e = 0; e < a.E; ++e) {
-      base[e] = run;
-      a.off[e] = run;
-      run += a.cnt[e];
-    }
-    a.off[a.E] = run;
+// Token lists per expert, one block an expert: its start by a prefix over the counts, then
+// its tokens in token order (each thread a contiguous part of the tokens).  One block for
+// all experts, a thread an expert, read G one token after another.
+constexpr int kLT = 256;
+__global__ void __launch_bounds__(kLT) k_imp_lists(ImpArgs a) {
+  __shared__ int red[3][kLT / 32];
+  const int e = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  int pre = 0, pret = 0;   // lists and tiles of the experts before
+  for (int i = tid; i < e; i += kLT) {
+    const int c = a.cnt[i];
+    pre += c;
+    pret += (c + kTN - 1) / kTN;
+  }
+  const int per = (a.T + kLT - 1) / kLT, t0 = min(a.T, tid * per), t1 = min(a.T, t0 + per);
+  int c = 0;
+  for (int t = t0; t < t1; ++t) c += a.G[(size_t)t * a.E + e] != 0.f;
+  int ci = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xFFFFFFFFu, ci, o);
+    if (lane >= o) ci += v;
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    pre += __shfl_xor_sync(0xFFFFFFFFu, pre, o);
+    pret += __shfl_xor_sync(0xFFFFFFFFu, pret, o);
+  }
+  if (lane == 31) red[0][wid] = ci;
+  if (lane == 0) {
+    red[1][wid] = pre;
+    red[2][wid] = pret;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < a.E; e += blockDim.x) {
-    int w = base[e];
-    for (int t = 0; t < a.T; ++t) {
-      const float g = a.G[(size_t)t * a.E + e];
-      if (g != 0.f) {
-        a.tok[w] = t;
-        a.tw[w] = g;
-        ++w;
-      }
+  int base = 0, tiles = 0, w = ci - c;
+  for (int i = 0; i < kLT / 32; ++i) {
+    base += red[1][i];
+    tiles += red[2][i];
+    if (i < wid) w += red[0][i];
+  }
+  if (tid == 0) {
+    a.off[e] = base;
+    a.toff[e] = tiles;
+    if (e == a.E - 1) {
+      const int n = a.cnt[e];
+      a.off[a.E] = base + n;
+      a.toff[a.E] = tiles + (n + kTN - 1) / kTN;
+    }
+  }
+  w += base;
+  for (int t = t0; t < t1; ++t) {
+    const float g = a.G[(size_t)t * a.E + e];
+    if (g != 0.f) {
+      a.tok[w] = t;
+      a.tw[w] = g;
+      ++w;
     }
   }
 }
@@ -135,150 +170,290 @@ __global__ void k_imp_lists(ImpArgs a) {
 // ---------------------------------------------------------------------------
 // fp32 contractions C = A B (M x N over K) with the operands of each step read in place
 // (transposed, gathered, squared or scaled on load) and the step's epilogue.
+//
+// Bound by the fp32 FMA pipe.  A 128 x 64 tile a block, 8 x 4 outputs a thread, multiplied
+// in row pairs (fma.f32x2: two products an issue slot, so the shared-memory reads and the
+// operand loads issue beside the FMAs); the next K step's operands are loaded while the
+// current one is multiplied, into the other of two buffers.  64 columns: an expert's token
+// list is cut into tiles of 64, its last tile computed 32 wide when no more are left.
+// Qwen3-shaped layer, 2048 tokens: 64 x 64 tiles of 4 x 4 outputs, single-buffered with
+// z gathered token by token, took 9.8 ms (19 TFLOP/s).
 // ---------------------------------------------------------------------------
 template <int KIND>
+__host__ __device__ constexpr bool per_expert() { return KIND == kAG || KIND == kAUH || KIND == kDN; }
+// whether consecutive kk are contiguous in memory (then a thread loads four kk of a row)
+template <int KIND>
+__host__ __device__ constexpr bool a_k_contig() { return KIND == kAG || KIND == kAUH; }
+template <int KIND>
+__host__ __device__ constexpr bool b_k_contig() { return KIND == kZ || KIND == kAG || KIND == kAUH; }
+
 struct Op {
-  int M, N, K, e, col0;   // col0: first column of the expert's token list
+  int M, N, K, e, col0;   // e: expert (or projection); col0: first column of the expert's token list
 };
 
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+// Four consecutive floats at p, of which `left` are inside (VEC: p 16-byte aligned when left >= 4)
+template <bool VEC>
+__device__ __forceinline__ float4 load4(const float* p, int left) {
+  if (VEC && left >= 4) return __ldg(reinterpret_cast<const float4*>(p));
+  float4 v;
+  v.x = left > 0 ? __ldg(p) : 0.f;
+  v.y = left > 1 ? __ldg(p + 1) : 0.f;
+  v.z = left > 2 ? __ldg(p + 2) : 0.f;
+  v.w = left > 3 ? __ldg(p + 3) : 0.f;
+  return v;
+}
+
+// Chunk q (of two) of this thread's part of the A tile at K step k0: four m of one kk, or four kk of one m.
+template <int KIND, bool VEC>
+__device__ __forceinline__ float4 a_load(const ImpArgs& a, const Op& o, int m0, int k0, int q) {
+  const int lin = threadIdx.x + kGT * q;
+  if (a_k_contig<KIND>()) {
+    const int m = m0 + (lin >> 2), kk = k0 + (lin & 3) * 4;
+    if (m >= o.M) return make_float4(0.f, 0.f, 0.f, 0.f);
+    return load4<VEC>(a.P[KIND == kAG ? 0 : 1] + ((size_t)o.e * a.I + m) * a.n + kk, o.K - kk);
+  }
+  const int kk = k0 + (lin >> 5), m = m0 + (lin & 31) * 4;
+  if (kk >= o.K) return make_float4(0.f, 0.f, 0.f, 0.f);
+  if (KIND == kZ) return load4<VEC>(a.phi[o.e] + (size_t)kk * a.n + m, o.M - m);                     // Phi_h^T
+  if (KIND == kDN) return load4<VEC>(a.P[2] + ((size_t)o.e * a.I + kk) * a.n + m, o.M - m);           // P_dn^T
+  float4 v = load4<VEC>(a.z + ((size_t)o.e * a.T + kk) * a.n + m, o.M - m);                           // z^2
+  v.x *= v.x;
+  v.y *= v.y;
+  v.z *= v.z;
+  v.w *= v.w;
+  return v;
+}
 template <int KIND>
-__device__ __forceinline__ Op<KIND> op_of(const ImpArgs& a) {
-  Op<KIND> o;
-  o.e = blockIdx.z;
-  o.col0 = 0;
-  if (KIND == kZ) {
-    o.M = a.n; o.N = a.T; o.K = a.D;
-  } else if (KIND == kBGU) {
-    o.M = a.n; o.N = a.E; o.K = a.T;
-  } else if (KIND == kAG || KIND == kAUH) {
-    o.col0 = a.off[o.e];
-    o.M = a.I; o.N = a.off[o.e + 1] - o.col0; o.K = a.n;
+__device__ __forceinline__ void a_store(float (*As)[kTM + 4], int q, const float4& v) {
+  const int lin = threadIdx.x + kGT * q;
+  if (a_k_contig<KIND>()) {
+    const int m = lin >> 2, kk = (lin & 3) * 4;
+    As[kk][m] = v.x;
+    As[kk + 1][m] = v.y;
+    As[kk + 2][m] = v.z;
+    As[kk + 3][m] = v.w;
   } else {
-    o.col0 = a.off[o.e];
-    o.M = a.n; o.N = a.off[o.e + 1] - o.col0; o.K = a.I;
+    *reinterpret_cast<float4*>(&As[lin >> 5][(lin & 31) * 4]) = v;
   }
-  return o;
 }
 
-// A(m, kk) and B(kk, j) of each kind (in bounds: the caller checks)
-template <int KIND>
-__device__ __forceinline__ float a_at(const ImpArgs& a, const Op<KIND>& o, int m, int kk) {
-  if (KIND == kZ) return a.phi[o.e][(size_t)kk * a.n + m];                       // Phi_h^T
-  if (KIND == kBGU) {
-    const float v = a.z[((size_t)o.e * a.n + m) * a.T + kk];
-    return v * v;                                                                  // z^2
-  }
-  if (KIND == kAG) return a.P[0][((size_t)o.e * a.I + m) * a.n + kk];
-  if (KIND == kAUH) return a.P[1][((size_t)o.e * a.I + m) * a.n + kk];
-  return a.P[2][((size_t)o.e * a.I + kk) * a.n + m];                               // P_dn^T
-}
-template <int KIND>
-__device__ __forceinline__ float b_at(const ImpArgs& a, const Op<KIND>& o, int kk, int j) {
+// This thread's four elements of the B tile: four kk of column j (row: this column's row of z or x), or four
+// columns of one kk.
+template <int KIND, bool VEC>
+__device__ __forceinline__ float4 b_load(const ImpArgs& a, const Op& o, int j0, int k0, size_t row) {
   const size_t TK = (size_t)a.T * a.k;
-  if (KIND == kZ) return bf16f(a.x[(size_t)j * a.D + kk]);                        // X^T
-  if (KIND == kBGU) return a.G[(size_t)kk * a.E + j];
-  if (KIND == kAG || KIND == kAUH) {
+  if (b_k_contig<KIND>()) {
+    const int j = j0 + (threadIdx.x >> 2), kk = k0 + (threadIdx.x & 3) * 4, left = o.K - kk;
+    if (j >= o.N || left <= 0) return make_float4(0.f, 0.f, 0.f, 0.f);
+    if (KIND == kZ) {   // X^T
+      const uint16_t* xp = a.x + row * a.D + kk;
+      if (VEC && left >= 4) {
+        const uint2 w = __ldg(reinterpret_cast<const uint2*>(xp));
+        return make_float4(bf16lo(w.x), bf16hi(w.x), bf16lo(w.y), bf16hi(w.y));
+      }
+      return make_float4(bf16f(xp[0]), left > 1 ? bf16f(xp[1]) : 0.f, left > 2 ? bf16f(xp[2]) : 0.f,
+                         left > 3 ? bf16f(xp[3]) : 0.f);
+    }
     const int h = KIND == kAG ? 0 : 1;
-    const int t = a.tok[o.col0 + j];
-    return a.alpha[h][(size_t)o.e * a.n + kk] * a.z[((size_t)h * a.n + kk) * a.T + t];
+    const float4 z = load4<VEC>(a.z + ((size_t)h * a.T + row) * a.n + kk, left);
+    const float4 al = load4<VEC>(a.alpha[h] + (size_t)o.e * a.n + kk, left);
+    return make_float4(al.x * z.x, al.y * z.y, al.z * z.z, al.w * z.w);
   }
-  return a.ag[(size_t)kk * TK + o.col0 + j];                                      // h
+  const int kk = k0 + (threadIdx.x >> 4), j = j0 + (threadIdx.x & 15) * 4;
+  if (kk >= o.K) return make_float4(0.f, 0.f, 0.f, 0.f);
+  const float* p = KIND == kBGU ? a.G + (size_t)kk * a.E + j : a.ag + (size_t)kk * TK + o.col0 + j;   // G, h
+  return load4<false>(p, o.N - j);   // (a list starts anywhere in its row)
 }
-// whether consecutive kk are contiguous in memory (then a warp walks kk while loading)
 template <int KIND>
-__host__ __device__ constexpr bool a_k_contig() { return KIND == kBGU || KIND == kAG || KIND == kAUH; }
-template <int KIND>
-__host__ __device__ constexpr bool b_k_contig() { return KIND == kZ; }
+__device__ __forceinline__ void b_store(float (*Bs)[kTN + 4], const float4& v) {
+  if (b_k_contig<KIND>()) {
+    const int j = threadIdx.x >> 2, kk = (threadIdx.x & 3) * 4;
+    Bs[kk][j] = v.x;
+    Bs[kk + 1][j] = v.y;
+    Bs[kk + 2][j] = v.z;
+    Bs[kk + 3][j] = v.w;
+  } else {
+    *reinterpret_cast<float4*>(&Bs[threadIdx.x >> 4][(threadIdx.x & 15) * 4]) = v;
+  }
+}
 
-template <int KIND>
-__global__ void __launch_bounds__(kGT) k_gemm(ImpArgs a) {
-  __shared__ float As[kTK][kTM + 4];
-  __shared__ float Bs[kTK][kTN + 4];
-  const Op<KIND> o = op_of<KIND>(a);
-  const int m0 = blockIdx.y * kTM, j0 = blockIdx.x * kTN;
-  if (m0 >= o.M || j0 >= o.N) return;
+// One output tile, TN (4 or 2) columns a thread: 16 TN columns from j0.
+template <int KIND, bool VEC, int TN>
+__device__ __forceinline__ void tile(const ImpArgs& a, const Op& o, int m0, int j0, float (*As)[kTK][kTM + 4],
+                                     float (*Bs)[kTK][kTN + 4]) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  float acc[4][4];
+  size_t row = 0;   // the token of this thread's column of B
+  if (b_k_contig<KIND>()) {
+    const int j = min(j0 + (tid >> 2), o.N - 1);
+    row = KIND == kZ ? (size_t)j : (size_t)a.tok[o.col0 + j];
+  }
+  unsigned long long acc[4][TN];
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-  for (int k0 = 0; k0 < o.K; k0 += kTK) {
+    for (int c = 0; c < TN; ++c) acc[r][c] = 0ull;
+  float4 av[2], bv;
+  auto fetch = [&](int k0) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int idx = tid + kGT * r;
-      int mm, kk, jj, kb;
-      if (a_k_contig<KIND>()) {
-        kk = idx % kTK;
-        mm = idx / kTK;
-      } else {
-        mm = idx % kTM;
-        kk = idx / kTM;
-      }
-      if (b_k_contig<KIND>()) {
-        kb = idx % kTK;
-        jj = idx / kTK;
-      } else {
-        jj = idx % kTN;
-        kb = idx / kTN;
-      }
-      const int gm = m0 + mm, gk = k0 + kk, gj = j0 + jj, gkb = k0 + kb;
-      As[kk][mm] = (gm < o.M && gk < o.K) ? a_at<KIND>(a, o, gm, gk) : 0.f;
-      Bs[kb][jj] = (gkb < o.K && gj < o.N) ? b_at<KIND>(a, o, gkb, gj) : 0.f;
-    }
-    __syncthreads();
+    for (int q = 0; q < 2; ++q) av[q] = a_load<KIND, VEC>(a, o, m0, k0, q);
+    bv = b_load<KIND, VEC>(a, o, j0, k0, row);
+  };
+  auto put = [&](int s) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) a_store<KIND>(As[s], q, av[q]);
+    b_store<KIND>(Bs[s], bv);
+  };
+  fetch(0);
+  put(0);
+  __syncthreads();
+  for (int k0 = 0, s = 0; k0 < o.K; k0 += kTK, s ^= 1) {
+    const bool more = k0 + kTK < o.K;
+    if (more) fetch(k0 + kTK);
 #pragma unroll
     for (int kk = 0; kk < kTK; ++kk) {
-      const float4 av = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-      const float4 bv = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-      const float ar[4] = {av.x, av.y, av.z, av.w}, br[4] = {bv.x, bv.y, bv.z, bv.w};
+      const ulonglong2 p0 = *reinterpret_cast<const ulonglong2*>(&As[s][kk][ty * 8]);
+      const ulonglong2 p1 = *reinterpret_cast<const ulonglong2*>(&As[s][kk][ty * 8 + 4]);
+      const unsigned long long ar[4] = {p0.x, p0.y, p1.x, p1.y};
+      float br[TN];
+      if (TN == 4) {
+        const float4 w = *reinterpret_cast<const float4*>(&Bs[s][kk][tx * 4]);
+        br[0] = w.x;
+        br[1] = w.y;
+        br[TN - 2] = w.z;
+        br[TN - 1] = w.w;
+      } else {
+        const float2 w = *reinterpret_cast<const float2*>(&Bs[s][kk][tx * 2]);
+        br[0] = w.x;
+        br[1] = w.y;
+      }
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int c = 0; c < TN; ++c) {
+        const unsigned long long bb = pack2(br[c], br[c]);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(ar[r], br[c], acc[r][c]);
+        for (int r = 0; r < 4; ++r) fma2(acc[r][c], ar[r], bb);
+      }
     }
+    if (more) put(s ^ 1);
     __syncthreads();
   }
   // epilogues
   const size_t TK = (size_t)a.T * a.k;
-  if (KIND == kDN) {
+  float v[8][TN];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < TN; ++c) {
+      const float2 p = unpack2(acc[r][c]);
+      v[2 * r][c] = p.x;
+      v[2 * r + 1][c] = p.y;
+    }
+  const int gm0 = m0 + ty * 8, gj0 = j0 + tx * TN;
+  if constexpr (KIND == kDN) {
     // beta_dn[e, m] += sum_j g_j acc(m, j)^2: the 16 threads of a row group add their columns
+    float gw[TN];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      float v = 0.f;
+    for (int c = 0; c < TN; ++c) gw[c] = gj0 + c < o.N ? a.tw[o.col0 + gj0 + c] : 0.f;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int gj = j0 + tx * 4 + c;
-        if (gj < o.N) v = fmaf(a.tw[o.col0 + gj], acc[r][c] * acc[r][c], v);
-      }
+    for (int r = 0; r < 8; ++r) {
+      float s = 0.f;
 #pragma unroll
-      for (int sh = 8; sh; sh >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, sh);
-      const int gm = m0 + ty * 4 + r;
-      if (tx == 0 && gm < o.M && v != 0.f) atomicAdd(a.beta + ((size_t)2 * a.E + o.e) * a.n + gm, v);
+      for (int c = 0; c < TN; ++c)
+        if (gj0 + c < o.N) s = fmaf(gw[c], v[r][c] * v[r][c], s);
+#pragma unroll
+      for (int sh = 8; sh; sh >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, sh);
+      if (tx == 0 && gm0 + r < o.M && s != 0.f) atomicAdd(a.beta + ((size_t)2 * a.E + o.e) * a.n + gm0 + r, s);
     }
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int gm = m0 + ty * 4 + r;
-    if (gm >= o.M) continue;
+  for (int c = 0; c < TN; ++c) {
+    const int gj = gj0 + c;
+    if (gj >= o.N) continue;
+    if (KIND == kZ || KIND == kBGU) {   // rows contiguous
+      float* p = KIND == kZ ? a.z + ((size_t)o.e * a.T + gj) * a.n + gm0 : a.beta + ((size_t)o.e * a.E + gj) * a.n + gm0;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int gj = j0 + tx * 4 + c;
-      if (gj >= o.N) continue;
-      if (KIND == kZ) {
-        a.z[((size_t)o.e * a.n + gm) * a.T + gj] = acc[r][c];
-      } else if (KIND == kBGU) {
-        a.beta[((size_t)o.e * a.E + gj) * a.n + gm] = acc[r][c];
-      } else if (KIND == kAG) {
-        a.ag[(size_t)gm * TK + o.col0 + gj] = acc[r][c];
-      } else {   // h = SiLU(a_g) * a_u
-        float* hp = a.ag + (size_t)gm * TK + o.col0 + gj;
-        const float g = *hp;
-        *hp = g / (1.f + expf(-g)) * acc[r][c];
+      for (int r = 0; r < 8; r += 4) {
+        if (VEC && gm0 + r + 4 <= o.M && KIND == kZ) {
+          *reinterpret_cast<float4*>(p + r) = make_float4(v[r][c], v[r + 1][c], v[r + 2][c], v[r + 3][c]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (gm0 + r + q < o.M) p[r + q] = v[r + q][c];
+        }
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        if (gm0 + r >= o.M) continue;
+        float* hp = a.ag + (size_t)(gm0 + r) * TK + o.col0 + gj;
+        if (KIND == kAG) {
+          *hp = v[r][c];
+        } else {   // h = SiLU(a_g) * a_u
+          const float g = *hp;
+          *hp = g / (1.f + expf(-g)) * v[r][c];
+        }
       }
     }
   }
+  }
+}
+
+// grid: x column tiles (of all experts' lists: the expert by its first tile), y row tiles, z projection
+template <int KIND, bool VEC>
+__global__ void __launch_bounds__(kGT, 2) k_gemm(ImpArgs a) {
+  __shared__ __align__(16) float As[2][kTK][kTM + 4];
+  __shared__ __align__(16) float Bs[2][kTK][kTN + 4];
+  Op o;
+  int jt = blockIdx.x;
+  o.col0 = 0;
+  if (per_expert<KIND>()) {
+    if (jt >= a.toff[a.E]) return;
+    int lo = 0, hi = a.E;   // the last expert whose first tile is at or before jt: one with tiles
+    while (hi - lo > 1) {
+      const int md = (lo + hi) >> 1;
+      if (a.toff[md] <= jt) lo = md;
+      else hi = md;
+    }
+    o.e = lo;
+    jt -= a.toff[lo];
+    o.col0 = a.off[lo];
+    o.N = a.off[lo + 1] - o.col0;
+    o.M = KIND == kDN ? a.n : a.I;
+    o.K = KIND == kDN ? a.I : a.n;
+  } else {
+    o.e = blockIdx.z;
+    o.M = a.n;
+    o.N = KIND == kZ ? a.T : a.E;
+    o.K = KIND == kZ ? a.D : a.T;
+  }
+  const int m0 = blockIdx.y * kTM, j0 = jt * kTN;
+  if (o.N - j0 > kTN / 2) tile<KIND, VEC, 4>(a, o, m0, j0, As, Bs);
+  else tile<KIND, VEC, 2>(a, o, m0, j0, As, Bs);
+}
+
+template <bool VEC>
+void run_gemms(const ImpArgs& a, cudaStream_t st) {
+  auto up = [](int64_t v, int d) { return (unsigned)((v + d - 1) / d); };
+  // column tiles of all lists: at most one partial tile an expert
+  const unsigned lists = (unsigned)((int64_t)a.T * a.k / kTN + a.E);
+  k_gemm<kZ, VEC><<<dim3(up(a.T, kTN), up(a.n, kTM), 2), kGT, 0, st>>>(a);
+  k_gemm<kBGU, VEC><<<dim3(up(a.E, kTN), up(a.n, kTM), 2), kGT, 0, st>>>(a);
+  k_gemm<kAG, VEC><<<dim3(lists, up(a.I, kTM)), kGT, 0, st>>>(a);
+  k_gemm<kAUH, VEC><<<dim3(lists, up(a.I, kTM)), kGT, 0, st>>>(a);
+  k_gemm<kDN, VEC><<<dim3(lists, up(a.n, kTM)), kGT, 0, st>>>(a);
 }
 
 }  // namespace
@@ -286,7 +461,7 @@ __global__ void __launch_bounds__(kGT) k_gemm(ImpArgs a) {
 namespace bmoe {
 
 struct ImpLayout {
-  size_t G, z, cnt, off, tok, tw, ag, total;
+  size_t G, z, cnt, off, toff, tok, tw, ag, total;
 };
 static ImpLayout imp_layout(int64_t T, int E, int I, int n, int k) {
   ImpLayout l;
@@ -300,6 +475,7 @@ static ImpLayout imp_layout(int64_t T, int E, int I, int n, int k) {
   l.z = put((size_t)2 * n * T * 4);
   l.cnt = put((size_t)E * 4);
   l.off = put(((size_t)E + 1) * 4);
+  l.toff = put(((size_t)E + 1) * 4);
   l.tok = put((size_t)T * k * 4);
   l.tw = put((size_t)T * k * 4);
   l.ag = put((size_t)I * T * k * 4);
@@ -348,6 +524,7 @@ int bitsmoe_importance(const void* x, const float* logits, int64_t T, int D, int
   a.z = reinterpret_cast<float*>(w + l.z);
   a.cnt = reinterpret_cast<int*>(w + l.cnt);
   a.off = reinterpret_cast<int*>(w + l.off);
+  a.toff = reinterpret_cast<int*>(w + l.toff);
   a.tok = reinterpret_cast<int*>(w + l.tok);
   a.tw = reinterpret_cast<float*>(w + l.tw);
   a.ag = reinterpret_cast<float*>(w + l.ag);
@@ -356,14 +533,13 @@ int bitsmoe_importance(const void* x, const float* logits, int64_t T, int D, int
   const size_t rsm = ((size_t)E + 2 * top_k) * 4;
   if (rsm > 48 * 1024) return BITSMOE_ERR_SHAPE;
   k_imp_route<<<(unsigned)T, 256, rsm, st>>>(a);
-  k_imp_lists<<<1, 256, 0, st>>>(a);
-  const unsigned tT = (unsigned)((T + kTN - 1) / kTN);
-  k_gemm<kZ><<<dim3(tT, (n + kTM - 1) / kTM, 2), kGT, 0, st>>>(a);
-  k_gemm<kBGU><<<dim3((E + kTN - 1) / kTN, (n + kTM - 1) / kTM, 2), kGT, 0, st>>>(a);
-  // an expert has at most T tokens; blocks past its count return at once
-  k_gemm<kAG><<<dim3(tT, (I + kTM - 1) / kTM, E), kGT, 0, st>>>(a);
-  k_gemm<kAUH><<<dim3(tT, (I + kTM - 1) / kTM, E), kGT, 0, st>>>(a);
-  k_gemm<kDN><<<dim3(tT, (n + kTM - 1) / kTM, E), kGT, 0, st>>>(a);
+  k_imp_lists<<<(unsigned)E, kLT, 0, st>>>(a);
+  // rows of the factors, bases, energies, z and x that a thread may read four elements at a time
+  uintptr_t al = reinterpret_cast<uintptr_t>(a.z) | reinterpret_cast<uintptr_t>(x);
+  for (int h = 0; h < 2; ++h) al |= reinterpret_cast<uintptr_t>(basis[h]) | reinterpret_cast<uintptr_t>(alpha[h]);
+  for (int h = 0; h < 3; ++h) al |= reinterpret_cast<uintptr_t>(factor[h]);
+  if (n % 4 == 0 && D % 4 == 0 && (al & 15) == 0) run_gemms<true>(a, st);
+  else run_gemms<false>(a, st);
   e = cudaGetLastError();
   return e == cudaSuccess ? BITSMOE_OK : fail(e);
 }

@@ -70,6 +70,35 @@ def test_importance_matches_oracle(env, D, n, E, I, k, T):
     assert np.all(beta >= 0)
 
 
+@pytest.mark.parametrize("D,n,I", [(51, 37, 100), (50, 38, 66), (52, 36, 132), (17, 130, 40)])
+def test_importance_list_lengths_and_unaligned_widths(env, D, n, I):
+    """Experts with list lengths around the token tiles' edges (none, one, 31 to 33, 64, 65, 129 tokens), at widths
+    that 16-byte loads divide and that they do not (element-wise loads)."""
+    torch, bm = env
+    lengths = [0, 1, 31, 32, 33, 64, 65, 129]
+    E, T = len(lengths), sum(lengths)
+    Phi = [np.linalg.qr(np.random.default_rng(h).standard_normal((max(D, n), min(D, n))))[0].astype(np.float32)
+           for h in range(2)]
+    Phi = [p if D >= n else np.ascontiguousarray(p.T) for p in Phi]
+    rng = np.random.default_rng(D)
+    alpha = [rng.uniform(0.1, 1.0, (E, n)).astype(np.float32) for _ in range(3)]
+    P = [(rng.standard_normal((E, I, n)) / np.sqrt(I)).astype(np.float32) for _ in range(3)]
+    x = synth.f32_to_bf16_bits(rng.standard_normal((T, D)).astype(np.float32))
+    owner = rng.permutation(np.repeat(np.arange(E), lengths))
+    logits = np.zeros((T, E), np.float32)
+    logits[np.arange(T), owner] = 4.0
+    ref = C.factor_importance(Phi + [Phi[0]], alpha, [[P[h][e] for e in range(E)] for h in range(3)], x, logits, 1)
+    dev = torch.device("cuda")
+    put = lambda a: torch.from_numpy(a).to(dev)
+    beta = bm.importance(put(x.view(np.int16)), put(logits), 1, [put(p) for p in Phi], [put(a) for a in alpha[:2]],
+                         [put(p) for p in P]).cpu().numpy().astype(np.float64)
+    assert not beta[:, 0].any()
+    for h in range(3):
+        for e in range(1, E):
+            err = np.max(np.abs(beta[h, e] - ref[h, e])) / np.max(np.abs(ref[h, e]))
+            assert err <= TOL, (h, e, err)
+
+
 def test_importance_no_tokens_and_bad_args(env):
     torch, bm = env
     D, n, E, I, k = 64, 32, 4, 64, 2
