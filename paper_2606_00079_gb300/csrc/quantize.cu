@@ -22,13 +22,16 @@
 // error winning with ties to the smaller candidate index, so the result is a
 // deterministic function of the inputs.
 //
-// Work decomposition: one warp per (unit, group).  The group's elements are
-// staged in shared memory; for the scale search each lane owns grid / 32
-// candidates in registers and scores them all on every element it reads (a
-// broadcast read), so the inner loop is eight fp32 instructions per
-// (element, candidate) — six for the upper quarter of the candidates, which
-// provably never clip — and no shuffles; one lexicographic (error, index)
-// warp reduction picks the scale.  The search is ALU-bound: the fp32 input is
+// Work decomposition: one warp per (unit, group), the group's elements staged in shared
+// memory.  The scale search first scores every ST-th candidate (one or two a lane); the
+// others are scored only where a lower bound on their error does not exceed the least
+// one found.  The bound: the codes of a scale are the nearest ones, so with the codes q'
+// of s', ||x - s q(s)|| <= ||x - s q'|| <= ||x - s' q'|| + |s - s'| ||q'||, and ||q'|| <=
+// ||q(s_lo)|| for every s' >= s_lo (the levels shrink as the scale grows); taken from the
+// scored neighbours on both sides, with 1e-4 of each term for rounding (the sums' and
+// near ties': below 2e-5).  What is left is scored in full, in the same steps, so the
+// least error and its index are those of a search over all.  One lexicographic (error,
+// index) warp reduction picks the scale.  The search is ALU-bound: the fp32 input is
 // read once and the codes written once.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -72,78 +75,170 @@ __device__ __forceinline__ float candidate(float top, int c, int grid) {
   return f16_round(__fdiv_rn(__fmul_rn(top, (float)c), (float)grid));
 }
 
-// Scores of the NC candidates of a lane over the group.  With FREE, the candidates
-// m >= kFree(NC) skip the clamp: their index c > 3 grid / 4, so with a normal fp16 scale
-// |v| / s <= 2^(b-2) (grid / c) (1 + 2^-10) < 1.34 * 2^(b-2) < 2^(b-1) - 1/2 for b <= 4,
-// and round(v / s) is already a level: the clamp would change nothing.
-template <int NC>
-__host__ __device__ constexpr int kFree() { return (3 * NC + 3) / 4; }
-template <int NC, bool FREE>
-__device__ __forceinline__ void score(const float* v, int g, const float (&sc)[NC], const float (&rc)[NC],
-                                      float (&e)[NC], float qmin, float qmax) {
-#pragma unroll 2
+// Scores of K candidates (scale sc, reciprocal rc) of a lane over the group, and with NORM the squared norm of
+// their codes.  Two elements at a time in packed fp32 (every operation rounded as the scalar one: 5.5 issue
+// slots an element and candidate instead of 8, the two clamps on the other pipe); the squares are added one by
+// one, in order.
+template <int K, bool NORM>
+__device__ __forceinline__ void score(const float* v, int g, const float (&sc)[K], const float (&rc)[K], float (&e)[K],
+                                      float (&nn)[K], float qmin, float qmax) {
+  using u64 = unsigned long long;
+  auto pack = [](float a, float b) {
+    u64 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+  };
+  auto unpack = [](u64 r, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r)); };
+  const u64 up = pack(kRne, kRne), down = pack(-kRne, -kRne);
+  u64 s2[K], r2[K], n2[K];
+#pragma unroll
+  for (int m = 0; m < K; ++m) {
+    s2[m] = pack(-sc[m], -sc[m]);
+    r2[m] = pack(rc[m], rc[m]);
+    n2[m] = 0ull;
+  }
+#pragma unroll 4
   for (int i = 0; i < g; i += 4) {
-    const float4 x4 = *reinterpret_cast<const float4*>(v + i);
-    const float xs[4] = {x4.x, x4.y, x4.z, x4.w};
+    const ulonglong2 x4 = *reinterpret_cast<const ulonglong2*>(v + i);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int h = 0; h < 2; ++h) {
+      const u64 x = h ? x4.y : x4.x;
 #pragma unroll
-      for (int m = 0; m < NC; ++m) {
-        const float q = (FREE && m >= kFree<NC>())
-                            ? __fsub_rn(__fadd_rn(__fmul_rn(xs[k], rc[m]), kRne), kRne)
-                            : level(xs[k], rc[m], qmin, qmax);
-        const float d = fmaf(-sc[m], q, xs[k]);   // sc * q is exact (11 x 4 significant bits)
-        e[m] = __fadd_rn(e[m], __fmul_rn(d, d));
+      for (int m = 0; m < K; ++m) {
+        u64 t, q, d;
+        float a, b;
+        asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(x), "l"(r2[m]));
+        unpack(t, a, b);
+        a = fminf(fmaxf(a, qmin), qmax);
+        b = fminf(fmaxf(b, qmin), qmax);
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(q) : "l"(pack(a, b)), "l"(up));
+        asm("add.rn.f32x2 %0, %0, %1;" : "+l"(q) : "l"(down));
+        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(s2[m]), "l"(q), "l"(x));   // sc * q is exact (11 x 4 bits)
+        asm("mul.rn.f32x2 %0, %0, %0;" : "+l"(d));
+        if constexpr (NORM) asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(n2[m]) : "l"(q));
+        unpack(d, a, b);
+        e[m] = __fadd_rn(__fadd_rn(e[m], a), b);
       }
+    }
+  }
+  if constexpr (NORM) {
+#pragma unroll
+    for (int m = 0; m < K; ++m) {
+      float a, b;
+      unpack(n2[m], a, b);
+      nn[m] = a + b;
     }
   }
 }
 
-// Scale search of one group for b in {2, 3, 4}: NC candidates per lane.
+// (error, index) of the better of two, the smaller index on ties.
+__device__ __forceinline__ void better(float& be, int& bc, float e, int c) {
+  if (e < be || (e == be && c < bc)) {
+    be = e;
+    bc = c;
+  }
+}
+__device__ __forceinline__ void warp_better(float& be, int& bc) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) better(be, bc, __shfl_xor_sync(0xFFFFFFFFu, be, o), __shfl_xor_sync(0xFFFFFFFFu, bc, o));
+}
+
+// One warp's scored candidates and the list of those left to score.
 template <int NC>
-__device__ float search_scale(const float* v, int g, float rho, int b, int grid, int lane) {
+struct SearchMem {
+  static constexpr int K = NC == 1 || NC == 4 ? 1 : 2;   // candidates a lane scores first
+  static constexpr int ST = NC / K;                      // their stride
+  float s[32 * K], err[32 * K], norm[32 * K];            // scale, ||x - s q|| and ||q||
+  uint16_t list[ST > 1 ? 32 * NC : 1];
+};
+
+// Scores the candidates c[k] (0: none).
+template <int K, bool NORM>
+__device__ __forceinline__ void score_candidates(const float* v, int g, float top, int grid, const int (&c)[K], float qmin,
+                                                 float qmax, float (&sc)[K], float (&e)[K], float (&nn)[K]) {
+  float rc[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {   // a skipped candidate starts (and stays) at +inf error
+    const float s = c[k] ? candidate(top, c[k], grid) : 0.f;
+    const bool ok = usable(s);
+    sc[k] = ok ? s : 1.f;
+    rc[k] = __frcp_rn(sc[k]);
+    e[k] = ok ? 0.f : __int_as_float(0x7F800000);
+  }
+  score<K, NORM>(v, g, sc, rc, e, nn, qmin, qmax);
+}
+
+// Scale search of one group for b in {2, 3, 4}: 32 NC candidates.
+template <int NC>
+__device__ float search_scale(const float* v, int g, float rho, int b, int grid, int lane, SearchMem<NC>& sm) {
+  constexpr int K = SearchMem<NC>::K, ST = SearchMem<NC>::ST;
   const float qmax = (float)((1 << (b - 1)) - 1), qmin = -(float)(1 << (b - 1));
   const float top = __fmul_rn(rho, b == 2 ? 1.f : (b == 3 ? 0.5f : 0.25f));
   const float kInf = __int_as_float(0x7F800000);
-  float sc[NC], rc[NC], e[NC];
+  float be = kInf;
+  int bc = 0x7FFFFFFF;
+  const float cap = sqrtf((float)g) * -qmin;   // ||q|| of any codes
+  {
+    int c[K];
+    float sc[K], e[K], nn[K];
 #pragma unroll
-  for (int m = 0; m < NC; ++m) {   // a skipped candidate starts (and stays) at +inf error
-    const float s = candidate(top, lane + 1 + 32 * m, grid);
-    const bool ok = usable(s);
-    sc[m] = ok ? s : 1.f;
-    rc[m] = __frcp_rn(sc[m]);
-    e[m] = ok ? 0.f : kInf;
-  }
-  // the clamp-free path needs every lane's upper candidates to be normal fp16 scales (or skipped)
-  bool normal = true;
+    for (int k = 0; k < K; ++k) c[k] = (lane + 32 * k + 1) * ST;
+    score_candidates<K, (ST > 1)>(v, g, top, grid, c, qmin, qmax, sc, e, nn);
 #pragma unroll
-  for (int m = kFree<NC>(); m < NC; ++m) normal &= (sc[m] >= 6.103515625e-05f) || e[m] == kInf;
-  if (__all_sync(0xFFFFFFFFu, normal)) score<NC, true>(v, g, sc, rc, e, qmin, qmax);
-  else score<NC, false>(v, g, sc, rc, e, qmin, qmax);
-  float be = e[0];
-  int bc = lane + 1;
-#pragma unroll
-  for (int m = 1; m < NC; ++m) {
-    if (e[m] < be) {
-      be = e[m];
-      bc = lane + 1 + 32 * m;
+    for (int k = 0; k < K; ++k) {
+      better(be, bc, e[k], c[k]);
+      if constexpr (ST > 1) {   // no bound from a skipped candidate or an overflowed sum
+        const bool ok = e[k] < kInf;
+        sm.s[lane + 32 * k] = candidate(top, c[k], grid);
+        sm.err[lane + 32 * k] = ok ? sqrtf(e[k]) * 0.9999f : 0.f;
+        sm.norm[lane + 32 * k] = ok ? sqrtf(nn[k]) * 1.0001f : cap;
+      }
     }
+    warp_better(be, bc);
   }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    const float oe = __shfl_xor_sync(0xFFFFFFFFu, be, o);
-    const int oc = __shfl_xor_sync(0xFFFFFFFFu, bc, o);
-    if (oe < be || (oe == be && oc < bc)) {
-      be = oe;
-      bc = oc;
+  if constexpr (ST > 1) {
+    __syncwarp();
+    const float lim = sqrtf(be) * 1.0001f;
+    int cnt = 0;
+#pragma unroll 1
+    for (int m = 0; m < NC; ++m) {
+      const int c = lane + 1 + 32 * m, hi = c / ST, lo = hi - 1;   // scored neighbours: (lo + 1) ST < c < (hi + 1) ST
+      const float s = candidate(top, c, grid);
+      bool keep = c % ST != 0 && usable(s);
+      if (keep) {
+        const float nq = lo >= 0 ? sm.norm[lo] : cap;
+        if (sm.err[hi] - (sm.s[hi] - s) * nq > lim) keep = false;
+        if (lo >= 0 && sm.err[lo] - (s - sm.s[lo]) * nq > lim) keep = false;
+      }
+      const unsigned mk = __ballot_sync(0xFFFFFFFFu, keep);
+      if (keep) sm.list[cnt + __popc(mk & ((1u << lane) - 1u))] = (uint16_t)c;
+      cnt += __popc(mk);
     }
+    __syncwarp();
+    int i = 0;
+    for (; cnt - i > 32; i += 64) {
+      const int c[2] = {(int)sm.list[i + lane], i + 32 + lane < cnt ? (int)sm.list[i + 32 + lane] : 0};
+      float sc[2], e[2], nn[2];
+      score_candidates<2, false>(v, g, top, grid, c, qmin, qmax, sc, e, nn);
+      better(be, bc, e[0], c[0]);
+      if (c[1]) better(be, bc, e[1], c[1]);
+    }
+    if (i < cnt) {
+      const int c[1] = {i + lane < cnt ? (int)sm.list[i + lane] : 0};
+      float sc[1], e[1], nn[1];
+      score_candidates<1, false>(v, g, top, grid, c, qmin, qmax, sc, e, nn);
+      if (c[0]) better(be, bc, e[0], c[0]);
+    }
+    warp_better(be, bc);
+    __syncwarp();   // the next group's search writes the lists
   }
-  return be == kInf ? 0.f : candidate(top, bc, grid);
+  return be < kInf ? candidate(top, bc, grid) : 0.f;
 }
 
 template <int NC>
 __global__ void __launch_bounds__(kQThreads) k_quantize(QArgs a) {
   __shared__ __align__(16) float sv[kQWarps][kQMaxGroup];
+  __shared__ SearchMem<NC> found[kQWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float* v = sv[w];
   const int g = a.group;
@@ -183,7 +278,7 @@ __global__ void __launch_bounds__(kQThreads) k_quantize(QArgs a) {
     } else {
       const float half = (float)(1 << (b - 1));
       if (b <= 4) {
-        s = search_scale<NC>(v, g, rho, b, a.grid, lane);
+        s = search_scale<NC>(v, g, rho, b, a.grid, lane, found[w]);
       } else {
         s = f16_round(__fdiv_rn(rho, half - 1.f));
         if (!usable(s)) s = 0.f;

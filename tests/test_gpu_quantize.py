@@ -83,6 +83,25 @@ def test_scaled_and_extreme_values(env):
     assert_same(gpu_quantize(env, P, bits, 64, 128)[:3], Q.quantize_units(P, bits, 64, 128))
 
 
+@pytest.mark.parametrize("group,grid", [(32, 128), (64, 256), (128, 512), (256, 1024), (256, 256)])
+def test_bounded_search_on_many_shapes_of_groups(env, group, grid):
+    """Groups on which the pruned scale search keeps many, few or exactly tied candidates: Gaussian, uniform, heavy
+    tails, one outlier, two levels, constant, values that are codes times a scale (zero error), one sign, and the
+    same at subnormal scales and near the fp16 limit."""
+    rng = np.random.default_rng([group, grid])
+    I = 2 * group
+    rows = [rng.standard_normal(I), rng.uniform(-1, 1, I), rng.standard_t(1.5, I), rng.laplace(size=I) ** 3,
+            np.where(np.arange(I) % group == 3, 50.0, rng.standard_normal(I)), rng.choice([-1.0, 0.7], I),
+            np.full(I, 0.25), rng.integers(-2, 2, I) * 0.125, rng.integers(-8, 8, I) * 0.0625,
+            np.abs(rng.standard_normal(I)), -np.abs(rng.standard_normal(I)), np.eye(1, I, 5)[0],
+            np.linspace(-1, 1, I), rng.standard_normal(I) * 1e-5]
+    rows = np.stack(rows).astype(np.float32)
+    rows = np.concatenate([rows, rows * np.float32(3e-7), rows * np.float32(6e4)])
+    P = np.repeat(rows, 3, axis=0)
+    bits = np.tile(np.array([2, 3, 4], np.uint8), rows.shape[0])
+    assert_same(gpu_quantize(env, P, bits, group, grid)[:3], Q.quantize_units(P, bits, group, grid))
+
+
 def test_layer_sized_sample(env):
     """One Qwen3-shaped expert's worth of units (3 x 2048 units of 768, group 128, mean 2.0
     bits) in one launch; every 12th unit compared with the oracle."""
