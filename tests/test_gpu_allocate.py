@@ -106,6 +106,31 @@ def test_budget_extremes(env, budget):
         assert not got.any()
 
 
+@pytest.mark.parametrize("U,d", [(33, 4), (65, 388), (40, 1536), (40, 1540), (1, 64)])
+def test_row_lengths_at_the_edges_of_the_staging(env, U, d):
+    """Rows of 32 and of a ragged number to a stage, one row that fills a stage, one that does not fit."""
+    P, alpha, beta = _inputs(U, d, 11)
+    for per_unit in (0.4, 2.3):
+        budget = int(per_unit * U)
+        got, _ = gpu_alloc(env, P, alpha, beta, 0.5, budget)
+        assert_same(got, oracle_alloc(P, alpha, beta, 0.5, budget))
+
+
+@pytest.mark.parametrize("same", [True, False])
+def test_more_keys_in_one_bucket_than_the_list_holds(env, same):
+    """70000 units whose increments share their leading digits (identical units, or weights that differ in the
+    last bits): the cut's bucket is looked for among all keys again."""
+    U = 70000
+    P = np.repeat(_inputs(1, 64, 12)[0], U, axis=0)
+    alpha = np.full(U, 0.5, np.float32)
+    beta = np.ones(U, np.float32)
+    if not same:
+        beta += np.random.default_rng(0).integers(0, 200, U).astype(np.float32) * np.float32(2.0 ** -23)
+    for budget in (1001, 2 * U + 7):
+        got, _ = gpu_alloc(env, P, alpha, beta, 1.0, budget)
+        assert_same(got, oracle_alloc(P, alpha, beta, 1.0, budget))
+
+
 def test_duplicated_and_zero_units(env):
     """Identical units tie on every efficiency (the lower unit index goes first); all-zero
     units have zero high-bit distortion."""
