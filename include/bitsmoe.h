@@ -400,7 +400,7 @@ int bitsmoe_quantize_units(const float* p, const uint8_t* bits, int64_t U, int I
  *   ws      device workspace of >= bitsmoe_allocate_workspace_bytes(U)
  *           bytes, 256-byte aligned, caller-owned; no initialisation needed
  * Host-side checks only (INVALID_ARG, SHAPE, ALIGNMENT,
- * WORKSPACE_TOO_SMALL); never allocates, never synchronises.  43 kernel
+ * WORKSPACE_TOO_SMALL); never allocates, never synchronises.  10 kernel
  * launches and one memset on `stream`. */
 size_t bitsmoe_allocate_workspace_bytes(int64_t U);
 /* The budget of one projection type, B_h = floor(E n b_eq - 16 n^2 / m) (Eq.
@@ -466,7 +466,7 @@ int bitsmoe_importance(const void* x, const float* logits, int64_t T, int D, int
  *                           = Phi S V^T, P~_cat = V S split by input channels
  *   alpha[e][k] = ||P~_e[:, k]||_2, P_e = P~_e / alpha_e (P~_e where alpha = 0).
  * Computed as the eigendecomposition of G = W_cat^T W_cat (side 0) or W_cat W_cat^T
- * (side 1), D x D, in fp32 (cyclic two-sided Jacobi), then P~ = W_cat Phi (side 0)
+ * (side 1), D x D, in fp32 (blocked cyclic two-sided Jacobi), then P~ = W_cat Phi (side 0)
  * or W_cat^T Phi (side 1).  n = min(D, E d) columns, by descending singular
  * value (ties: the lower eigenvector index); each basis column's largest
  * |component| is positive (the first one on ties).  Singular values and
@@ -490,8 +490,8 @@ int bitsmoe_importance(const void* x, const float* logits, int64_t T, int D, int
  *           grid-barrier wait of the solver ran out (the call then leaves its
  *           outputs undefined); it is not cleared by the call
  * Host-side checks (INVALID_ARG, WORKSPACE_TOO_SMALL, ALIGNMENT, SHAPE when the
- * solver's block cannot be resident); never allocates, never synchronises.  Six
- * kernel launches (one cooperative). */
+ * solver's block cannot be resident); never allocates, never synchronises.  At
+ * most seven kernel launches (one cooperative). */
 #define BITSMOE_DECOMPOSE_MAX_D 8192
 size_t bitsmoe_decompose_workspace_bytes(int side, int E, int d, int D);
 int bitsmoe_shared_basis(int side, const float* W, int E, int d, int D, float* phi, float* sigma, float* alpha,

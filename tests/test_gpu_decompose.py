@@ -107,6 +107,23 @@ def test_properties_on_random_weights(env, side, E, d, D):
     assert np.max(np.abs(norms[live] - 1.0)) <= 1e-5
 
 
+@pytest.mark.parametrize("side,E,d,D", [("in", 1, 2, 2), ("in", 3, 700, 130), ("out", 2, 600, 252), ("in", 2, 850, 1600)])
+def test_row_ranges_and_block_counts(env, side, E, d, D):
+    """One pair of index blocks; Gram matrices summed over several ranges of rows (widths that 16-byte loads divide
+    and that they do not); so many pairs that V^T is updated after G."""
+    rng = np.random.default_rng(D)
+    W = [rng.standard_normal((d, D) if side == "in" else (D, d)).astype(np.float32) for _ in range(E)]
+    phi, sig, alpha, P, _ = run(env, W, side)
+    n = min(E * d, D)
+    Wcat = np.concatenate([w.astype(np.float64) for w in W], axis=0 if side == "in" else 1)
+    S_r = np.linalg.svd(Wcat, compute_uv=False)
+    assert np.max(np.abs(sig ** 2 - S_r[:n] ** 2)) <= (1e-5 + 8e-7 * np.sqrt(D)) * S_r[0] ** 2
+    assert np.max(np.abs(phi.T @ phi - np.eye(n))) <= 2e-5
+    Pt = np.concatenate([P[e].T * alpha[e][None, :] for e in range(E)], axis=0)
+    rebuilt = Pt @ phi.T if side == "in" else phi @ Pt.T
+    assert np.linalg.norm(rebuilt - Wcat) <= 2e-5 * np.linalg.norm(Wcat)
+
+
 def test_zero_expert_block(env):
     """An expert whose weights are all zero has alpha = 0 and P = 0 (P~_e / 1)."""
     W = prescribed(3, 16, 40, "in", seed=9)
