@@ -273,9 +273,10 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
       }
     }
     }
-    if (g.zero && blockIdx.z == 0) {   // a buffer that the following kernels accumulate into
-      const size_t nthr = (size_t)gridDim.x * gridDim.y * kStagers;
-      for (size_t i = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kStagers + bt; i < g.zero_n; i += nthr)
+    if (g.zero) {   // a buffer that the following kernels accumulate into (by every CTA: 50 MB at 1024 tokens)
+      const size_t nthr = (size_t)gridDim.x * gridDim.y * gridDim.z * kStagers;
+      const size_t cta = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+      for (size_t i = cta * kStagers + bt; i < g.zero_n; i += nthr)
         g.zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if (wid < 6) {
