@@ -155,6 +155,46 @@ __device__ __forceinline__ void split_pair(float a, float b, uint32_t& hi, uint3
   lo = *reinterpret_cast<const uint32_t*>(&l2);
 }
 
+// Packed fp32 pairs (each operation rounded as the scalar one; one issue slot for two: the gate/up kernel's
+// operands so, 386 -> 368 us at 1024 tokens).
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t r, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// split_pair of (v0, v2) and (v1, v3), given (v0, v1) and (v2, v3)
+__device__ __forceinline__ void split_quad(uint64_t v01, uint64_t v23, uint32_t (&hi)[2], uint32_t (&lo)[2]) {
+  const uint64_t kMask = 0xFFFFE000FFFFE000ull, minus = pack2(-1.f, -1.f);
+  const uint64_t h01 = v01 & kMask, h23 = v23 & kMask;
+  const uint64_t r01 = fma2(h01, minus, v01), r23 = fma2(h23, minus, v23);
+  float a, b, c, d;
+  auto half2 = [](float x, float y) {
+    const __half2 h = __floats2half2_rn(x, y);
+    return *reinterpret_cast<const uint32_t*>(&h);
+  };
+  unpack2(h01, a, b);
+  unpack2(h23, c, d);
+  hi[0] = half2(a, c);
+  hi[1] = half2(b, d);
+  unpack2(r01, a, b);
+  unpack2(r23, c, d);
+  lo[0] = half2(a, c);
+  lo[1] = half2(b, d);
+}
+
 // 2^S with m 2^S in [2^13, 2^14) (1 for m = 0 or not finite), |S| <= 100.
 __device__ __forceinline__ float scale_pow2(float m) {
   if (!(m > 0.f) || !(m < 3.0e38f)) return 1.f;
@@ -280,20 +320,23 @@ __device__ __forceinline__ void gu_bucket(const uint8_t* code, int ntl, const ui
   for (int ks = 0; ks < nks; ++ks) {
     const int sl = 16 * ks + 4 * t, slc = min(sl, nsl - 4);
     const float f = sl < nsl ? fB : 0.f;   // past the bucket: the codes read are another slot's
-    float4 zc[NT];
+    const uint64_t f2 = pack2(f, f);
+    ulonglong2 zc[NT];
 #pragma unroll
-    for (int n = 0; n < NT; ++n) zc[n] = *reinterpret_cast<const float4*>(az + (slc >> 2) * kQS + 128 * n);
+    for (int n = 0; n < NT; ++n) zc[n] = *reinterpret_cast<const ulonglong2*>(az + (slc >> 2) * kQS + 128 * n);
 #pragma unroll
     for (int gl = 0; gl < G; ++gl) {
       uint32_t bh[NT][2], bl[NT][2];
       const uint4 sz = *reinterpret_cast<const uint4*>(ssz + gl * zs + slc);
-      const float w0 = f16lo(sz.x) * f, w1 = f16lo(sz.y) * f, w2 = f16lo(sz.z) * f, w3 = f16lo(sz.w) * f;
+      const uint64_t w01 = mul2(pack2(f16lo(sz.x), f16lo(sz.y)), f2), w23 = mul2(pack2(f16lo(sz.z), f16lo(sz.w)), f2);
 #pragma unroll
       for (int n = 0; n < NT; ++n) {
-        const float v0 = w0 * zc[n].x, v1 = w1 * zc[n].y, v2 = w2 * zc[n].z, v3 = w3 * zc[n].w;
+        const uint64_t v01 = mul2(w01, zc[n].x), v23 = mul2(w23, zc[n].y);
+        float v0, v1, v2, v3;
+        unpack2(v01, v0, v1);
+        unpack2(v23, v2, v3);
         ce[gl][n] = fmaf(f16hi(sz.x), v0, fmaf(f16hi(sz.y), v1, fmaf(f16hi(sz.z), v2, fmaf(f16hi(sz.w), v3, ce[gl][n]))));
-        split_pair(v0, v2, bh[n][0], bl[n][0]);
-        split_pair(v1, v3, bh[n][1], bl[n][1]);
+        split_quad(v01, v23, bh[n], bl[n]);
       }
 #pragma unroll
       for (int jj = 0; jj < 4 / G; jj += JP) {
@@ -709,14 +752,15 @@ __device__ __forceinline__ void ul_a(const UlWords<B>& u, int k, int t, uint32_t
 }
 
 // One row block of a tile: out += scale (P 2^(24 - S) - zero sum(h)) per group.  The hi and lo products of a
-// token group keep accumulators of their own, so that consecutive products do not wait for one another.
+// K-step go into the same accumulators, all hi ones first (apart, they took 16 registers more and spilled: 283 us
+// at 1024 tokens against 272).
 template <int B, int NT, int NTM, int G>
 __device__ __forceinline__ void dn_rb(const uint8_t* code, const uint4* hf, int hstride, const float4* hz, int zstride,
                                       const uint32_t* sz, int lane, float (&out)[2][NTM][4]) {
   constexpr float fP = 1.f / (float)(1 << code_pos<B>());   // the codes' position
   constexpr int KS = 8 / G;                                  // K-steps of a group
   const int g = lane >> 2, t = lane & 3;
-  float P[2][NT][4], Q[2][NT][4];
+  float P[2][NT][4];
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
     UlWords<B> w[4];
@@ -731,18 +775,23 @@ __device__ __forceinline__ void dn_rb(const uint8_t* code, const uint4* hf, int 
 #pragma unroll
           for (int n = 0; n < NT; ++n)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) P[m][n][q] = Q[m][n][q] = 0.f;
+            for (int q = 0; q < 4; ++q) P[m][n][q] = 0.f;
       }
-      uint32_t lo[4], hi[4];
+      uint32_t lo[4], hi[4], bl[NT][2];
 #pragma unroll
       for (int u = 0; u < 4; ++u) ul_a<B>(w[u], k, t, lo[u], hi[u]);
 #pragma unroll
       for (int n = 0; n < NT; ++n) {
         const uint4 b = hf[n * hstride + ks * 32 + lane];
+        bl[n][0] = b.z;
+        bl[n][1] = b.w;
         mma_16816(P[0][n], lo[0], lo[1], hi[0], hi[1], b.x, b.y);
         mma_16816(P[1][n], lo[2], lo[3], hi[2], hi[3], b.x, b.y);
-        mma_16816(Q[0][n], lo[0], lo[1], hi[0], hi[1], b.z, b.w);
-        mma_16816(Q[1][n], lo[2], lo[3], hi[2], hi[3], b.z, b.w);
+      }
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        mma_16816(P[0][n], lo[0], lo[1], hi[0], hi[1], bl[n][0], bl[n][1]);
+        mma_16816(P[1][n], lo[2], lo[3], hi[2], hi[3], bl[n][0], bl[n][1]);
       }
       if (ks % KS == KS - 1) {
         float sc[4], zp[4];
@@ -759,10 +808,10 @@ __device__ __forceinline__ void dn_rb(const uint8_t* code, const uint4* hf, int 
           z.w *= fP;
 #pragma unroll
           for (int m = 0; m < 2; ++m) {
-            out[m][n][0] = fmaf(sc[2 * m], fmaf(P[m][n][0] + Q[m][n][0], z.y, -zp[2 * m] * z.x), out[m][n][0]);
-            out[m][n][1] = fmaf(sc[2 * m], fmaf(P[m][n][1] + Q[m][n][1], z.w, -zp[2 * m] * z.z), out[m][n][1]);
-            out[m][n][2] = fmaf(sc[2 * m + 1], fmaf(P[m][n][2] + Q[m][n][2], z.y, -zp[2 * m + 1] * z.x), out[m][n][2]);
-            out[m][n][3] = fmaf(sc[2 * m + 1], fmaf(P[m][n][3] + Q[m][n][3], z.w, -zp[2 * m + 1] * z.z), out[m][n][3]);
+            out[m][n][0] = fmaf(sc[2 * m], fmaf(P[m][n][0], z.y, -zp[2 * m] * z.x), out[m][n][0]);
+            out[m][n][1] = fmaf(sc[2 * m], fmaf(P[m][n][1], z.w, -zp[2 * m] * z.z), out[m][n][1]);
+            out[m][n][2] = fmaf(sc[2 * m + 1], fmaf(P[m][n][2], z.y, -zp[2 * m + 1] * z.x), out[m][n][2]);
+            out[m][n][3] = fmaf(sc[2 * m + 1], fmaf(P[m][n][3], z.w, -zp[2 * m + 1] * z.z), out[m][n][3]);
           }
         }
       }
