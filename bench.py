@@ -597,7 +597,8 @@ def run_quantize(args, spec, rank, world, local):
     value = job_throughput(world, args.steps, U, ms)
     # roofline: the search's lane-instructions against the fp32 lanes at the clock seen under load
     low = ((bits >= 2) & (bits <= 4)).sum().item()
-    evals = float(low) * ng * group * grid
+    # the candidates that every group's search scores in full; the others only where a bound leaves them
+    evals = float(low) * ng * group * (64 if grid == 64 or grid >= 256 else 32)
     ops = evals * QUANT_OPS_PER_EVAL
     sec = ms_own / args.steps / 1e3
     peaks, _ = measured_peaks()
@@ -867,20 +868,21 @@ def run_decompose(args, spec, rank, world, local):
     value = world * args.steps * E * n / (ms / 1e3)
     sec = ms_own / args.steps / 1e3
     # the dominant kernel is the Jacobi solver (its share: the launch list under profiles/); its
-    # arithmetic per round: 8 flops per element of G (row and column rotations) and 4 per element
-    # of V^T, D^2 elements each, (D - 1) rounds a sweep, sweeps + 1 sweeps (the last one checks)
-    m = D + (D & 1)
-    jac_flops = 12.0 * D * D * (m - 1) * (sweeps + 1 if sweeps < 30 else 30)
+    # arithmetic per round of block pairs (h pairs of 64 indices): two 64^3 products for each of G's
+    # h (h - 1) / 2 tiles and one for each of V^T's h^2, 2 h - 1 rounds a sweep, sweeps + 1 sweeps
+    # (the last one checks)
+    h = (D + 63) // 64
+    jac_flops = 2.0 * 64 ** 3 * (h * (h - 1) + h * h) * (2 * h - 1) * (sweeps + 1 if sweeps < 30 else 30)
     peaks, _ = measured_peaks()
     sm_mhz = clocks.get("sm_mhz") or float(peaks.get("sm_max_mhz", 2070.0))
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     peak = sms * FP32_FLOPS_PER_SM_CLK * sm_mhz * 1e6 / 1e12
-    roofline = {"bound": "alu", "kernel": "k_jacobi (cyclic Jacobi eigensolver of the D x D Gram matrix, fp32)",
+    roofline = {"bound": "alu", "kernel": "k_jacobi (blocked cyclic Jacobi eigensolver of the D x D Gram matrix, fp32)",
                 "achieved": jac_flops / sec / 1e12, "peak": peak, "unit": "TFLOP/s",
                 "frac": jac_flops / sec / 1e12 / peak,
                 "peak_source": f"{sms} SMs x 128 fp32 lanes x 2 flops x {sm_mhz:.0f} MHz (median SM clock under load)",
-                "note": "the whole call's time in the denominator; the solver is bound by its rounds (one grid "
-                        "barrier and a pass over its rows of G and V^T each), not by arithmetic",
+                "note": "the whole call's time in the denominator; the solver is bound by its rounds (a chain of "
+                        "dependent rotations and two grid barriers each), not by arithmetic",
                 "traffic": None, "flops_per_launch": jac_flops, "duration_us": sec * 1e6, "sweeps": sweeps}
     # e2e: weights in from pinned host memory, basis + energies + spectral vectors back, every step
     ne = 2
@@ -979,10 +981,10 @@ def run_allocate(args, spec, rank, world, local):
     # roofline of the dominant phase (the profiling call times the three phases alone, with CUDA
     # events on the launching stream): algorithmic bytes of each phase
     #   costs_and_hull   k_alloc_cost: the unit rows, alpha, beta                       U (4 I + 8)
-    #   cut_and_result   4 radix passes over the increments (key 8 B + reach 1 B, 7 a unit),
-    #                    their 64 Ki-bin histograms read and cleared, the cut applied and
-    #                    the bit-widths written                                         5 U 63 + U + 4 MB
-    #   fill             16 rounds over every unit's next key and bit count             16 U 9
+    #   cut_and_result   the increments (key 8 B + reach 1 B, 7 a unit) read by the bucket's pass
+    #                    and by the final one, four 64 Ki-bin histograms read and cleared, the
+    #                    bit-widths written                                             2 U 63 + U + 4 MB
+    #   fill             the per-block table of next keys (512 x 17)                    70 KB
     nprof = 6
     ph = np.zeros(3)
     for i in range(nprof):
@@ -991,10 +993,10 @@ def run_allocate(args, spec, rank, world, local):
     peaks, peak_src = measured_peaks()
     peak = float(peaks.get("hbm_gbs", FALLBACK_HBM_GBS))
     names = ["costs_and_hull", "cut_and_result", "fill"]
-    kernels = ["k_alloc_cost (distortions, costs and hull of every unit)",
-               "radix select: k_alloc_hist + k_alloc_scan (4 passes), k_alloc_final",
-               "fill: 16 rounds of k_fill_max + k_fill_take"]
-    pbytes = [U * (4.0 * I + 8.0), 5.0 * U * 63 + U + 4 * 2 * 65536 * 8.0, 16.0 * U * 9]
+    kernels = ["k_alloc_cost_bulk (distortions, costs and hull of every unit)",
+               "radix select: k_alloc_compact, k_alloc_hist, k_alloc_scan (4 passes), k_alloc_final",
+               "fill: k_fill"]
+    pbytes = [U * (4.0 * I + 8.0), 2.0 * U * 63 + U + 4 * 2 * 65536 * 8.0, 512 * 17 * 8.0]
     dom = int(np.argmax(ph))
     gbs = [pbytes[i] / (ph[i] / 1e3) / 1e9 for i in range(3)]
     roofline = {"bound": "hbm", "kernel": kernels[dom], "achieved": gbs[dom], "peak": peak,

@@ -143,17 +143,19 @@ size_t bitsmoe_workspace_bytes(const bitsmoe_layer* layer, int T, int top_k);
  * (no counterpart in the paper: for callers that capture the forward into a
  * CUDA graph or count launches).  A single token runs as one fused persistent
  * kernel (1) when the layer's per-block shares of the bases and factors fit
- * in shared memory, and up to 4 tokens as one such kernel per token (T);
+ * in shared memory, and up to 3 tokens (4 when D n < 32768 or with 16-bit units) as one such
+ * kernel per token (T);
  * otherwise the forward is a chain of 5 kernels (routing, projection, gate/up,
- * down, output basis; see bitsmoe_forward_plan), 6 past 16 tokens on layers
+ * down, output basis; see bitsmoe_forward_plan), 6 past 64 tokens on layers
  * without 16-bit units (the spectral accumulator split for the output basis).
  * Returns a negative error code for invalid arguments. */
 int bitsmoe_forward_launches(const bitsmoe_layer* layer, int T, int top_k);
 
 /* How a forward of T tokens runs on this layer, as a bit set:
- *   1  the fused single-token kernel (once per token for up to 4 tokens)
+ *   1  the fused single-token kernel (once per token for up to 3 tokens, 4 when
+ *      D n < 32768 or with 16-bit units)
  *   2  the small-batch decode chain (T <= 8 on a layer that does not fit the
- *      fused kernel, else 5 <= T <= 8)
+ *      fused kernel, else the token counts past those of bit 1)
  *   4  tensor-core (tcgen05) shared-basis projections (every T > 8; the decode
  *      chain from 4 tokens)
  *   8  past 8 tokens: tensor-core gate/up factors (mma.sync over tiles of 8 or

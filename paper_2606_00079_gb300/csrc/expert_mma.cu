@@ -242,6 +242,7 @@ __device__ __forceinline__ void a_regs2(uint32_t w, int sh, uint32_t mul, uint32
 constexpr int kHW = 4;                       // helper warps of both kernels
 constexpr int kMmThreads = (kCW + kHW) * 32;
 constexpr int kMaxKH = 4;
+static_assert(kCW <= 16, "a stage's copies are issued by 16 lanes each for the codes and the scale/zero rows");
 
 struct GCur {
   int pos;               // unit at which the current (tile, projection, row group) run starts (>= hi: the end)

@@ -458,9 +458,9 @@ cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cud
   std::memset(&bmap, 0, sizeof(bmap));
   const int mtiles = (g.M + 127) / 128;
   // Token tiles of at most 256 (mode 1, whose stage holds hi and lo: 128).  B by TMA wherever its rows are
-  // 16-byte aligned: x always could be staged by warps instead, but past 16 tokens the staging loads' latency
+  // 16-byte aligned: x always could be staged by warps instead, but past 64 tokens the staging loads' latency
   // and, for s, its conversion by every row tile bound the kernel (128 tokens: 12 and 19 us of staging);
-  // mode 1 then needs s split beforehand (k_split, about 3 us with its launch: not worth it up to 16 tokens).
+  // mode 1 then needs s split beforehand (k_split, about 3 us with its launch: not worth it up to 64 tokens).
   const bool rows16 = mode == 0 ? p.D % 8 == 0 : p.sb != nullptr && p.T > kSplitTokens;
   g.N = (std::min(p.T, mode == 1 && rows16 ? 128 : 256) + 15) / 16 * 16;
   g.btma = rows16 && (mode == 0 ? make_map(&bmap, p.x, p.T, p.D, g.N) : make_map(&bmap, p.sb, 2 * p.T, p.n_pad, g.N));
