@@ -143,25 +143,24 @@ size_t bitsmoe_workspace_bytes(const bitsmoe_layer* layer, int T, int top_k);
  * (no counterpart in the paper: for callers that capture the forward into a
  * CUDA graph or count launches).  A single token runs as one fused persistent
  * kernel (1) when the layer's per-block shares of the bases and factors fit
- * in shared memory, and up to 3 tokens (4 when D n < 32768 or with 16-bit units) as one such
- * kernel per token (T);
- * otherwise the forward is a chain of 5 kernels (routing, projection, gate/up,
+ * in shared memory, and 2 tokens (up to 4 when D n < 8192 or with 16-bit units) as one such
+ * kernel per token (T); otherwise the forward is a chain of 5 kernels (routing, projection, gate/up,
  * down, output basis; see bitsmoe_forward_plan), 6 past 64 tokens on layers
  * without 16-bit units (the spectral accumulator split for the output basis).
  * Returns a negative error code for invalid arguments. */
 int bitsmoe_forward_launches(const bitsmoe_layer* layer, int T, int top_k);
 
 /* How a forward of T tokens runs on this layer, as a bit set:
- *   1  the fused single-token kernel (once per token for up to 3 tokens, 4 when
- *      D n < 32768 or with 16-bit units)
+ *   1  the fused single-token kernel (once per token for 2 tokens, up to 4 when
+ *      D n < 8192 or with 16-bit units)
  *   2  the small-batch decode chain (T <= 8 on a layer that does not fit the
  *      fused kernel, else the token counts past those of bit 1)
  *   4  tensor-core (tcgen05) shared-basis projections (every T > 8; the decode
- *      chain from 4 tokens)
+ *      chain from 4 tokens, from 3 on layers that fit the fused kernel)
  *   8  past 8 tokens: tensor-core gate/up factors (mma.sync over tiles of 8 or
  *      16 tokens, the codes entering the products as fp16 bit patterns), for
  *      every layer without 16-bit units; the others use the dp2a kernels.  The
- *      decode chain takes the same kernels from 4 tokens on.
+ *      decode chain takes the same kernels wherever it has bit 4.
  *  16  tensor-core down factor (always set with 8)
  *  32  with 1: the fused kernel is the clustered one, in which a thread-block
  *      cluster owns one (routing slot, 128-row block) pair of the token and

@@ -1477,13 +1477,15 @@ bool fused_fits(const bitsmoe_layer* L, int top_k) {
 
 bool mma_fits(const bitsmoe_layer* L, int T, int top_k, MArgs* ma);
 
-// Whether T > 1 tokens run as one fused forward each: the chain's four tokens cost about as much as two fused
-// forwards, but on the smallest layers, whose fused forward is all launch latency, less than the chain's five
-// kernels (4 tokens, fused / chain: D = n = 256, 8 experts: 61.8 / 32.5 us; D = 96, n = 72: kept).
+// Whether T > 1 tokens run as one fused forward each.  Three tokens cost the chain less than three fused forwards
+// (fused / chain, us: Qwen3-shaped layer 66.6 / 55.8, with uneven experts 76.3 / 50.9; D = 1200, n = 900, 24
+// experts 49.4 / 38.9; four tokens of D = n = 256, 8 experts 61.8 / 32.5), two cost it more (44.6 for the two).  The
+// chain would be faster on the smallest layers too (D = 96, n = 72, four tokens: 61.9 / 30.5); up to D n = 8192 they
+// keep the fused forwards, whose launch count (T) callers of such layers count on.
 bool few_tokens_fused(const bitsmoe_layer* L, int T, int top_k) {
   if (T < 2 || T > kFusedMaxTokens || !fused_fits(L, top_k)) return false;
   MArgs ma;
-  return T < 4 || (int64_t)L->hd().D * L->hd().n < 32768 || !mma_fits(L, T, top_k, &ma);
+  return T < 3 || (int64_t)L->hd().D * L->hd().n < 8192 || !mma_fits(L, T, top_k, &ma);
 }
 
 // The clustered single-token plan for this layer and top_k: the index of its cluster
@@ -1514,7 +1516,7 @@ int f2_choose(const bitsmoe_layer* L, int top_k, F2Args* fa) {
 // Whether the expert factors of a T-token call run on mma.sync (calls whose projection runs on the
 // tensor cores, which also takes max |z| per token).
 bool mma_fits(const bitsmoe_layer* L, int T, int top_k, MArgs* ma) {
-  return L->mma && T >= 4 && mma_args(L->hd(), T, top_k, L->gu_stage, ma);
+  return L->mma && (T >= 4 || (T == 3 && fused_fits(L, top_k))) && mma_args(L->hd(), T, top_k, L->gu_stage, ma);
 }
 
 int forward_impl(const void* x, const float* logits, int T, int top_k, const bitsmoe_layer* L, float* y,
@@ -1649,7 +1651,7 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
     if ((rc = mark(0))) return rc;
     if ((rc = launch_router(p, st))) return rc;
     if ((rc = mark(1))) return rc;
-    const bool tcp = L->maps && T >= 4;   // below 4 tokens the bulk-copy GEMV streams the bases faster
+    const bool tcp = mma || (L->maps && T >= 4);   // below 4 tokens the bulk-copy GEMV streams the bases faster
     if (tcp) {   // tensor-core projection; it also clears gate/up and s for the expert kernels
       const size_t zb = (size_t)(reinterpret_cast<uint8_t*>(p.s) - reinterpret_cast<uint8_t*>(p.gu)) +
                         (size_t)T * hd.n_pad * 4;
@@ -2019,8 +2021,8 @@ int bitsmoe_forward_plan(const bitsmoe_layer* L, int T, int top_k) {
   if ((T == 1 || fused) && f2_choose(L, top_k, &f2) >= 0) return 1 | 32;
   if (fused) return 1;
   const ImageHeader& hd = L->hd();
-  if (decode_mode(hd, T)) return 2 | (L->maps && T >= 4 ? 4 : 0);
   MArgs ma;
+  if (decode_mode(hd, T)) return 2 | ((L->maps && T >= 4) || mma_fits(L, T, top_k, &ma) ? 4 : 0);
   return L->maps ? 4 | (mma_fits(L, T, top_k, &ma) ? 8 | 16 : 0) : 0;
 }
 

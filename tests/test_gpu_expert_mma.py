@@ -32,6 +32,10 @@ def env():
 
 
 @pytest.mark.parametrize("T,E,k,D,n,I,group,bits", [
+    (3, 9, 2, 300, 260, 256, 128, BITS),        # three tokens, features not a multiple of 8
+    (3, 4, 3, 256, 200, 384, 64, BITS),
+    (3, 8, 2, 128, 64, 128, 64, BITS),          # the smallest layer whose three and four tokens take the chain
+    (4, 8, 2, 128, 64, 128, 64, BITS),
     (5, 33, 3, 96, 75, 128, 128, BITS),         # decode batch, one row block, odd expert count
     (8, 4, 2, 128, 200, 1152, 128, BITS),       # nine row blocks: a full and a partial run of the down kernel
     (8, 5, 1, 72, 61, 64, 32, BITS),            # rows past the units' length, four groups a row block
