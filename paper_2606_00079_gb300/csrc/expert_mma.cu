@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
       const uint32_t rwn2 = record(n2);
       const int prn2 = n2.pos < hi && n2.first ? pair_of(n2) : prn;
       if (i >= 2) ok &= mbar_wait(&empty[gr][s], (uint32_t)((i >> 1) - 1) & 1u);
-      __syncwarp();
+      if (!__all_sync(0xFFFFFFFFu, ok)) break;
       if (i > 0 && sub == 0) copies();
       if (c.first && sub == 0 && lane < 16) {
         runs[gr][run & 1].pair[lane] = pr;
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
       for (int i = 0;; ++i) {
         const int s = i & 1;
         ok &= mbar_wait(&full[gr][s], (uint32_t)(i >> 1) & 1u);
-        __syncwarp();
+        if (!__all_sync(0xFFFFFFFFu, ok)) break;   // a wait ran out: nothing of the stage can be used
         const GInfo& f = infos[gr][s];
         const int flags = f.flags;
         if (flags & 4) break;
@@ -754,7 +754,7 @@ __device__ __forceinline__ void ul_a(const UlWords<B>& u, int k, int t, uint32_t
 
 // One row block of a tile: out += scale (P 2^(24 - S) - zero sum(h)) per group.  The hi and lo products of a
 // K-step go into the same accumulators, all hi ones first (apart, they took 16 registers more and spilled: 283 us
-// at 1024 tokens against 272).
+// at 1024 tokens against 272; 258 with nothing spilled).
 template <int B, int NT, int NTM, int G>
 __device__ __forceinline__ void dn_rb(const uint8_t* code, const uint4* hf, int hstride, const float4* hz, int zstride,
                                       const uint32_t* sz, int lane, float (&out)[2][NTM][4]) {
@@ -941,7 +941,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
       const int pr = p.pair_list[tb.pst[c.a] + c.tt * kNT + min(lane & 15, ntk - 1)];
       const float pw = hw == 0 ? p.pair_weight[pr] : 0.f;
       if (k >= 2) ok &= mbar_wait(&hempty[s], (uint32_t)((k >> 1) - 1) & 1u);
-      __syncwarp();
+      if (!__all_sync(0xFFFFFFFFu, ok)) break;
       uint4* hf = reinterpret_cast<uint4*>(msm + L.hf + s * L.hfs);     // [NTM][RC][8 K-steps][32 lanes]
       float2* hz = reinterpret_cast<float2*>(msm + L.hz + s * L.hzs);   // [RC][G][kNT] (sum of h, 2^(24 - S))
       if (hw == 0 && lane < 16) {
@@ -1072,6 +1072,8 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
     uint32_t cph = 0;   // stage and phase of the piece being consumed
     while (c.p < hi) {   // a unit tile
       hold(c.ord);
+      bool live = __all_sync(0xFFFFFFFFu, ok);   // a wait that ran out ends the warp's work
+      if (!live) break;
       const int hs = held & 1, nrb = run_nrb(c), ntk = min(kNT, tb.cnt[c.a] - c.tt * kNT);
       const uint4* hf = reinterpret_cast<const uint4*>(msm + L.hf + hs * L.hfs);
       const float4* hz4 = reinterpret_cast<const float4*>(msm + L.hz + hs * L.hzs);
@@ -1088,7 +1090,8 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
         __syncwarp();   // the stage before has been read by every lane
         issue();
         ok &= mbar_wait(&bars[wid][cs], cph);
-        __syncwarp();
+        live = __all_sync(0xFFFFFFFFu, ok);
+        if (!live) break;
         if (rb == 0) bits = tbits[wid][c.ms];
         const int np = piece_len(bits, nrb - rb);
         const uint8_t* code = ring + (size_t)cs * kStagePiece;
@@ -1103,6 +1106,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
           cph ^= 1u;
         }
       }
+      if (!live) break;
       // s += g alpha out
       const int* un = reinterpret_cast<const int*>(md);
       const float* al = reinterpret_cast<const float*>(md + 128);
