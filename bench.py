@@ -598,7 +598,7 @@ def run_quantize(args, spec, rank, world, local):
     # roofline: the search's lane-instructions against the fp32 lanes at the clock seen under load
     low = ((bits >= 2) & (bits <= 4)).sum().item()
     # the candidates that every group's search scores in full; the others only where a bound leaves them
-    evals = float(low) * ng * group * (64 if grid == 64 or grid >= 256 else 32)
+    evals = float(low) * ng * group * (64 if grid == 64 or grid >= 512 else 32)
     ops = evals * QUANT_OPS_PER_EVAL
     sec = ms_own / args.steps / 1e3
     peaks, _ = measured_peaks()
