@@ -1367,8 +1367,14 @@ int launch_gemv_bulk(bool proj, const Fwd& p, int sms, cudaStream_t st, bool pdl
   return launch_gemv_bulk_tb<8>(proj, p, sms, st, pdl);
 }
 
+// Most pairs of a call: the grouping keeps a pair's place in its expert's list in 16 bits, so an expert may hold
+// 65535 pairs; P + 2 E < 51200 keeps below that (a call past it has always been refused).
+constexpr int kRouteWords = 51200;
+
 // Selection: 32 rows of keys; grouping: the pairs' experts and 32 warps' counts in 16 bits, counts and starts.
 int launch_router(const Fwd& p, cudaStream_t st) {
+  static_assert(kRouteWords <= 65536, "16-bit places");
+  if ((int64_t)p.P + 2 * p.E >= kRouteWords) return BITSMOE_ERR_SHAPE;
   const size_t smem = std::max((size_t)kRouteWarps * p.E * 4, 2 * ((size_t)p.P + 2 + kRouteWarps * ((size_t)p.E + 1)) +
                                                                   4 * (2 * (size_t)p.E + 2));
   if (smem > 200 * 1024) return BITSMOE_ERR_SHAPE;

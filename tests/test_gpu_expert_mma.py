@@ -70,6 +70,29 @@ def test_expert_tiles(env, T, E, k, D, n, I, group, bits):
     assert np.max(np.abs(y.cpu().numpy() - ref)) <= TOL * np.max(np.abs(ref))
 
 
+@pytest.mark.parametrize("E", [1, 3])
+def test_most_pairs(env, E):
+    """The router takes P + 2 E < 51200 pairs (its places inside an expert's list have 16 bits): the last accepted
+    call, with nearly all tokens on one expert, against the oracle; one pair more, and past 65536, is refused."""
+    torch, bm = env
+    spec = synth.scaled_spec(synth.WORKLOADS["tiny"], D=64, E=E, I=64, n=48, group=64, top_k=1)
+    layer = synth.make_layer(spec, seed=E, bits_dist=BITS, alpha_scale=4.0)
+    L = bm.bitsmoe_pack(layer, device=0)
+    T = 51200 - 2 * E - 1
+    x, logits = synth.make_inputs(spec, T, seed=E)
+    logits[:, 0] += 100.0
+    logits[7::1000, E - 1] += 200.0
+    y = bm.moe_forward(L, torch.from_numpy(x.view(np.int16)).cuda(), torch.from_numpy(logits).cuda(), 1)
+    ref = oracle.moe_forward_factored(layer, x, logits, 1)
+    assert np.max(np.abs(y.cpu().numpy() - ref)) <= TOL * np.max(np.abs(ref))
+    for over in (T + 1, 70000):
+        x2 = torch.zeros((over, spec.D), dtype=torch.int16, device="cuda")
+        lg = torch.zeros((over, E), dtype=torch.float32, device="cuda")
+        with pytest.raises(bm.BitsMoEError) as err:
+            bm.moe_forward(L, x2, lg, 1)
+        assert err.value.code == bm.ERR_CODE["SHAPE"]
+
+
 def wide_layer(spec, seed, bits):
     """A layer with more units than features (n > D): random bases of norm-1 columns."""
     layer = synth.make_layer(synth.scaled_spec(spec, D=spec.n), seed=seed, bits_dist=bits, alpha_scale=4.0,
