@@ -167,6 +167,7 @@ struct CostArgs {
   int64_t U;
   int d;
   AllocWs w;
+  int lose;   // testing hook: the warps of block 0 take their second wait for a stage as run out
 };
 
 // floor(|x| 2^40) for |x| < 32 as A 2^22 + B with A = floor(y), B = floor(frac(y) 2^22),
@@ -300,7 +301,41 @@ __global__ void __launch_bounds__(kAW * 32) k_alloc_cost(CostArgs a) {
 // all of them at their hulls at once (several microseconds without a request) the stream stood still.
 // HBM-bound: 262144 units of 768 floats, 805 MB: 196 us with the loads between the sums, 200 us by bulk copies
 // with the hulls in step, 149 us so (5.4 TB/s, 0.81 of the copy bandwidth).
+//
+// A wait for a stage that runs out (its bound is about a second) costs speed, not results: the warp requests no more,
+// reads the rows from that stage's on by ordinary loads, and before it leaves waits once more for the copies it
+// still has in flight.
 constexpr uint32_t kStageMax = 6144, kRowMax = kStageMax;
+
+// Rows k0 .. k0 + r - 1 of a warp's units, the first at `rows` (rb bytes apart), two side by side.
+__device__ __forceinline__ void rows_sums(const uint8_t* rows, uint32_t rb, int r, int d, int k0, float& rho, long long& l1) {
+  const int lane = threadIdx.x & 31;
+  for (int q0 = 0; q0 < r; q0 += 2) {
+    float mx[2];
+    uint32_t sa[2], sb[2], cnt = 0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      mx[q] = 0.f;
+      sa[q] = sb[q] = 0u;
+    }
+#pragma unroll 2
+    for (int i = lane; i < d / 4; i += 32) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float4 x = *reinterpret_cast<const float4*>(rows + (size_t)min(q0 + q, r - 1) * rb + 16 * i);
+        fix_add(fabsf(x.x), mx[q], sa[q], sb[q]);
+        fix_add(fabsf(x.y), mx[q], sa[q], sb[q]);
+        fix_add(fabsf(x.z), mx[q], sa[q], sb[q]);
+        fix_add(fabsf(x.w), mx[q], sa[q], sb[q]);
+      }
+      cnt += 4;
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (q0 + q < r) row_sums(mx[q], sa[q], sb[q], cnt, k0 + q0 + q, rho, l1);
+  }
+}
+
 __global__ void __launch_bounds__(kBW * 32) k_alloc_cost_bulk(CostArgs a, int rows) {
   extern __shared__ __align__(128) uint8_t ring_raw[];
   __shared__ unsigned long long sk[kBW][kNS * 32];
@@ -320,16 +355,17 @@ __global__ void __launch_bounds__(kBW * 32) k_alloc_cost_bulk(CostArgs a, int ro
   }
   __syncwarp();
   int64_t nb = u0;   // the stage to be requested next: rows nk .. of the group at nb
-  int nk = 0, ns = 0;
+  int nk = 0;
+  uint32_t asked = 0, had = 0;   // stages requested and consumed: the i-th is slot i & 1, parity (i >> 1) & 1
   auto request = [&]() {
     if (nb >= u1) return;
-    const int nu = group(nb), r = min(rows, nu - nk);
+    const int nu = group(nb), r = min(rows, nu - nk), s = (int)(asked & 1u);
     if (lane == 0) {
       fence_proxy_async();   // the stage was last read by the generic proxy
-      mbar_expect_tx(&bars[wid][ns], (uint32_t)r * rb);
-      bulk_g2s(ring + (size_t)ns * sb_, a.p + (size_t)(nb + nk) * a.d, (uint32_t)r * rb, &bars[wid][ns]);
+      mbar_expect_tx(&bars[wid][s], (uint32_t)r * rb);
+      bulk_g2s(ring + (size_t)s * sb_, a.p + (size_t)(nb + nk) * a.d, (uint32_t)r * rb, &bars[wid][s]);
     }
-    ns ^= 1;
+    ++asked;
     nk += r;
     if (nk == nu) {
       nk = 0;
@@ -337,49 +373,31 @@ __global__ void __launch_bounds__(kBW * 32) k_alloc_cost_bulk(CostArgs a, int ro
     }
   };
   request();
-  int cs = 0;
-  uint32_t ph = 0;
+  bool bulk = true;   // no wait has run out
+  const bool lose = a.lose && blockIdx.x == 0;
   for (int64_t base = u0; base < u1;) {
     const int nu = group(base);
     float my_rho = 0.f;
     long long my_l1 = 0;
     for (int k0 = 0; k0 < nu; k0 += rows) {
-      __syncwarp();   // the other stage has been read by every lane
-      request();
-      mbar_wait(&bars[wid][cs], ph);
-      __syncwarp();
-      const uint8_t* st = ring + (size_t)cs * sb_;
       const int r = min(rows, nu - k0);
-      for (int q0 = 0; q0 < r; q0 += 2) {   // two rows side by side
-        float mx[2];
-        uint32_t sa[2], sb[2], cnt = 0;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          mx[q] = 0.f;
-          sa[q] = sb[q] = 0u;
-        }
-#pragma unroll 2
-        for (int i = lane; i < a.d / 4; i += 32) {
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const float4 x = *reinterpret_cast<const float4*>(st + (size_t)min(q0 + q, r - 1) * rb + 16 * i);
-            fix_add(fabsf(x.x), mx[q], sa[q], sb[q]);
-            fix_add(fabsf(x.y), mx[q], sa[q], sb[q]);
-            fix_add(fabsf(x.z), mx[q], sa[q], sb[q]);
-            fix_add(fabsf(x.w), mx[q], sa[q], sb[q]);
-          }
-          cnt += 4;
-        }
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-          if (q0 + q < r) row_sums(mx[q], sa[q], sb[q], cnt, k0 + q0 + q, my_rho, my_l1);
+      if (bulk) {
+        __syncwarp();   // the other stage has been read by every lane
+        request();
+        const bool here = mbar_wait(&bars[wid][had & 1u], (had >> 1) & 1u) && !(lose && had == 1u);
+        bulk = __all_sync(0xFFFFFFFFu, here);
       }
-      if (cs) ph ^= 1u;
-      cs ^= 1;
+      if (bulk) {
+        rows_sums(ring + (size_t)(had & 1u) * sb_, rb, r, a.d, k0, my_rho, my_l1);
+        ++had;
+      } else {
+        rows_sums(reinterpret_cast<const uint8_t*>(a.p + (size_t)(base + k0) * a.d), rb, r, a.d, k0, my_rho, my_l1);
+      }
     }
     warp_hulls(a, base, nu, my_rho, my_l1, sk[wid], sr[wid]);
     base += nu;
   }
+  for (; had != asked; ++had) mbar_wait(&bars[wid][had & 1u], (had >> 1) & 1u);   // (only after a wait that ran out)
 }
 
 // Bits of increment s of unit u (its key is not 0).
@@ -683,7 +701,7 @@ int allocate_impl(const float* p, const float* alpha, const float* beta, float g
   cudaError_t e = cudaMemsetAsync(wb + off[0], 0, off[2], st);   // state and histograms
   if (e != cudaSuccess) return fail(e);
   if (phase_ms) cudaEventRecord(ev[0], st);
-  CostArgs ca{p, alpha, beta, gamma, kappa[0], kappa[1], kappa[2], U, d, w};
+  CostArgs ca{p, alpha, beta, gamma, kappa[0], kappa[1], kappa[2], U, d, w, bmoe::debug_skip_arrival()};
   const int64_t groups = (U + 31) / 32;
   const uint32_t row = (uint32_t)d * 4u;
   if (d % 4 == 0 && row <= kRowMax) {

@@ -87,7 +87,8 @@ namespace {
 constexpr int kF2Sizes[5] = {8, 4, 3, 2, 1};
 
 // Testing hook (bitsmoe_debug_wait_limit): bound of the single-token kernels' waits
-// and whether block 0 skips its arrival at their first grid barrier.
+// and whether block 0 skips its arrival at their first grid barrier (in the bit allocation's
+// cost kernel: takes a wait of each warp as run out).
 std::atomic<long long> g_dbg_spin{0};
 std::atomic<int> g_dbg_skip{0};
 // Testing hook (bitsmoe_debug_single_token_kernel): 1 keeps single-token forwards on the
@@ -1906,6 +1907,7 @@ int noalloc_scratch(int device, cudaStream_t st, void** out) {
 
 namespace bmoe {
 int record_cuda_error(int cuda_error) { return cuda_fail(static_cast<cudaError_t>(cuda_error)); }
+int debug_skip_arrival() { return g_dbg_skip.load(); }
 }  // namespace bmoe
 
 extern "C" {

@@ -168,3 +168,18 @@ def test_general_gamma_is_feasible_and_as_good(env):
 def test_empty_call_is_a_no_op(env):
     torch, bm = env
     assert bm.bitsmoe_allocate_bits(0, 0, 0, 0.5, 0, 16, KAPPA3, 10, 0, 0, 0, 0) is None
+
+
+@pytest.mark.parametrize("U,d", [(5000, 768), (3000, 1536), (2500, 4)])
+def test_copy_wait_that_runs_out(env, U, d):
+    """The warps of the cost kernel's block 0 take their second wait for a copied stage as run out (testing hook):
+    they go on by ordinary loads, and the bits are the same."""
+    torch, bm = env
+    P, alpha, beta = _inputs(U, d, 11)
+    want = oracle_alloc(P, alpha, beta, 0.5, 2 * U)
+    bm.bitsmoe_debug_wait_limit(1, 0)
+    try:
+        got, _ = gpu_alloc(env, P, alpha, beta, 0.5, 2 * U)
+    finally:
+        bm.bitsmoe_debug_wait_limit(0, 0)
+    assert_same(got, want)
