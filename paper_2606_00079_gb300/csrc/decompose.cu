@@ -594,6 +594,7 @@ __device__ void jacobi_solve_cross(const JacobiArgs& ja, int pair, int2 blk, flo
     pp = rj.x * xp - rj.y * xq;
     const float r1 = rj.x * xq + rj.y * xp, r2 = rj.x * yp - rj.y * yq;
     qq = rj.x * yq + rj.y * yp;
+    if (w == 0) __syncwarp();   // warp 0's upper lanes have read the elements that its lower lanes write
     if (mine) {
       *e1 = r1;
       *e2 = r2;
