@@ -172,14 +172,16 @@ int bitsmoe_forward_launches(const bitsmoe_layer* layer, int T, int top_k);
 int bitsmoe_forward_plan(const bitsmoe_layer* layer, int T, int top_k);
 
 /* Testing hook (no counterpart in the paper): bound every wait of the fused
- * single-token kernels to `spin_clocks` SM clocks (<= 0: the default, about one
- * second), and when skip_arrival is 1 let block 0 skip its arrival at the
- * first grid barrier, so that every other block's bounded wait runs out.  The
- * calls after it report BITSMOE_ERR_TIMEOUT through the device status word and
- * return; the workspace is left ready for the next call.  With skip_arrival = 1
- * the bit allocation's cost kernel also takes one wait of each warp of its block
- * 0 as run out (it then reads its rows by ordinary loads: the same bits).
- * Applies to calls issued after it on any host thread; skip_arrival = 0 with spin_clocks = 0
+ * single-token kernels, and the waits inside a block of the expert kernels of
+ * several tokens, to `spin_clocks` SM clocks (<= 0: the default, about one
+ * second), and when skip_arrival is 1 let block 0 skip an arrival (the former:
+ * at their first grid barrier, the latter: at a stage in shared memory), so that
+ * the bounded waits for it run out.  The calls after it report
+ * BITSMOE_ERR_TIMEOUT through the device status word and return; the workspace
+ * is left ready for the next call.  With skip_arrival = 1 the bit allocation's
+ * cost kernel also takes one wait of each warp of its block 0 as run out (it
+ * then reads its rows by ordinary loads: the same bits).  Applies to calls
+ * issued after it on any host thread; skip_arrival = 0 with spin_clocks = 0
  * restores the normal behaviour.  Returns BITSMOE_OK. */
 int bitsmoe_debug_wait_limit(int skip_arrival, long long spin_clocks);
 

@@ -63,6 +63,8 @@ struct MArgs {
   const DStage* dst;      // [E][ul_max_tiles]
   const uint8_t* meta;    // the records' slot metadata (mirror of the image's)
   const float* msa;       // [2][E] max over groups and slots of |scale * alpha| of gate/up (h, e)
+  long long spin;         // bound of the waits inside a block, in SM clocks
+  int lose;               // testing hook: an arrival of block 0 is left out, so that waits of its warps run out
 };
 
 // Staging records of the fused single-token kernel, derived from the image
@@ -313,11 +315,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
                : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
-// Bounded wait on an mbarrier phase (about one second of SM clock at most).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+// Bounded wait on an mbarrier phase (by default about one second of SM clock at most).
+constexpr long long kWaitClocks = 2ll << 30;
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit = kWaitClocks) {
   const long long t0 = clock64();
   while (!mbar_try_wait(bar, parity))
-    if (clock64() - t0 > (2ll << 30)) return false;
+    if (clock64() - t0 > limit) return false;
   return true;
 }
 // Copy `bytes` (16-byte multiple, 16-byte aligned ends) to shared memory on one

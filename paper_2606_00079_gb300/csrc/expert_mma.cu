@@ -497,12 +497,13 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
     units(rw, lane, uc, ac);
     int tok = 0, run = 0;
     float bs = 1.f;
-    for (int i = 0;; ++i) {
+    int i = 0;
+    for (;; ++i) {
       const int s = i & 1;
       GInfo& f = infos[gr][s];
       if (c.pos >= hi) {
-        if (i >= 2) ok &= mbar_wait(&empty[gr][s], (uint32_t)((i >> 1) - 1) & 1u);
-        __syncwarp();
+        if (i >= 2) ok &= mbar_wait(&empty[gr][s], (uint32_t)((i >> 1) - 1) & 1u, x.spin);
+        if (!__all_sync(0xFFFFFFFFu, ok)) break;
         if (lane == 0) {
           if (sub == 0) {
             f.flags = 4;
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
       if (n.pos < hi) advance(n2);
       const uint32_t rwn2 = record(n2);
       const int prn2 = n2.pos < hi && n2.first ? pair_of(n2) : prn;
-      if (i >= 2) ok &= mbar_wait(&empty[gr][s], (uint32_t)((i >> 1) - 1) & 1u);
+      if (i >= 2) ok &= mbar_wait(&empty[gr][s], (uint32_t)((i >> 1) - 1) & 1u, x.spin);
       if (!__all_sync(0xFFFFFFFFu, ok)) break;
       if (i > 0 && sub == 0) copies();
       if (c.first && sub == 0 && lane < 16) {
@@ -607,6 +608,11 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
       uc = un;
       ac = an;
     }
+    // No block leaves with copies in flight, whichever wait ran out: those of the last stage, and after a wait that
+    // ran out here those of the stage before it (otherwise it was consumed, and its slot holds the end mark).
+    if (sub == 0)
+      for (int j = max(0, __all_sync(0xFFFFFFFFu, ok) ? i - 1 : i - 2); j < i; ++j)
+        mbar_wait(&full[gr][j & 1], (uint32_t)(j >> 1) & 1u);
   } else {
     // ---- consumers
     pdl_wait();   // gate/up are cleared by the projection
@@ -617,7 +623,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
       float cs[G][NTM];
       for (int i = 0;; ++i) {
         const int s = i & 1;
-        ok &= mbar_wait(&full[gr][s], (uint32_t)(i >> 1) & 1u);
+        ok &= mbar_wait(&full[gr][s], (uint32_t)(i >> 1) & 1u, x.spin);
         if (!__all_sync(0xFFFFFFFFu, ok)) break;   // a wait ran out: nothing of the stage can be used
         const GInfo& f = infos[gr][s];
         const int flags = f.flags;
@@ -675,7 +681,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
           }
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[gr][s]);
+        if (lane == 0 && !(i == 0 && x.lose && blockIdx.x == 0)) mbar_arrive(&empty[gr][s]);
       }
     }
   }
@@ -940,7 +946,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
       const int s = k & 1, nrb = run_nrb(c), ntk = min(kNT, tb.cnt[c.a] - c.tt * kNT), rb0 = c.rc * RC;
       const int pr = p.pair_list[tb.pst[c.a] + c.tt * kNT + min(lane & 15, ntk - 1)];
       const float pw = hw == 0 ? p.pair_weight[pr] : 0.f;
-      if (k >= 2) ok &= mbar_wait(&hempty[s], (uint32_t)((k >> 1) - 1) & 1u);
+      if (k >= 2) ok &= mbar_wait(&hempty[s], (uint32_t)((k >> 1) - 1) & 1u, x.spin);
       if (!__all_sync(0xFFFFFFFFu, ok)) break;
       uint4* hf = reinterpret_cast<uint4*>(msm + L.hf + s * L.hfs);     // [NTM][RC][8 K-steps][32 lanes]
       float2* hz = reinterpret_cast<float2*>(msm + L.hz + s * L.hzs);   // [RC][G][kNT] (sum of h, 2^(24 - S))
@@ -986,7 +992,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
         }
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&hfull[s]);
+      if (lane == 0 && !(k == 0 && x.lose && blockIdx.x == 0)) mbar_arrive(&hfull[s]);
     }
   } else {
     // ---- consumers
@@ -1064,8 +1070,8 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
           if (lane == 0) mbar_arrive(&hempty[held & 1]);
         }
         ++held;
-        ok &= mbar_wait(&hfull[held & 1], (uint32_t)(held >> 1) & 1u);
-        __syncwarp();
+        ok &= mbar_wait(&hfull[held & 1], (uint32_t)(held >> 1) & 1u, x.spin);
+        if (!__all_sync(0xFFFFFFFFu, ok)) return;
       }
     };
     int cs = 0;
@@ -1089,7 +1095,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
       for (int rb = 0; rb < nrb;) {
         __syncwarp();   // the stage before has been read by every lane
         issue();
-        ok &= mbar_wait(&bars[wid][cs], cph);
+        ok &= mbar_wait(&bars[wid][cs], cph, x.spin);
         live = __all_sync(0xFFFFFFFFu, ok);
         if (!live) break;
         if (rb == 0) bits = tbits[wid][c.ms];
@@ -1106,7 +1112,14 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
           cph ^= 1u;
         }
       }
-      if (!live) break;
+      if (!live) {   // the piece waited for is in flight too
+        mbar_wait(&bars[wid][cs], cph);
+        if (++cs == S) {
+          cs = 0;
+          cph ^= 1u;
+        }
+        break;
+      }
       // s += g alpha out
       const int* un = reinterpret_cast<const int*>(md);
       const float* al = reinterpret_cast<const float*>(md + 128);
@@ -1129,8 +1142,17 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
       __syncwarp();   // the tile's metadata slot may be refilled
       advance(c, nrb);
     }
+    // No block leaves with copies in flight: after a wait that ran out, the pieces requested and not waited for
+    // (fewer than S).
+    while (cs != ps) {
+      mbar_wait(&bars[wid][cs], cph);
+      if (++cs == S) {
+        cs = 0;
+        cph ^= 1u;
+      }
+    }
     // the segments that are left (the cursor has walked to the block's end: ord = their number)
-    if (c.ord > 0) hold(c.ord - 1);
+    if (__all_sync(0xFFFFFFFFu, ok) && c.ord > 0) hold(c.ord - 1);
   }
   if (!ok && lane == 0) atomicCAS(p.status, 0, BITSMOE_ERR_TIMEOUT);
 }

@@ -86,9 +86,9 @@ namespace {
 // bitsmoe_layer's f2_* arrays).
 constexpr int kF2Sizes[5] = {8, 4, 3, 2, 1};
 
-// Testing hook (bitsmoe_debug_wait_limit): bound of the single-token kernels' waits
-// and whether block 0 skips its arrival at their first grid barrier (in the bit allocation's
-// cost kernel: takes a wait of each warp as run out).
+// Testing hook (bitsmoe_debug_wait_limit): bound of the single-token and expert kernels' waits
+// and whether block 0 skips its arrival at the former's first grid barrier (in the expert kernels:
+// at a shared-memory stage; in the bit allocation's cost kernel: takes a wait of each warp as run out).
 std::atomic<long long> g_dbg_spin{0};
 std::atomic<int> g_dbg_skip{0};
 // Testing hook (bitsmoe_debug_single_token_kernel): 1 keeps single-token forwards on the
@@ -1607,6 +1607,8 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
     ma.dst = L->d_dst;
     ma.meta = L->d_meta;
     ma.msa = L->d_msa;
+    ma.spin = g_dbg_spin.load() > 0 ? g_dbg_spin.load() : kWaitClocks;
+    ma.lose = g_dbg_skip.load();
     p.zmax = reinterpret_cast<uint32_t*>(wb + w.zmax);
     if (!p.decode && T > kSplitTokens) p.sb = reinterpret_cast<uint16_t*>(wb + w.sb);
   }

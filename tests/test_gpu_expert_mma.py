@@ -93,6 +93,35 @@ def test_most_pairs(env, E):
         assert err.value.code == bm.ERR_CODE["SHAPE"]
 
 
+@pytest.mark.parametrize("T,E,k,n,I", [(16, 8, 8, 1100, 1152), (600, 2, 2, 1100, 256)])   # tiles of 8 and of 16 tokens
+def test_waits_that_run_out(env, T, E, k, n, I):
+    """Block 0 of both expert kernels leaves out the arrivals at its first stage (testing hook) and every wait inside
+    a block is bounded to about a millisecond: both kernels return after it (their copies in flight waited for), the
+    status word reports TIMEOUT, and the next call on the same workspace is correct."""
+    torch, bm = env
+    spec = synth.scaled_spec(synth.WORKLOADS["tiny"], D=64, E=E, I=I, n=n, group=128, top_k=k)
+    layer = wide_layer(spec, T, {4: 1.0})
+    L = bm.bitsmoe_pack(layer, device=0)
+    assert bm.bitsmoe_forward_plan(L, T, k) & bm.PLAN_TC_GATE_UP
+    x, logits = synth.make_inputs(spec, T, seed=T)
+    xd, ld = torch.from_numpy(x.view(np.int16)).cuda(), torch.from_numpy(logits).cuda()
+    ws = bm.Workspace(L, T, k)
+    y = torch.empty((T, spec.D), dtype=torch.float32, device="cuda")
+    clocks = 2_000_000
+    bm.bitsmoe_debug_wait_limit(1, clocks)
+    try:
+        ms = bm.bitsmoe_profile_forward(xd.data_ptr(), ld.data_ptr(), T, k, L, y.data_ptr(), ws.ptr, ws.nbytes,
+                                        torch.cuda.current_stream().cuda_stream)
+    finally:
+        bm.bitsmoe_debug_wait_limit(0, 0)
+    assert 0.4 * clocks / 1e6 < min(ms[2:4]) and max(ms[2:4]) < 500, ms   # gate/up and down (SM clock up to 2.1 GHz)
+    assert bm.bitsmoe_last_device_status(ws.ptr) == bm.ERR_CODE["TIMEOUT"]
+    y = bm.moe_forward(L, xd, ld, k, ws=ws)
+    assert bm.bitsmoe_last_device_status(ws.ptr) == 0
+    ref = oracle.moe_forward_factored(layer, x, logits, k)
+    assert np.max(np.abs(y.cpu().numpy() - ref)) <= TOL * np.max(np.abs(ref))
+
+
 def wide_layer(spec, seed, bits):
     """A layer with more units than features (n > D): random bases of norm-1 columns."""
     layer = synth.make_layer(synth.scaled_spec(spec, D=spec.n), seed=seed, bits_dist=bits, alpha_scale=4.0,
