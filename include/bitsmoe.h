@@ -172,8 +172,8 @@ int bitsmoe_forward_launches(const bitsmoe_layer* layer, int T, int top_k);
 int bitsmoe_forward_plan(const bitsmoe_layer* layer, int T, int top_k);
 
 /* Testing hook (no counterpart in the paper): bound every wait of the fused
- * single-token kernels, and the waits inside a block of the expert kernels of
- * several tokens, to `spin_clocks` SM clocks (<= 0: the default, about one
+ * single-token kernels, and the waits inside a block of the tensor-core
+ * projections and the expert kernels of several tokens, to `spin_clocks` SM clocks (<= 0: the default, about one
  * second), and when skip_arrival is 1 let block 0 skip an arrival (the former:
  * at their first grid barrier, the latter: at a stage in shared memory), so that
  * the bounded waits for it run out.  The calls after it report

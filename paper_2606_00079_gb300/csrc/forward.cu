@@ -86,9 +86,9 @@ namespace {
 // bitsmoe_layer's f2_* arrays).
 constexpr int kF2Sizes[5] = {8, 4, 3, 2, 1};
 
-// Testing hook (bitsmoe_debug_wait_limit): bound of the single-token and expert kernels' waits
-// and whether block 0 skips its arrival at the former's first grid barrier (in the expert kernels:
-// at a shared-memory stage; in the bit allocation's cost kernel: takes a wait of each warp as run out).
+// Testing hook (bitsmoe_debug_wait_limit): bound of the single-token kernels', the tensor-core
+// projections' and the expert kernels' waits, and whether block 0 skips its arrival at the first ones'
+// first grid barrier (in the others: at a shared-memory stage; in the bit allocation's cost kernel: takes a wait of each warp as run out).
 std::atomic<long long> g_dbg_spin{0};
 std::atomic<int> g_dbg_skip{0};
 // Testing hook (bitsmoe_debug_single_token_kernel): 1 keeps single-token forwards on the
@@ -1910,6 +1910,7 @@ int noalloc_scratch(int device, cudaStream_t st, void** out) {
 namespace bmoe {
 int record_cuda_error(int cuda_error) { return cuda_fail(static_cast<cudaError_t>(cuda_error)); }
 int debug_skip_arrival() { return g_dbg_skip.load(); }
+long long debug_wait_clocks() { return g_dbg_spin.load(); }
 }  // namespace bmoe
 
 extern "C" {

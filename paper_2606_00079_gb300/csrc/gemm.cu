@@ -78,6 +78,8 @@ struct GemmArgs {
   float* y;          // mode 1: [T][D]
   float4* zero;      // null, or a buffer of later kernels to clear
   size_t zero_n;     // its length in float4
+  long long spin;    // bound of the waits, in SM clocks
+  int lose;          // testing hook: the first CTA's ring never reports its first slot free
   int* status;
 };
 
@@ -86,7 +88,9 @@ struct GemmArgs {
 // the activations (B) into the same ring, warp 1 issues tcgen05.mma; then warps 2-5
 // read the fp32 partial tile out of TMEM into shared memory, and the cluster's CTAs
 // add the partials of their share of the rows through distributed shared memory
-// and store the result (no atomics, nothing to clear beforehand).
+// and store the result (no atomics, nothing to clear beforehand).  A warp whose wait runs
+// out stops its part: the tile is then wrong and the status word says TIMEOUT, but no slot
+// is filled again under a pending copy or product, and no CTA leaves with copies in flight.
 __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant__ CUtensorMap amap,
                                                           const __grid_constant__ CUtensorMap bmap, GemmArgs g) {
   extern __shared__ uint8_t gsm_raw[];
@@ -147,14 +151,20 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
         if (g.mode == 1) pdl_wait();   // the split of s; x comes from kernels before the router
         for (int i = 0; i < pre; ++i) load_b(i, i);
       }
-      for (int i = pre, st = 0, u = 1; i < nk; ++i) {
-        ok &= mbar_wait(empty + st, (uint32_t)(u - 1) & 1u);
+      int i = pre;
+      for (int st = 0, u = 1; i < nk; ++i) {
+        ok = mbar_wait(empty + st, (uint32_t)(u - 1) & 1u, g.spin);
+        if (!ok) break;
         load_a(i, st);
         if (g.btma) load_b(i, st);
         if (++st == S) {
           st = 0;
           ++u;
         }
+      }
+      for (int j = max(0, i - S); j < i; ++j) {   // the copies that may still be in flight
+        mbar_wait(full_a + j % S, (uint32_t)(j / S) & 1u);
+        if (g.btma) mbar_wait(full_b + j % S, (uint32_t)(j / S) & 1u);
       }
     }
   } else if (wid == 1) {
@@ -164,8 +174,8 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
       const uint64_t da = sw128_desc(smem_u32(gsm)), db = sw128_desc(smem_u32(gsm) + kATile);
       const uint32_t sstep = g.stage >> 4, lstep = b_bytes >> 4;
       for (int i = 0, st = 0, u = 0; i < nk; ++i) {
-        ok &= mbar_wait(full_a + st, (uint32_t)u & 1u);
-        ok &= mbar_wait(full_b + st, (uint32_t)u & 1u);
+        ok = mbar_wait(full_a + st, (uint32_t)u & 1u, g.spin) && mbar_wait(full_b + st, (uint32_t)u & 1u, g.spin);
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t a0 = da + (uint64_t)st * sstep, b0 = db + (uint64_t)st * sstep;
 #pragma unroll
@@ -175,7 +185,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
           for (int k16 = 0; k16 < kKB / 16; ++k16)
             mma_f16(tmem + (uint32_t)g.N, a0 + 2 * k16, b0 + lstep + 2 * k16, idesc, (i | k16) != 0);
         }
-        mma_commit(empty + st);
+        if (!(g.lose && i == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0)) mma_commit(empty + st);
         if (++st == S) {
           st = 0;
           ++u;
@@ -242,7 +252,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
     float4 vc[4][2], vn[4][2];
     load4(0, vc);
     int sb = 0, ub = 0;   // ring slot and use of the batch's first K-block
-    for (int f0 = 0; f0 < nf; f0 += 4 * kStagers) {
+    for (int f0 = 0; f0 < nf && ok; f0 += 4 * kStagers) {
       if (f0 + 4 * kStagers < nf) load4(f0 + 4 * kStagers, vn);
       const int ib = f0 >> lg;
 #pragma unroll
@@ -251,13 +261,15 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
         if (i >= nk) continue;   // (uniform in a warp: a K-block has a multiple of 32 chunks)
         const int st0 = sb + i - ib, st = st0 >= S ? st0 - S : st0, u = st0 >= S ? ub + 1 : ub;
         if (u > 0) {   // the ring slot: its previous MMAs must be done
-          if (lane == 0) ok &= mbar_wait(empty + st, (uint32_t)(u - 1) & 1u);
-          __syncwarp();
+          if (lane == 0) ok = mbar_wait(empty + st, (uint32_t)(u - 1) & 1u, g.spin);
+          ok = __all_sync(0xFFFFFFFFu, ok);
+          if (!ok) break;
         }
         if (c < nch) store1(gsm + (size_t)st * g.stage + kATile, c, vc[q]);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> tensor-core reads
       __syncwarp();
+      if (!ok) break;
       const int in = (f0 + 4 * kStagers) >> lg;   // K-blocks that this batch completes: ib .. in - 1
       for (int i = ib; i < in; ++i) {
         if (lane == 0 && i < nk) mbar_arrive(full_b + sb);
@@ -281,7 +293,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_gemm_tc(const __grid_constant_
     }
     if (wid < 6) {
     // partial tile out of TMEM: warp w holds accumulator lanes (rows) 32 (w % 4) ..
-    if (lane == 0) ok &= mbar_wait(done, 0);
+    if (lane == 0) ok &= mbar_wait(done, 0, g.spin);
     __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const int r = 32 * (wid & 3) + lane;
@@ -452,6 +464,8 @@ cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cud
   g.zero = static_cast<float4*>(zero);
   g.zero_n = zero_bytes / 16;
   g.y = p.y;
+  g.spin = debug_wait_clocks() > 0 ? debug_wait_clocks() : kWaitClocks;
+  g.lose = debug_skip_arrival();
   g.status = p.status;
   CUtensorMap amap, bmap;
   std::memcpy(&amap, map, sizeof(amap));

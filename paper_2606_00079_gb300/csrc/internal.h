@@ -30,8 +30,9 @@ inline const ExpertDesc* desc_of(const uint8_t* img) {
 // thread) and return BITSMOE_ERR_CUDA.
 int record_cuda_error(int cuda_error);
 
-// Testing hook (bitsmoe_debug_wait_limit): whether a skipped arrival is asked for.
+// Testing hook (bitsmoe_debug_wait_limit): whether a skipped arrival is asked for, and the waits' bound (0: default).
 int debug_skip_arrival();
+long long debug_wait_clocks();
 
 // Supported quantisation groups and their checks.
 inline bool group_ok(int g) { return g == 32 || g == 64 || g == 128 || g == 256; }

@@ -122,6 +122,34 @@ def test_waits_that_run_out(env, T, E, k, n, I):
     assert np.max(np.abs(y.cpu().numpy() - ref)) <= TOL * np.max(np.abs(ref))
 
 
+@pytest.mark.parametrize("D", [4096, 4098])   # tokens copied by TMA, and staged by warps
+def test_projection_waits_that_run_out(env, D):
+    """The first CTA of the tensor-core projection never reports its first ring slot free (testing hook): the kernel
+    returns within the bounds of its waits, the status word reports TIMEOUT, and the next call is correct."""
+    torch, bm = env
+    T = 256
+    spec = synth.scaled_spec(synth.WORKLOADS["tiny"], D=D, E=2, I=64, n=64, group=64, top_k=1)
+    layer = synth.make_layer(spec, seed=D, bits_dist=BITS, alpha_scale=4.0, basis_method="householder")
+    L = bm.bitsmoe_pack(layer, device=0)
+    x, logits = synth.make_inputs(spec, T, seed=D)
+    xd, ld = torch.from_numpy(x.view(np.int16)).cuda(), torch.from_numpy(logits).cuda()
+    ws = bm.Workspace(L, T, 1)
+    y = torch.empty((T, D), dtype=torch.float32, device="cuda")
+    clocks = 2_000_000
+    bm.bitsmoe_debug_wait_limit(1, clocks)
+    try:
+        ms = bm.bitsmoe_profile_forward(xd.data_ptr(), ld.data_ptr(), T, 1, L, y.data_ptr(), ws.ptr, ws.nbytes,
+                                        torch.cuda.current_stream().cuda_stream)
+    finally:
+        bm.bitsmoe_debug_wait_limit(0, 0)
+    assert 0.4 * clocks / 1e6 < ms[1] < 500, ms
+    assert bm.bitsmoe_last_device_status(ws.ptr) == bm.ERR_CODE["TIMEOUT"]
+    y = bm.moe_forward(L, xd, ld, 1, ws=ws)
+    assert bm.bitsmoe_last_device_status(ws.ptr) == 0
+    ref = oracle.moe_forward_factored(layer, x, logits, 1)
+    assert np.max(np.abs(y.cpu().numpy() - ref)) <= TOL * np.max(np.abs(ref))
+
+
 def wide_layer(spec, seed, bits):
     """A layer with more units than features (n > D): random bases of norm-1 columns."""
     layer = synth.make_layer(synth.scaled_spec(spec, D=spec.n), seed=seed, bits_dist=bits, alpha_scale=4.0,
