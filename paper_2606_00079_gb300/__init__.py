@@ -524,7 +524,8 @@ def bitsmoe_debug_single_token_kernel(which: int) -> None:
 
 def bitsmoe_debug_bounds(on: int) -> None:
     """Testing hook: debug bounds checks of the single-token kernels' staging records (and a
-    zero-filled slack after the image of layers packed while it is on)."""
+    zero-filled slack after the image of layers packed while it is on); 2: also an impossible
+    count in the routing that the expert kernels of several tokens check."""
     _check(_lib().bitsmoe_debug_bounds(on), "bitsmoe_debug_bounds")
 
 

@@ -64,7 +64,8 @@ struct MArgs {
   const uint8_t* meta;    // the records' slot metadata (mirror of the image's)
   const float* msa;       // [2][E] max over groups and slots of |scale * alpha| of gate/up (h, e)
   long long spin;         // bound of the waits inside a block, in SM clocks
-  int lose;               // testing hook: an arrival of block 0 is left out, so that waits of its warps run out
+  int lose;               // testing hooks: bit 0: an arrival of block 0 is left out, so that waits of its warps run out;
+                          // bit 1: the first expert's count is taken as T more than it is
 };
 
 // Staging records of the fused single-token kernel, derived from the image

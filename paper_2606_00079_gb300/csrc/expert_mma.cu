@@ -68,20 +68,32 @@ __device__ MTiles mtiles_at(uint8_t* sm, int A_max) {
 // 8 tokens, the operand and the products are not).
 __device__ __forceinline__ int tile_weight(int nt) { return 1 + ((nt + 7) >> 3); }
 
-// Whole block; the routing is published.  per_tile(e): units of a token tile of expert e.
+// Whole block; the routing is published.  per_tile(e): units of a token tile of expert e.  An expert, a count or a
+// list outside the call's (another call on the same workspace, or a workspace that was not zero-filled) gets no
+// units, and the status word says so.  (An early return instead cost the down kernel spills in its consumers.)
 template <class F>
-__device__ void mtiles_build(const Fwd& p, int A_max, int NT, MTiles& t, F per_tile) {
+__device__ void mtiles_build(const Fwd& p, int A_max, int lose, int NT, MTiles& t, F per_tile) {
   const int tid = threadIdx.x, lane = tid & 31;
-  t.na = min(p.active[0], A_max);
+  const int na = p.active[0];
+  bool bad = na < 0 || na > A_max;
+  t.na = bad ? 0 : na;
   for (int a = tid; a < t.na; a += (int)blockDim.x) {
-    const int e = p.active[1 + a], c = p.expert_count[e];
+    const int e = p.active[1 + a];
+    const bool in = e >= 0 && e < p.E;
+    const int c = in ? p.expert_count[e] + ((lose & 2) && a == 0 ? p.T : 0) : 0, start = in ? p.expert_start[e] : 0;
+    if (c < 1 || c > p.T || start < 0 || start > p.P - c) {
+      bad = true;
+      t.ub[a] = t.wb[a] = t.cnt[a] = 0;
+      continue;
+    }
     t.e[a] = e;
     t.cnt[a] = c;
-    t.pst[a] = p.expert_start[e];
+    t.pst[a] = start;
     const int m = per_tile(e), f = c / NT, r = c - f * NT;
     t.ub[a] = (f + (r > 0)) * m;
     t.wb[a] = (f * tile_weight(NT) + (r > 0 ? tile_weight(r) : 0)) * m;
   }
+  if (bad) atomicCAS(p.status, 0, BITSMOE_ERR_WORKSPACE_STATE);
   __syncthreads();
   if (tid < 32) {   // exclusive prefixes
     int ru = 0, rw = 0;
@@ -420,7 +432,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
     return;
   }
   const int nrg = (p.NRB + R - 1) / R, M = 2 * nrg * p.nseg;
-  mtiles_build(p, x.A_max, kNT, tb, [&](int) { return M; });
+  mtiles_build(p, x.A_max, x.lose, kNT, tb, [&](int) { return M; });
   bool ok = true;
 
   if (wid >= kCW) {
@@ -681,7 +693,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
           }
         }
         __syncwarp();
-        if (lane == 0 && !(i == 0 && x.lose && blockIdx.x == 0)) mbar_arrive(&empty[gr][s]);
+        if (lane == 0 && !(i == 0 && (x.lose & 1) && blockIdx.x == 0)) mbar_arrive(&empty[gr][s]);
       }
     }
   }
@@ -917,7 +929,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
     pdl_wait();
     return;
   }
-  mtiles_build(p, x.A_max, kNT, tb, [&](int e) { return nrc * __ldg(&dd[e].ntiles); });
+  mtiles_build(p, x.A_max, x.lose, kNT, tb, [&](int e) { return nrc * __ldg(&dd[e].ntiles); });
   const int lo = cut_unit(tb, kNT, (int)blockIdx.x, (int)gridDim.x);
   const int hi = cut_unit(tb, kNT, (int)blockIdx.x + 1, (int)gridDim.x);
   bool ok = true;
@@ -992,7 +1004,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
         }
       }
       __syncwarp();
-      if (lane == 0 && !(k == 0 && x.lose && blockIdx.x == 0)) mbar_arrive(&hfull[s]);
+      if (lane == 0 && !(k == 0 && (x.lose & 1) && blockIdx.x == 0)) mbar_arrive(&hfull[s]);
     }
   } else {
     // ---- consumers

@@ -96,7 +96,8 @@ std::atomic<int> g_dbg_skip{0};
 std::atomic<int> g_dbg_kernel{0};
 // testing hook: debug bounds checks in the single-token kernels; layers uploaded while it is
 // on get a zero-filled slack of the image's own size after it (so that a record shifted past
-// the image, as the tests do, still reads mapped memory)
+// the image, as the tests do, still reads mapped memory); 2: the expert kernels of several tokens
+// also find a wrong count in the routing, which their check must refuse
 std::atomic<int> g_dbg_bounds{0};
 
 thread_local int g_last_cuda = 0;
@@ -1608,7 +1609,7 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
     ma.meta = L->d_meta;
     ma.msa = L->d_msa;
     ma.spin = g_dbg_spin.load() > 0 ? g_dbg_spin.load() : kWaitClocks;
-    ma.lose = g_dbg_skip.load();
+    ma.lose = g_dbg_skip.load() | (g_dbg_bounds.load() == 2 ? 2 : 0);
     p.zmax = reinterpret_cast<uint32_t*>(wb + w.zmax);
     if (!p.decode && T > kSplitTokens) p.sb = reinterpret_cast<uint16_t*>(wb + w.sb);
   }
@@ -2230,7 +2231,7 @@ int bitsmoe_debug_wait_limit(int skip_arrival, long long spin_clocks) {
 }
 
 int bitsmoe_debug_bounds(int on) {
-  g_dbg_bounds.store(on ? 1 : 0);
+  g_dbg_bounds.store(on == 2 ? 2 : on ? 1 : 0);
   return BITSMOE_OK;
 }
 

@@ -150,6 +150,29 @@ def test_projection_waits_that_run_out(env, D):
     assert np.max(np.abs(y.cpu().numpy() - ref)) <= TOL * np.max(np.abs(ref))
 
 
+@pytest.mark.parametrize("T", [8, 40])
+def test_impossible_routing_is_refused(env, T):
+    """A routing whose first expert holds more tokens than the call has (testing hook) is left out and reported as
+    WORKSPACE_STATE; the next call on the same workspace is correct."""
+    torch, bm = env
+    spec = synth.scaled_spec(synth.WORKLOADS["tiny"], D=128, E=8, I=256, n=96, group=128, top_k=3)
+    layer = synth.make_layer(spec, seed=T, bits_dist=BITS, alpha_scale=4.0)
+    L = bm.bitsmoe_pack(layer, device=0)
+    x, logits = synth.make_inputs(spec, T, seed=T)
+    xd, ld = torch.from_numpy(x.view(np.int16)).cuda(), torch.from_numpy(logits).cuda()
+    ws = bm.Workspace(L, T, spec.top_k)
+    bm.bitsmoe_debug_bounds(2)
+    try:
+        bm.moe_forward(L, xd, ld, spec.top_k, ws=ws)
+        assert bm.bitsmoe_last_device_status(ws.ptr) == bm.ERR_CODE["WORKSPACE_STATE"]
+    finally:
+        bm.bitsmoe_debug_bounds(0)
+    y = bm.moe_forward(L, xd, ld, spec.top_k, ws=ws)
+    assert bm.bitsmoe_last_device_status(ws.ptr) == 0
+    ref = oracle.moe_forward_factored(layer, x, logits, spec.top_k)
+    assert np.max(np.abs(y.cpu().numpy() - ref)) <= TOL * np.max(np.abs(ref))
+
+
 def wide_layer(spec, seed, bits):
     """A layer with more units than features (n > D): random bases of norm-1 columns."""
     layer = synth.make_layer(synth.scaled_spec(spec, D=spec.n), seed=seed, bits_dist=bits, alpha_scale=4.0,
