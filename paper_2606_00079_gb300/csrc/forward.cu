@@ -1385,29 +1385,23 @@ int launch_router(const Fwd& p, cudaStream_t st) {
   return launch(k_router, dim3((p.T + kRouteWarps - 1) / kRouteWarps), dim3(kRouteWarps * 32), smem, st, false, p);
 }
 
-// parts: 1 the gate/up kernel, 2 the down kernel, 3 both
+// The dp2a gate/up and down kernels (between: called between their launches).
 template <int G, int TB>
-int launch_k2k3_dec(const Fwd& p, int A_max, int sms, cudaStream_t st, bool pdl,
-                    const std::function<int()>& between, int parts = 3) {
+int launch_k2k3_dec(const Fwd& p, int A_max, cudaStream_t st, bool pdl, const std::function<int()>& between) {
   int rc;
-  const size_t rbytes = 0;
-  if (parts & 1) {
-    const size_t smax = (size_t)p.s16 - 8;
-    const size_t pw2 = (size_t)p.seg_bytes + smax * 4 * (2 + G) + (size_t)G * TB * p.s16 * 2 + 16;
-    const size_t sm2 = rbytes + kK2DecWarps * pw2;
-    const int items2 = A_max * 2 * p.NRB * p.nseg;
-    if ((rc = set_smem(k_gateup_dec<G, TB>, sm2))) return rc;
-    if ((rc = launch(k_gateup_dec<G, TB>, dim3((items2 + kK2DecWarps - 1) / kK2DecWarps), dim3(kK2DecWarps * 32),
-                     sm2, st, pdl, p)))
-      return rc;
-  }
+  const size_t smax = (size_t)p.s16 - 8;
+  const size_t pw2 = (size_t)p.seg_bytes + smax * 4 * (2 + G) + (size_t)G * TB * p.s16 * 2 + 16;
+  const size_t sm2 = kK2DecWarps * pw2;
+  const int items2 = A_max * 2 * p.NRB * p.nseg;
+  if ((rc = set_smem(k_gateup_dec<G, TB>, sm2))) return rc;
+  if ((rc = launch(k_gateup_dec<G, TB>, dim3((items2 + kK2DecWarps - 1) / kK2DecWarps), dim3(kK2DecWarps * 32),
+                   sm2, st, pdl, p)))
+    return rc;
   if (between && (rc = between())) return rc;
-  if (!(parts & 2)) return BITSMOE_OK;
   const size_t nrm = (size_t)p.rbc * kRows;
   const int ngc_max = std::max(1, (int)(nrm / p.group));
   const size_t pw3 = (size_t)p.ul_bytes + (size_t)ngc_max * 32 * 4 + 16;
-  const size_t sm3 = rbytes + TB * nrm * 6 + TB * 64 * 4 + kK3DecWarps * TB * 4 + ((TB + 3) & ~3) * 4 +
-                     kK3DecWarps * pw3;
+  const size_t sm3 = TB * nrm * 6 + TB * 64 * 4 + kK3DecWarps * TB * 4 + ((TB + 3) & ~3) * 4 + kK3DecWarps * pw3;
   const int ntg = (p.ul_max_tiles + kK3DecWarps - 1) / kK3DecWarps;
   const int nrc = (p.NRB + p.rbc - 1) / p.rbc;
   if ((rc = set_smem(k_down_dec<G, TB>, sm3))) return rc;
@@ -1676,13 +1670,13 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
       if ((rc = mark(3))) return rc;
       BM_CK(launch_expert_mma(true, p, ma, sms, st, pdl));
     } else if (T == 1) {
-      if (G == 1) rc = launch_k2k3_dec<1, 1>(p, A_max, sms, st, pdl, between);
-      else if (G == 2) rc = launch_k2k3_dec<2, 1>(p, A_max, sms, st, pdl, between);
-      else rc = launch_k2k3_dec<4, 1>(p, A_max, sms, st, pdl, between);
+      if (G == 1) rc = launch_k2k3_dec<1, 1>(p, A_max, st, pdl, between);
+      else if (G == 2) rc = launch_k2k3_dec<2, 1>(p, A_max, st, pdl, between);
+      else rc = launch_k2k3_dec<4, 1>(p, A_max, st, pdl, between);
     } else {
-      if (G == 1) rc = launch_k2k3_dec<1, 4>(p, A_max, sms, st, pdl, between);
-      else if (G == 2) rc = launch_k2k3_dec<2, 4>(p, A_max, sms, st, pdl, between);
-      else rc = launch_k2k3_dec<4, 4>(p, A_max, sms, st, pdl, between);
+      if (G == 1) rc = launch_k2k3_dec<1, 4>(p, A_max, st, pdl, between);
+      else if (G == 2) rc = launch_k2k3_dec<2, 4>(p, A_max, st, pdl, between);
+      else rc = launch_k2k3_dec<4, 4>(p, A_max, st, pdl, between);
     }
     if (rc) return rc;
     if ((rc = mark(4))) return rc;
@@ -1717,9 +1711,9 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
     if ((rc = mark(2))) return rc;
     // gate/up factors (the staged dp2a kernel over batches of 4 tokens), then down
     std::function<int()> between = ev ? std::function<int()>([&]() { return mark(3); }) : std::function<int()>();
-    if (G == 1) rc = launch_k2k3_dec<1, 4>(p, A_max, sms, st, pdl, between);
-    else if (G == 2) rc = launch_k2k3_dec<2, 4>(p, A_max, sms, st, pdl, between);
-    else rc = launch_k2k3_dec<4, 4>(p, A_max, sms, st, pdl, between);
+    if (G == 1) rc = launch_k2k3_dec<1, 4>(p, A_max, st, pdl, between);
+    else if (G == 2) rc = launch_k2k3_dec<2, 4>(p, A_max, st, pdl, between);
+    else rc = launch_k2k3_dec<4, 4>(p, A_max, st, pdl, between);
   }
   if (rc) return rc;
   if ((rc = mark(4))) return rc;
