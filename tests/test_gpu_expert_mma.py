@@ -1,8 +1,9 @@
 """GPU parity of the multi-token expert factors (mma.sync tiles of 8 and 16 tokens) at the sizes where
 their tiling can go wrong: expert loads around a token group (1, 7, 8, 9, 15 .. 17, 33), one and several
 row blocks and runs of row blocks, several segments, K-step remainders of every bit-width, odd expert
-counts, all scale groups, and both sides of the decode batch (operand gathered in the kernel or by its
-own launch).
+counts, all scale groups, and both sides of the decode batch and of the 256 tokens past which the down
+kernel takes longer runs of row blocks.  Also the largest routing, waits that run out, and a routing
+that is not the call's.
 
 Tolerance: the operands are fp16 pairs (at least 21 bits) and the codes exact, so what remains is fp32
 summation over at most n + I terms and the output basis' bf16 pair (2^-17 of each term of s): below
@@ -45,6 +46,10 @@ def env():
     (34, 2, 2, 256, 1100, 256, 128, {1: 1.0}),  # several segments of one bit-width
     (34, 2, 2, 64, 1030, 128, 128, {3: .5, 4: .5}),
     (40, 2, 1, 64, 515, 256, 32, {6: .5, 8: .5}),
+    (257, 5, 2, 64, 75, 768, 128, BITS),        # past 256 tokens: one run of six row blocks, a ring of two stages
+    (257, 3, 2, 64, 75, 1152, 128, BITS),       # runs of five and four row blocks
+    (257, 3, 2, 64, 75, 1280, 256, BITS),       # runs of six and four, groups of two row blocks
+    (300, 3, 2, 64, 75, 768, 32, BITS),         # runs of four and two, four groups a row block
 ])
 def test_expert_tiles(env, T, E, k, D, n, I, group, bits):
     torch, bm = env
@@ -55,6 +60,9 @@ def test_expert_tiles(env, T, E, k, D, n, I, group, bits):
     plan = bm.bitsmoe_forward_plan(L, T, k)
     assert plan == (bm.PLAN_DECODE_CHAIN | bm.PLAN_TC_PROJECTIONS if T <= 8 else
                     bm.PLAN_TC_PROJECTIONS | bm.PLAN_TC_GATE_UP | bm.PLAN_TC_DOWN)
+    # The plan of the decode batch does not name its expert kernels.  They are these whenever 16 tokens take them:
+    # the same layer and tiles of 8 tokens, and a shared-memory plan that grows with the routed experts alone.
+    assert bm.bitsmoe_forward_plan(L, max(T, 16), k) & bm.PLAN_TC_GATE_UP
     x, logits = synth.make_inputs(spec, T, seed=T)
     # uneven loads: the first experts hold 1, 7, 8, 9, .. of the first choices
     e, t = 0, 0

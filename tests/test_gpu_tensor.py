@@ -1,6 +1,7 @@
 """GPU parity of the multi-token path (T > 8): multi-block router, tensor-core
-projections (tcgen05, split-K), staged gate/up and down kernels with token
-batches, against the fp64 oracle.
+projections (tcgen05, split-K), tensor-core gate/up and down kernels over token
+tiles (mma.sync; dp2a kernels with token batches on layers with 16-bit units),
+against the fp64 oracle.
 
 Covers token counts at and around the MMA granularity (16), a count whose
 tokens span two launches of the projections (more than 256), ragged D and n
@@ -63,13 +64,13 @@ TC_BITS = {0: 0.1, 1: 0.15, 2: 0.2, 3: 0.15, 4: 0.15, 6: 0.15, 8: 0.1}
     (9, 8, 3, 100, 75, 256, 128),     # ragged n: the last K-block is partly padding
     (33, 8, 2, 256, 200, 384, 128),   # several slot ranges per block, three row blocks
     (130, 4, 2, 96, 72, 512, 256),    # group of two row blocks
-    (600, 4, 2, 64, 40, 256, 128),    # experts with more than 256 tokens: two token tiles
+    (600, 4, 2, 64, 40, 256, 128),    # experts with more than 256 tokens
 ])
 def test_tensor_expert_factors(env, T, E, k, D, n, I, group):
-    """Gate/up and down factors on tcgen05 (codes as fp16 bit patterns, decoded once per
-    row block; gate/up: scale * alpha * z as an fp16 pair with SiLU(gate) * up in the
-    epilogue; down: h as an fp16 pair, group scales applied to the per-row-block partial
-    sums): every bit-width below 16, token tiles split at 32 tokens."""
+    """Gate/up and down factors on mma.sync (codes as fp16 bit patterns, decoded once per
+    token tile; gate/up: scale * alpha * z as an fp16 pair, partial rows added in fp32;
+    down: h = SiLU(gate) * up as an fp16 pair, group scales applied to the per-group sums):
+    every bit-width below 16, tiles of 8 (up to 16 tokens) and of 16 tokens."""
     torch, bm = env
     spec = synth.scaled_spec(synth.WORKLOADS["tiny"], D=D, E=E, I=I, n=n, group=group, top_k=k)
     layer = synth.make_layer(spec, seed=T + n, bits_dist=TC_BITS, alpha_scale=4.0)
