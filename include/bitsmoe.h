@@ -160,7 +160,8 @@ int bitsmoe_forward_launches(const bitsmoe_layer* layer, int T, int top_k);
  *   8  past 8 tokens: tensor-core gate/up factors (mma.sync over tiles of 8 or
  *      16 tokens, the codes entering the products as fp16 bit patterns), for
  *      every layer without 16-bit units; the others use the dp2a kernels.  The
- *      decode chain takes the same kernels wherever it has bit 4.
+ *      decode chain does not report bits 8 and 16; where it has bit 4 it takes
+ *      the same kernels on the same layers.
  *  16  tensor-core down factor (always set with 8)
  *  32  with 1: the fused kernel is the clustered one, in which a thread-block
  *      cluster owns one (routing slot, 128-row block) pair of the token and
@@ -173,10 +174,11 @@ int bitsmoe_forward_plan(const bitsmoe_layer* layer, int T, int top_k);
 
 /* Testing hook (no counterpart in the paper): bound every wait of the fused
  * single-token kernels, and the waits inside a block of the tensor-core
- * projections and the expert kernels of several tokens, to `spin_clocks` SM clocks (<= 0: the default, about one
- * second), and when skip_arrival is 1 let block 0 skip an arrival (the former:
- * at their first grid barrier, the latter: at a stage in shared memory), so that
- * the bounded waits for it run out.  The calls after it report
+ * projections and the expert kernels of several tokens, to `spin_clocks` SM
+ * clocks (<= 0: the default, about one second), and when skip_arrival is 1 let
+ * block 0 skip an arrival (the former: at their first grid barrier, the latter:
+ * at a stage in shared memory), so that the bounded waits for it run out.  The
+ * calls after it report
  * BITSMOE_ERR_TIMEOUT through the device status word and return; the workspace
  * is left ready for the next call.  With skip_arrival = 1 the bit allocation's
  * cost kernel also takes one wait of each warp of its block 0 as run out (it

@@ -1,7 +1,6 @@
-// Device-side pieces shared by the kernels of the forward (forward.cu) and
-// the fused decode kernel (fused.cu): the argument block, PTX wrappers, the
-// block-level router and the integer dot-product helpers of the two packed
-// layouts.  Included by CUDA translation units only.
+// Device-side pieces shared by the kernels: the forward's argument blocks and
+// staging records, PTX wrappers, and the integer dot-product helpers of the two
+// packed layouts.  Included by CUDA translation units only.
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -214,9 +213,9 @@ bool fused_plan(const ImageHeader& hd, int T, int top_k, int seg_bytes, int ul_m
 cudaError_t launch_fused(const Fwd& p, const FusedArgs& f, int sms, cudaStream_t st, bool pdl);
 constexpr int kSplitTokens = 64;
 // Tensor-core projections (gemm.cu): a TMA map of a bf16 basis [rows][cols_pad]
-// (128 bytes, written to map_out), and the launch of z += Phi^T x (mode 0) or
-// y += Phi_dn s (mode 1) for all T tokens of p (z, resp. y, zeroed before
-// unless y carries a residual).
+// (128 bytes, written to map_out), and the launch of z = Phi^T x (mode 0) or of
+// y = Phi_dn s (mode 1; y += when p.accum) for all T tokens of p.  Mode 0 also
+// clears `zero` and takes max |z| per token into zmax (cleared by the router).
 bool make_basis_map(void* map_out, const void* base, int rows, int cols_pad);
 cudaError_t launch_gemm_tc(int mode, const void* map, const Fwd& p, int sms, cudaStream_t st, bool pdl,
                            void* zero = nullptr, size_t zero_bytes = 0, uint32_t* zmax = nullptr);

@@ -1219,7 +1219,11 @@ bool mma_args(const ImageHeader& hd, int T, int k, const uint32_t (&stages)[2][k
   // A down run: whole groups; at most 4 row blocks, so that the two h slots leave room for three stages a
   // consumer and that a block's 12 consumers have several items each (one of 13 items of a whole expert's rows,
   // 8 us each, doubled the 8-token call's time); up to 8 past 256 tokens, where the additions into s, one
-  // sector each, weigh more (1024 tokens: 334 us with runs of 3, 262 us with 6).
+  // sector each, weigh more (1024 tokens: 334 us with runs of 3, 262 us with 6).  Whole calls on both sides of the
+  // lines, us with 3 and 2 runs of at most 4 row blocks and with one run of up to 8 (Qwen3-shaped layer, uneven
+  // experts, 6 row blocks): 9 tokens 68 / 70 / 71, 16 77 / 80 / 83, 17 85 / 87 / 92, 48 115 / 118 / 129, 192
+  // 226 / 222 / 228, 256 281 / 275 / 275, 257 289 / 283 / 280, 400 396 / 392 / 375, 1024 879 / 875 / 808; even
+  // experts, 64 tokens 158 / 154 / 156, 256 271 / 265 / 263, 512 441 / 431 / 412.
   const int need = std::max(1, hd.group / kRows), most = T > 256 ? 8 : 4;
   const int runs = std::max((hd.NRB + most - 1) / most, T <= 16 ? 3 : T <= 256 ? 2 : 1), rows = (hd.NRB + runs - 1) / runs;
   const int rc0 = std::max(need, (rows + need - 1) / need * need);

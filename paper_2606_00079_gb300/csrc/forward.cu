@@ -9,18 +9,24 @@
 // dependent launch (PDL) so that a kernel's prologue overlaps the tail of the
 // previous one:
 //
-//   one token      k_fused (fused.cu): the whole layer in one persistent kernel
-//   2 .. 8 tokens  k_route_publish   routing by one block, published with a flag
-//                  k_gemv_bulk<P>    z_g = Phi_g^T x, z_u = Phi_u^T x (rows through
-//                                    a bulk-copy ring); zeroes the accumulators
-//                  k_gateup_dec      gate/up = P_hat (alpha * z): dp2a over
+//   one token      k_fused (fused.cu): the whole layer in one persistent kernel; a
+//                  few tokens (few_tokens_fused) as one such kernel each
+//   up to 8 tokens k_router          routing, published with a flag
+//                  projection        z_g = Phi_g^T x, z_u = Phi_u^T x: k_gemm_tc
+//                                    (gemm.cu, tensor cores), or below 4 tokens
+//                                    k_gemv_bulk<P> (rows through a bulk-copy ring);
+//                                    clears the accumulators
+//                  expert factors    k_gu_mma and k_dn_mma (expert_mma.cu: mma.sync over
+//                                    token tiles); on layers with 16-bit units, and
+//                                    where mma_fits says no, the dp2a kernels:
+//                    k_gateup_dec    gate/up = P_hat (alpha * z): dp2a over
 //                                    bucketed uniform-bit streams staged per warp
 //                                    item, int16 activation operand, vector red.add
-//                  k_down_dec        h = SiLU(gate) * up, then
+//                    k_down_dec      h = SiLU(gate) * up, then
 //                                    s += w_e * alpha_dn * (P_hat_dn^T h) per unit
-//                  k_gemv_bulk<O>    y = Phi_dn s (fp32 out)
-//   more tokens    k_router (multi-block), k_gemm_tc (gemm.cu: tensor cores) for
-//                  both projections, the same gate/up and down kernels
+//                  output basis      y = Phi_dn s (fp32 out): k_gemm_tc or k_gemv_bulk<O>
+//   more tokens    the same with k_gemm_tc for both projections (past 64 tokens
+//                  k_split before the second), where the tensor maps could be made
 //
 // The identity behind the association is Eq. app_normalized_decomposition
 // (W = P A Phi^T for gate/up, W = Phi A P^T for down); summing the experts'
@@ -1214,8 +1220,8 @@ __global__ void __launch_bounds__(kK3DecWarps * 32) k_down_dec(Fwd p) {
 #ifndef BITSMOE_DECODE_MAX_TOKENS
 #define BITSMOE_DECODE_MAX_TOKENS 8
 #endif
-// Small batches run the decode chain (every kernel routes all tokens itself; the
-// single token also the fused kernel), larger ones the tensor-core chain.
+// Small batches run the decode chain (a single token the fused kernel where it
+// fits), larger ones the tensor-core chain.
 inline bool decode_mode(const ImageHeader& hd, int T) {
   return T <= BITSMOE_DECODE_MAX_TOKENS && T * hd.E <= 4096;
 }
@@ -1481,9 +1487,10 @@ bool mma_fits(const bitsmoe_layer* L, int T, int top_k, MArgs* ma);
 
 // Whether T > 1 tokens run as one fused forward each.  Three tokens cost the chain less than three fused forwards
 // (fused / chain, us: Qwen3-shaped layer 66.6 / 55.8, with uneven experts 76.3 / 50.9; D = 1200, n = 900, 24
-// experts 49.4 / 38.9; four tokens of D = n = 256, 8 experts 61.8 / 32.5), two cost it more (44.6 for the two).  The
-// chain would be faster on the smallest layers too (D = 96, n = 72, four tokens: 61.9 / 30.5); up to D n = 8192 they
-// keep the fused forwards, whose launch count (T) callers of such layers count on.
+// experts 49.4 / 38.9; four tokens of D = n = 256, 8 experts 61.8 / 32.5), two cost it more (44.6 for the two).
+// Below D n = 8192 three and four tokens keep the fused forwards although the chain would be faster there too (D = 96,
+// n = 72, four tokens: 61.9 / 30.5): their plan and launch count (T) are those that such layers have always had and
+// that the interface states, not a measured optimum.
 bool few_tokens_fused(const bitsmoe_layer* L, int T, int top_k) {
   if (T < 2 || T > kFusedMaxTokens || !fused_fits(L, top_k)) return false;
   MArgs ma;
@@ -1516,7 +1523,9 @@ int f2_choose(const bitsmoe_layer* L, int top_k, F2Args* fa) {
 }
 
 // Whether the expert factors of a T-token call run on mma.sync (calls whose projection runs on the
-// tensor cores, which also takes max |z| per token).
+// tensor cores, which also takes max |z| per token): from four tokens, and three where they would otherwise be
+// three fused forwards.  Three tokens of a layer outside the fused plan keep the dp2a kernels as they had them; mma.sync
+// would be faster there too (Mixtral-shaped layer 458 / 176 us, 32 experts of 1536 x 4096 241 / 110).
 bool mma_fits(const bitsmoe_layer* L, int T, int top_k, MArgs* ma) {
   return L->mma && (T >= 4 || (T == 3 && fused_fits(L, top_k))) && mma_args(L->hd(), T, top_k, L->gu_stage, ma);
 }
@@ -1563,7 +1572,6 @@ int forward_impl(const void* x, const float* logits, int T, int top_k, const bit
   p.s16 = (int)align_up(std::max(hd.seg_max_slots, 8), 64) + 8;
   p.rbc = k3_rbc(hd);
   p.seg_bytes = L->seg_bytes;
-  // decode mode: every kernel can afford the routing of all tokens
   p.decode = decode_mode(hd, T);
   {   // down staging: keep a warp's tile within ~48 KB of shared memory
     const int need = std::max(1, hd.group / kRows);

@@ -146,8 +146,9 @@ __device__ __forceinline__ void warp_better(float& be, int& bc) {
 // One warp's scored candidates and the list of those left to score.
 template <int NC>
 struct SearchMem {
-  // candidates a lane scores first: strides of 4, 8, 8 and 16 from 128 candidates on (at 256, 16384 units of 768:
-  // 327 us with a stride of 4, 299 with 8)
+  // candidates a lane scores first: strides of 4, 8, 8 and 16 from 128 candidates on, below it all of them.  16384 units
+  // of 768, us with this and with the other K: 64 candidates 193 / 224, 128 233 / 310, 256 300 / 327, 512 435 / 414
+  // (the one stride that is not the faster), 1024 613 / 654.
   static constexpr int K = NC == 1 || NC == 4 || NC == 8 ? 1 : 2;
   static constexpr int ST = NC / K;                      // their stride
   float s[32 * K], err[32 * K], norm[32 * K];            // scale, ||x - s q|| and ||q||
