@@ -207,13 +207,18 @@ __device__ __forceinline__ void split_quad(uint64_t v01, uint64_t v23, uint32_t 
   lo[1] = half2(b, d);
 }
 
-// 2^S with m 2^S in [2^13, 2^14) (1 for m = 0 or not finite), |S| <= 100.
+// 2^S with m 2^S in [2^13, 2^14) (1 for m = 0 or not finite), LO <= S <= 126: below 2^-112 the operand shrinks towards
+// 1, which an fp16 pair still holds, above 2^(14 - LO) it grows up to fp16's largest.
+template <int LO>
 __device__ __forceinline__ float scale_pow2(float m) {
   if (!(m > 0.f) || !(m < 3.0e38f)) return 1.f;
   int ex;
   frexpf(m, &ex);
-  return ldexpf(1.f, max(-100, min(100, 14 - ex)));
+  return ldexpf(1.f, max(LO, min(126, 14 - ex)));
 }
+constexpr int kGuLo = -106;         // gate/up undo 2^(S - 21) in one factor
+constexpr int kDnLo = -114;         // down in two: 2^(12 - S) with h's sums, 2^12 with the gate weight (exact, and
+constexpr float kDnPart = 4096.f;   // whatever q h sums to stays inside fp32 where its product with the scale does)
 
 // Bit position of a B-bit code in its fp16 element: the code times 2^kPos stays below 2048, where the bit
 // pattern is linear.  As high as it fits: the tensor core aligns a product by its operands' exponents, so
@@ -562,7 +567,7 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_gu_mma(Fwd p, MArgs x) {
       }
       if (c.first) {
         tok = pr / p.k;
-        bs = scale_pow2(__ldg(x.msa + c.h * p.E + tb.e[c.a]) * __uint_as_float(__ldcg(p.zmax + c.h * p.T + tok)));
+        bs = scale_pow2<kGuLo>(__ldg(x.msa + c.h * p.E + tb.e[c.a]) * __uint_as_float(__ldcg(p.zmax + c.h * p.T + tok)));
       }
       float4 v[kRB];
       auto gather = [&](int r, const int4& u, bool live) {   // rows r .. r + kRB - 1 of one slot quad
@@ -770,7 +775,7 @@ __device__ __forceinline__ void ul_a(const UlWords<B>& u, int k, int t, uint32_t
   else a_regs<B>(u.w[k], sh, mul, lo, hi);
 }
 
-// One row block of a tile: out += scale (P 2^(24 - S) - zero sum(h)) per group.  The hi and lo products of a
+// One row block of a tile: out += scale (P 2^(24 - S) - zero sum(h)) / 2^12 per group.  The hi and lo products of a
 // K-step go into the same accumulators, all hi ones first (apart, they took 16 registers more and spilled: 283 us
 // at 1024 tokens against 272; 258 with nothing spilled).
 template <int B, int NT, int NTM, int G>
@@ -822,7 +827,7 @@ __device__ __forceinline__ void dn_rb(const uint8_t* code, const uint4* hf, int 
         }
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
-          float4 z = hz[gl * zstride + n * 4 + t];   // tokens 2 t and 2 t + 1: (sum, 2^(24 - S)) each
+          float4 z = hz[gl * zstride + n * 4 + t];   // tokens 2 t and 2 t + 1: (sum, 2^(24 - S)) / 2^12 each
           z.y *= fP;
           z.w *= fP;
 #pragma unroll
@@ -865,7 +870,7 @@ constexpr int kDnStages = 3;   // most stages of a consumer's ring
 // Rows of a segment's token tile.
 struct DRow {
   int off;      // token * n_pad
-  float pw;     // gate weight
+  float pw;     // gate weight times 2^12
 };
 
 // Shared-memory plan of k_dn_mma.
@@ -961,11 +966,11 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
       if (k >= 2) ok &= mbar_wait(&hempty[s], (uint32_t)((k >> 1) - 1) & 1u, x.spin);
       if (!__all_sync(0xFFFFFFFFu, ok)) break;
       uint4* hf = reinterpret_cast<uint4*>(msm + L.hf + s * L.hfs);     // [NTM][RC][8 K-steps][32 lanes]
-      float2* hz = reinterpret_cast<float2*>(msm + L.hz + s * L.hzs);   // [RC][G][kNT] (sum of h, 2^(24 - S))
+      float2* hz = reinterpret_cast<float2*>(msm + L.hz + s * L.hzs);   // [RC][G][kNT] (sum of h, 2^(24 - S)) / 2^12
       if (hw == 0 && lane < 16) {
         DRow r;
         r.off = pr / p.k * p.n_pad;
-        r.pw = pw;
+        r.pw = pw * kDnPart;
         reinterpret_cast<DRow*>(msm + L.rows)[s * 16 + lane] = r;
       }
       // a warp per (token, row block), 4 rows a lane; four at a time (rows past the tile's tokens are left
@@ -994,13 +999,13 @@ __global__ void __launch_bounds__(kMmThreads, 1) k_dn_mma(Fwd p, MArgs x) {
           float sum = (h4.x + h4.y) + (h4.z + h4.w);
 #pragma unroll
           for (int o = 16 / G; o; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-          const float sc = scale_pow2(am);
+          const float sc = scale_pow2<kDnLo>(am);
           uint4 v;
           split_pair(h4.x * sc, h4.z * sc, v.x, v.z);
           split_pair(h4.y * sc, h4.w * sc, v.y, v.w);
           hf[((size_t)(tk >> 3) * RC + rb) * 256 + (lane >> 2) * 32 + (tk & 7) * 4 + (lane & 3)] = v;
           if ((lane & (32 / G - 1)) == 0)
-            hz[((size_t)rb * G + lane / (32 / G)) * kNT + tk] = make_float2(sum, 16777216.f / sc);
+            hz[((size_t)rb * G + lane / (32 / G)) * kNT + tk] = make_float2(sum / kDnPart, (16777216.f / kDnPart) / sc);
         }
       }
       __syncwarp();

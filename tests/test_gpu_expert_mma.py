@@ -181,6 +181,28 @@ def test_impossible_routing_is_refused(env, T):
     assert np.max(np.abs(y.cpu().numpy() - ref)) <= TOL * np.max(np.abs(ref))
 
 
+@pytest.mark.parametrize("e", [-56, 57])
+@pytest.mark.parametrize("T,E,k,D,n,I,group", [
+    (4, 8, 2, 256, 256, 512, 64), (8, 16, 4, 256, 200, 384, 128), (40, 32, 8, 128, 100, 128, 32), (70, 8, 2, 512, 300, 256, 128)])
+def test_tiny_and_huge_activations(env, T, E, k, D, n, I, group, e):
+    """Tokens scaled by 2^e: h = SiLU(gate) * up near 2^-112 and 2^118, whose power-of-two scaling into fp16's range
+    takes the largest exponents.  Tolerance: that of ordinary tokens, and for the tiny ones fp32 additions into global
+    memory and bf16 products, which drop what lies below 2^-126: at most k + 1 such errors an element of s, uniform,
+    through rows of Phi of norm at most 1: four standard deviations."""
+    torch, bm = env
+    spec = synth.scaled_spec(synth.WORKLOADS["tiny"], D=D, E=E, I=I, n=n, group=group, top_k=k)
+    layer = synth.make_layer(spec, seed=3, bits_dist=BITS, alpha_scale=4.0)
+    L = bm.bitsmoe_pack(layer, device=0)
+    x, logits = synth.make_inputs(spec, T, seed=9)
+    xf = (x.astype(np.uint32) << 16).view(np.float32) * np.float32(2.0) ** e
+    x = synth.f32_to_bf16_bits(xf.astype(np.float32))
+    y = bm.moe_forward(L, torch.from_numpy(x.view(np.int16)).cuda(), torch.from_numpy(logits).cuda(), k)
+    with np.errstate(over="ignore"):   # exp of a huge gate in the oracle: SiLU is 0 there
+        ref = oracle.moe_forward_factored(layer, x, logits, k)
+    tol = TOL * np.max(np.abs(ref)) + 4.0 * np.sqrt((k + 1) / 3.0) * 2.0 ** -126
+    assert np.max(np.abs(y.cpu().numpy() - ref)) <= tol
+
+
 def wide_layer(spec, seed, bits):
     """A layer with more units than features (n > D): random bases of norm-1 columns."""
     layer = synth.make_layer(synth.scaled_spec(spec, D=spec.n), seed=seed, bits_dist=bits, alpha_scale=4.0,
