@@ -124,6 +124,21 @@ def test_row_ranges_and_block_counts(env, side, E, d, D):
     assert np.linalg.norm(rebuilt - Wcat) <= 2e-5 * np.linalg.norm(Wcat)
 
 
+@pytest.mark.parametrize("side", ["in", "out"])
+def test_low_rank_weights(env, side):
+    """Weights of rank 5: rounding noise among the zero eigenvalues is not rotated.  A vector is rotated about 5 times a
+    sweep, each time off by at most 2^-23: 1e-5 after some 15 sweeps.  A zero singular value is the root of G's
+    rounding, a quarter of 2^-24 of the largest eigenvalue."""
+    rng = np.random.default_rng(5)
+    E, d, D, r = 16, 96, 1500, 5
+    W = (rng.standard_normal((E * d, r)) @ rng.standard_normal((r, D))).astype(np.float32).reshape(E, d, D)
+    phi, sig, alpha, P, _ = run(env, [w if side == "in" else np.ascontiguousarray(w.T) for w in W], side)
+    assert np.max(np.abs(phi.T @ phi - np.eye(D))) <= 1e-5
+    assert np.all(sig[r:] <= np.sqrt(0.25 * 2.0 ** -24) * sig[0])
+    Pt = np.concatenate([P[e].T * alpha[e][None, :] for e in range(E)], axis=0)
+    assert np.linalg.norm(Pt @ phi.T - W.reshape(E * d, D)) <= 2e-5 * np.linalg.norm(W)
+
+
 def test_zero_expert_block(env):
     """An expert whose weights are all zero has alpha = 0 and P = 0 (P~_e / 1)."""
     W = prescribed(3, 16, 40, "in", seed=9)
