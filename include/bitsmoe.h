@@ -204,7 +204,7 @@ int bitsmoe_debug_single_token_kernel(int which);
  * BITSMOE_ERR_DEVICE_BOUNDS in the workspace status word (the call's output is
  * then undefined).  Layers packed or loaded while it is on are given a
  * zero-filled slack of the image's own size after the image.  on = 2 also makes
- * the expert kernels of several tokens find an impossible count in the routing,
+ * the expert kernels of several tokens find impossible counts in the routing,
  * which the check they always make of it (experts, counts and lists inside the
  * call's) leaves out and reports as BITSMOE_ERR_WORKSPACE_STATE.
  * Applies to calls issued after it; on = 0 turns the checks off.  Returns

@@ -64,7 +64,7 @@ struct MArgs {
   const float* msa;       // [2][E] max over groups and slots of |scale * alpha| of gate/up (h, e)
   long long spin;         // bound of the waits inside a block, in SM clocks
   int lose;               // testing hooks: bit 0: an arrival of block 0 is left out, so that waits of its warps run out;
-                          // bit 1: the first expert's count is taken as T more than it is
+                          // bit 1: the experts' counts are taken as 2 T more than they are
 };
 
 // Staging records of the fused single-token kernel, derived from the image

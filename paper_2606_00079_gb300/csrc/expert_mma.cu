@@ -70,7 +70,7 @@ __device__ __forceinline__ int tile_weight(int nt) { return 1 + ((nt + 7) >> 3);
 
 // Whole block; the routing is published.  per_tile(e): units of a token tile of expert e.  An expert, a count or a
 // list outside the call's (another call on the same workspace, or a workspace that was not zero-filled) gets no
-// units, and the status word says so.  (An early return instead cost the down kernel spills in its consumers.)
+// units, and the status word says so.  (An early return instead cost the down kernel spills.)
 template <class F>
 __device__ void mtiles_build(const Fwd& p, int A_max, int lose, int NT, MTiles& t, F per_tile) {
   const int tid = threadIdx.x, lane = tid & 31;
@@ -79,9 +79,11 @@ __device__ void mtiles_build(const Fwd& p, int A_max, int lose, int NT, MTiles& 
   t.na = bad ? 0 : na;
   for (int a = tid; a < t.na; a += (int)blockDim.x) {
     const int e = p.active[1 + a];
-    const bool in = e >= 0 && e < p.E;
-    const int c = in ? p.expert_count[e] + ((lose & 2) && a == 0 ? p.T : 0) : 0, start = in ? p.expert_start[e] : 0;
-    if (c < 1 || c > p.T || start < 0 || start > p.P - c) {
+    // Read side by side, at a place that is there whatever e is (one after the other's check: 8 tokens 60.9 us
+    // against 60.5; without a branch 60.1, but 1024 tokens 719 against 711).
+    const int es = (int)min((unsigned)e, (unsigned)p.E - 1u);
+    const int c = p.expert_count[es] + (lose & 2) * p.T, start = p.expert_start[es], m = per_tile(es);
+    if (e != es || (unsigned)(c - 1) >= (unsigned)p.T || (unsigned)start > (unsigned)(p.P - c)) {
       bad = true;
       t.ub[a] = t.wb[a] = t.cnt[a] = 0;
       continue;
@@ -89,7 +91,7 @@ __device__ void mtiles_build(const Fwd& p, int A_max, int lose, int NT, MTiles& 
     t.e[a] = e;
     t.cnt[a] = c;
     t.pst[a] = start;
-    const int m = per_tile(e), f = c / NT, r = c - f * NT;
+    const int f = c / NT, r = c - f * NT;
     t.ub[a] = (f + (r > 0)) * m;
     t.wb[a] = (f * tile_weight(NT) + (r > 0 ? tile_weight(r) : 0)) * m;
   }

@@ -160,7 +160,7 @@ def test_projection_waits_that_run_out(env, D):
 
 @pytest.mark.parametrize("T", [8, 40])
 def test_impossible_routing_is_refused(env, T):
-    """A routing whose first expert holds more tokens than the call has (testing hook) is left out and reported as
+    """A routing whose experts hold more tokens than the call has (testing hook) is left out and reported as
     WORKSPACE_STATE; the next call on the same workspace is correct."""
     torch, bm = env
     spec = synth.scaled_spec(synth.WORKLOADS["tiny"], D=128, E=8, I=256, n=96, group=128, top_k=3)
